@@ -266,13 +266,17 @@ int sdl_sparse_code(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const
     DeviceGuard g(c->device);
     if ((rc = ensure_workspace(c, p1, p2, n1, n2)) != SDL_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    grams(c, D1, p1, n1, D2, p2, n2, st);
     PassArgs a = base_args(c, Y, p1, p2, N, D1, n1, D2, n2, s);
     a.eps2 = eps > 0.f ? eps * eps : 0.f;
     a.support = support;
     a.coef = coef;
     a.nnz = nnz;
     a.res_energy = res_energy;
+    if (!(c->prec & SDL_PREC_BF16_CORR) && code_lanes_take(a, c->cap_part)) {
+        Trace tr(c, kCode, st);
+        return launch_code_lanes(a, c->part_f, c->cap_part, st, c->num_sms);
+    }
+    grams(c, D1, p1, n1, D2, p2, n2, st);
     if ((c->prec & SDL_PREC_BF16_CORR) && (rc = prepare_tc_pass(c, a, true, st)) != SDL_OK) return rc;
     {
         Trace tr(c, kCode, st);

@@ -25,6 +25,7 @@ struct sdl_batch {
     std::vector<int> generic;      // groups coded by the generic kernel
     std::vector<int> gslots[3];    // their partial-sum slots per pass side
     int n_fast = 0;                // groups in the multi-problem kernel
+    bool large_groups = false;     // each of them fills the GPU by itself
     std::vector<int> cta_begin;    // G + 1 prefix of CTAs per group
     std::vector<float> cost_us;    // time of one fused pass of the group alone
     int single_cps = 0;            // one group: the CTAs per SM the autotuner chose
@@ -50,6 +51,7 @@ struct sdl_batch {
     std::vector<float*> G1, G2, red_f, norms;
     std::vector<double*> red_d, part_d;
     std::vector<float*> part_f;
+    std::vector<size_t> part_cap;  // floats of each
     cudaGraphExec_t graph = nullptr;
 };
 
@@ -58,18 +60,37 @@ namespace {
 constexpr int kSlotsPerSm = 8;   // partial-sum slots reserved per SM and group
 constexpr int kMultiWarps = 8;   // warps per CTA of the persistent multi-problem kernel
 
+// Signals from which a group's code-only pass runs as its own launch of the
+// lane-group coder (omp_group.cuh) rather than inside the multi-problem launch.
+constexpr long long kLargeGroup = 8192;
+// (and up to which the list of an error-driven one fits its partial-sum slots)
+constexpr long long kMostListed = 1 << 20;
+
 // A coding pass of every group: one persistent multi-problem launch, or for a
 // single group its tiling's own kernel on the same CTAs (no other problem's
 // code shares its register allocation).
 int code_pass(const sdl_batch* b, int side, cudaStream_t st) {
     int rc = SDL_OK;
-    if (b->n_fast > 0) {
+    if (side == kCodeOnly && b->large_groups) {
+        for (int g = 0; g < b->G; ++g) {
+            if (b->shape[g] < 0) continue;
+            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], st, b->ctx->num_sms);
+            if (rc != SDL_OK) return rc;
+        }
+    } else if (b->n_fast > 0) {
         rc = b->G == 1 ? launch_code_pass_grid(b->args[side][0], side, b->shape[0], b->total_ctas, st)
                        : launch_code_multi(b->d_args[side], b->d_cta_begin, b->d_shape, b->G,
                                            b->total_ctas, b->smem[side], side, st, b->ctx->num_sms);
         if (rc != SDL_OK) return rc;
     }
     for (size_t i = 0; i < b->generic.size(); ++i) {
+        if (side == kCodeOnly) {
+            const int g = b->generic[i];
+            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], st, b->ctx->num_sms);
+            if (rc == SDL_OK) continue;
+            if (rc != SDL_ERR_UNSUPPORTED) return rc;
+            rc = SDL_OK;
+        }
         const int r = launch_code_pass_generic(b->args[side][b->generic[i]], side, st, b->ctx->num_sms);
         if (r < 0) return r;
         if (r != b->gslots[side][i]) return SDL_ERR_CUDA;   // the planned reduction would miss slots
@@ -176,6 +197,9 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         if (gen) b->generic.push_back(g);
     }
     b->n_fast = G - (int)b->generic.size();
+    b->large_groups = true;
+    for (int g = 0; g < G; ++g)
+        if (!variants[g].empty() && (groups[g].N < kLargeGroup || groups[g].N > kMostListed)) b->large_groups = false;
 
     // ---- device memory
     const int max_slots = c->num_sms * kSlotsPerSm;
@@ -185,11 +209,15 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         bytes += align256(n);
         return off;
     };
+    // partial sums of the larger side
+    auto nf_of = [](const sdl_group& q) {
+        return std::max<size_t>((size_t)q.n1 * q.n1 + (size_t)q.p1 * q.n1,
+                                (size_t)q.n2 * q.n2 + (size_t)q.p2 * q.n2);
+    };
     std::vector<size_t> o_g1(G), o_g2(G), o_pf(G), o_pd(G), o_rf(G), o_rd(G), o_nr(G);
     for (int g = 0; g < G; ++g) {
         const sdl_group& q = groups[g];
-        const size_t nf = std::max<size_t>((size_t)q.n1 * q.n1 + (size_t)q.p1 * q.n1,
-                                           (size_t)q.n2 * q.n2 + (size_t)q.p2 * q.n2);
+        const size_t nf = nf_of(q);
         o_g1[g] = take(sizeof(float) * q.n1 * q.n1);
         o_g2[g] = take(sizeof(float) * q.n2 * q.n2);
         o_pf[g] = take(sizeof(float) * nf * max_slots);
@@ -215,6 +243,7 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         b->G1.push_back(reinterpret_cast<float*>(b->dmem + o_g1[g]));
         b->G2.push_back(reinterpret_cast<float*>(b->dmem + o_g2[g]));
         b->part_f.push_back(reinterpret_cast<float*>(b->dmem + o_pf[g]));
+        b->part_cap.push_back(nf_of(groups[g]) * max_slots);
         b->part_d.push_back(reinterpret_cast<double*>(b->dmem + o_pd[g]));
         b->red_f.push_back(reinterpret_cast<float*>(b->dmem + o_rf[g]));
         b->red_d.push_back(reinterpret_cast<double*>(b->dmem + o_rd[g]));

@@ -842,7 +842,7 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     a.idx_count = n_fallback;
     {
         Trace tr(c, kCode, st);
-        rc = launch_code_pass_fast(a, kCodeOnly, st, c->num_sms);
+        rc = launch_code_group_fixed(a, false, st, c->num_sms);
         if (rc < 0) return rc;
     }
     // 4. the plain coder on the strided sample (residual energies only)
@@ -857,7 +857,7 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     g.idx_compact = 1;
     {
         Trace tr(c, kCode, st);
-        rc = launch_code_pass_fast(g, kCodeOnly, st, c->num_sms);
+        rc = launch_code_group_fixed(g, false, st, c->num_sms);
         if (rc < 0) return rc;
     }
     // 5. RMSE guard; when it trips, every signal is coded again by the plain coder
@@ -868,7 +868,7 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     a.idx_count = cnt_s + 1;
     {
         Trace tr(c, kCode, st);
-        rc = launch_code_pass_fast(a, kCodeOnly, st, c->num_sms);
+        rc = launch_code_group_fixed(a, false, st, c->num_sms);
     }
     return rc < 0 ? rc : SDL_OK;
 }

@@ -1,0 +1,706 @@
+// 2D-OMP coding pass with a small group of lanes per signal: a warp codes
+// 32 / GL signals at once, GL = 8 or 16 lanes each.
+//
+// Same method and arithmetic as the one-warp-per-signal coders (omp_fast.cu,
+// omp_pass.cu): every entry of Z, C0 and of the scores, the Cholesky rows and
+// both triangular solves are the same FMA chains in the same order, so the
+// codes are bit-identical to theirs.  What bounds a coding pass here is the
+// number of warp instructions, not the FMAs among them (about one in six in the
+// one-warp form).  With GL lanes per signal:
+//   * the per-signal scalar work (pick, Cholesky row, solves), which every lane
+//     of a signal repeats, is issued once for 32 / GL signals;
+//   * a lane's RI x RJ block is large, so each operand load feeds more FMAs;
+//   * the argmax takes three-input |max| (two entries per instruction) down
+//     the columns of the block and a compare/select only per column; the row
+//     comes from one read-back of the winning column;
+//   * the greedy loop is a loop over t, with only the Cholesky row unrolled per
+//     t, so that the code of all steps fits the instruction cache.
+// Scores are recomputed from C0 every step, as in the other coders.
+//
+// Measured (GB300, us per call, one warp per signal -> this kernel): 200 000 x
+// 12x12, 24x24 pairs, s = 6: 472 -> 324 (of the compiled tilings the fastest,
+// two signals per warp, takes 410); 247 009 x 16x16, 32x32, s = 8: 1636 -> 1003;
+// 99 991 x 10x9, 20x18, s = 5 (generic kernel before): 493 -> 167.  At 12x12 a
+// signal takes 1106 warp instructions (1877 before); 71 % of the shared-memory
+// bandwidth (operands of the rank-one updates, and C0 read back every step) and
+// 51 % of the issue slots are in use.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+#include <type_traits>
+
+#include "sdl_internal.cuh"
+
+namespace sdl {
+namespace group {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+__host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
+
+// SF / P1F ...: sizes fixed at compile time (0: taken from the call).
+// kFastNum: 1/sqrt by rsqrtf and back substitution in increasing row order
+// (the compiled tilings' forms); else 1/sqrtf and decreasing order (the
+// generic kernel's).  kW: C0 = (D1^T Y) D2 rather than D1^T (Y D2).
+template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,
+          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0>
+struct Cfg {
+    static constexpr int GL = GL_, LI = LI_, LJ = GL_ / LI_, RI = RI_, RJ = RJ_;
+    static constexpr int WARPS = WARPS_, MINB = MINB_;
+    static constexpr bool kFast = FAST_, kW = W_;
+    static constexpr int P1 = P1_, P2 = P2_, N1 = N1_, N2 = N2_, S = S_;
+    static constexpr int SPW = 32 / GL;                 // signals per warp
+    static constexpr int N1P = LI * RI, N2P = LJ * RJ;
+    static constexpr int RIP = up4(RI), RJP = up4(RJ);  // padded block lengths (16-byte loads)
+    static constexpr int LD1 = LI * RIP, LD2 = LJ * RJP;
+    static constexpr int E = RI * RJ;
+    // lane stride of the C0 blocks: an odd multiple of 4 floats, so that the 8
+    // lanes of a 128-bit load phase hit distinct banks
+    static constexpr int EP = (up4(E) / 4) % 2 ? up4(E) : up4(E) + 4;
+    static constexpr int CS = up4(RI);                  // the winning column's read-back buffer
+    // rows per lane and block of the Z stage (Y D2), columns of the W stage
+    static constexpr int ZA = P1 ? (P1 / LI) : 4;
+    static constexpr int WB = P2 ? (P2 / LJ) : 4;
+    static constexpr int SMAX = S ? S : 8;              // unrolled Cholesky rows
+    static_assert(N1P * LD1 <= 65536 && N2P * LD2 <= 65536, "16-bit row offsets");
+    static_assert(E % 4 == 0 && RI % 2 == 0, "row pairs, 16-byte block stores");
+    static_assert((LI & (LI - 1)) == 0 && LI * LJ == GL, "lane grid");
+    static_assert(!kW || P2 > 0, "the W stage is compiled for fixed sizes");
+    static_assert(P1 == 0 || (P1 % LI == 0 && ZA % 2 == 0 && P1 % 4 == 0 && P2 % LJ == 0), "fixed sizes");
+    static_assert(N1 == 0 || (N1 == N1P && N2 == N2P), "fixed sizes fill the tile");
+};
+
+// Shared memory of a CTA, in floats; every region starts 16-byte aligned.
+struct Layout {
+    int p1s;       // row stride of a staged signal's columns (p1 rounded up to 4)
+    int d1, d2, g1, g2, warp0;
+    int y, c0, col, rec, lf, iv, yv, sig_stride;   // per signal
+    int warp_stride, total;
+};
+
+template <class C>
+__host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
+    Layout L;
+    L.p1s = up4(p1);
+    L.d1 = 0;
+    L.d2 = L.d1 + p1 * C::LD1;
+    L.g1 = L.d2 + p2 * C::LD2;
+    L.g2 = L.g1 + C::N1P * C::LD1;
+    L.warp0 = L.g2 + C::N2P * C::LD2;
+    L.y = 0;
+    L.c0 = L.y + L.p1s * p2;
+    const int z = C::kW ? p2 * C::LD1 : up4(p1) * C::LD2;   // Z or W shares the C0 blocks' place
+    const int c = C::GL * C::EP;
+    L.col = L.c0 + (z > c ? z : c);
+    L.rec = L.col + C::CS;
+    L.lf = L.rec + up4(2 * s);
+    L.iv = L.lf + up4(s * (s - 1) / 2);
+    L.yv = L.iv + up4(s);
+    int st = L.yv + up4(s);
+    // neighbouring signals of a warp start 8 banks apart where they read the
+    // same offsets together
+    while (st % 32 != 8 && st % 32 != 24) st += 4;
+    L.sig_stride = st;
+    L.warp_stride = C::SPW * st;
+    L.total = L.warp0 + warps * L.warp_stride;
+    return L;
+}
+
+// ------------------------------------------------------------------ helpers
+template <int R>
+__device__ __forceinline__ void ld(float (&v)[R], const float* p) {   // 16-byte aligned p
+#pragma unroll
+    for (int k = 0; k + 4 <= R; k += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p + k);
+        v[k] = t.x; v[k + 1] = t.y; v[k + 2] = t.z; v[k + 3] = t.w;
+    }
+    constexpr int k0 = R & ~3;
+    if constexpr (R - k0 >= 2) {
+        const float2 t = *reinterpret_cast<const float2*>(p + k0);
+        v[k0] = t.x; v[k0 + 1] = t.y;
+    }
+    if constexpr ((R - k0) & 1) v[R - 1] = p[R - 1];
+}
+template <int R>
+__device__ __forceinline__ void ld2(float (&v)[R], const float* p) {   // 8-byte aligned p, R even
+#pragma unroll
+    for (int k = 0; k < R; k += 2) {
+        const float2 t = *reinterpret_cast<const float2*>(p + k);
+        v[k] = t.x; v[k + 1] = t.y;
+    }
+}
+template <int R>
+__device__ __forceinline__ void st(float* p, const float (&v)[R]) {   // 16-byte aligned p
+#pragma unroll
+    for (int k = 0; k + 4 <= R; k += 4)
+        *reinterpret_cast<float4*>(p + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    constexpr int k0 = R & ~3;
+    if constexpr (R - k0 >= 2) *reinterpret_cast<float2*>(p + k0) = make_float2(v[k0], v[k0 + 1]);
+    if constexpr ((R - k0) & 1) p[R - 1] = v[R - 1];
+}
+
+// d = a * b + d on two FP32 lanes at once (each half rounds as fmaf)
+__device__ __forceinline__ void ffma2(float& d0, float& d1, float a0, float a1, float b0, float b1) {
+    const unsigned long long A = ((unsigned long long)__float_as_uint(a1) << 32) | __float_as_uint(a0);
+    const unsigned long long B = ((unsigned long long)__float_as_uint(b1) << 32) | __float_as_uint(b0);
+    const unsigned long long C = ((unsigned long long)__float_as_uint(d1) << 32) | __float_as_uint(d0);
+    unsigned long long D;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(D) : "l"(A), "l"(B), "l"(C));
+    d0 = __uint_as_float((unsigned)(D & 0xffffffffu));
+    d1 = __uint_as_float((unsigned)(D >> 32));
+}
+// blk[c * R + r] += a[r] * b[c]
+template <int R, int N>
+__device__ __forceinline__ void rank1(float (&blk)[R * N], const float (&a)[R], const float (&b)[N]) {
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+#pragma unroll
+        for (int r = 0; r < R; r += 2) ffma2(blk[c * R + r], blk[c * R + r + 1], a[r], a[r + 1], b[c], b[c]);
+}
+// the same with the pairs along b (blk[r * N + c] += a[r] * b[c]); odd N leaves one scalar column
+template <int R, int N>
+__device__ __forceinline__ void rank1_rows(float (&blk)[R * N], const float (&a)[R], const float (&b)[N]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int c = 0; c + 2 <= N; c += 2) ffma2(blk[r * N + c], blk[r * N + c + 1], a[r], a[r], b[c], b[c + 1]);
+        if constexpr (N & 1) blk[r * N + N - 1] = fmaf(a[r], b[N - 1], blk[r * N + N - 1]);
+    }
+}
+__device__ __forceinline__ float max3abs(float a, float b, float c) {   // NaN operands are ignored
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+__device__ __forceinline__ unsigned sptr(const void* p) {
+    return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void cp16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sptr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sptr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One pick of a signal: its coefficient, and the offsets of its rows of G1
+// (low half) and G2 (high half) in shared memory, one 8-byte load.
+struct alignas(8) Rec {
+    float x;
+    unsigned o;
+    __device__ __forceinline__ int o1() const { return (int)(o & 0xffffu); }
+    __device__ __forceinline__ int o2() const { return (int)(o >> 16); }
+};
+
+// One greedy step's Cholesky row T and the coefficients of the T + 1 picks
+// (every lane of the signal holds the same values; `writer` stores them).
+// Returns false (state untouched) when the pick is degenerate or !live.
+template <int T, bool kFast>
+__device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, float* lf, float* iv, float* yv,
+                                          const float* G1s, const float* G2s, int c1, int c2, float Att,
+                                          float b, const Rec& pick, float& E) {
+    constexpr int NL = T * (T - 1) / 2;
+    float L[NL > 0 ? up4(NL) : 1], io[T > 0 ? up4(T) : 1], yo[T > 0 ? up4(T) : 1], am[T > 0 ? T : 1];
+    if constexpr (T > 0) {
+#pragma unroll
+        for (int m = 0; m < T; ++m) am[m] = G1s[rec[m].o1() + c1] * G2s[rec[m].o2() + c2];
+#pragma unroll
+        for (int k = 0; k < NL; k += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(lf + k);
+            L[k] = t.x; L[k + 1] = t.y; L[k + 2] = t.z; L[k + 3] = t.w;
+        }
+#pragma unroll
+        for (int k = 0; k < T; k += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(iv + k);
+            const float4 u = *reinterpret_cast<const float4*>(yv + k);
+            io[k] = t.x; io[k + 1] = t.y; io[k + 2] = t.z; io[k + 3] = t.w;
+            yo[k] = u.x; yo[k + 1] = u.y; yo[k + 2] = u.z; yo[k + 3] = u.w;
+        }
+    }
+    float w[T > 0 ? T : 1];
+    float ww = 0.f, wy = 0.f;
+#pragma unroll
+    for (int m = 0; m < T; ++m) {
+        float v = am[m];
+#pragma unroll
+        for (int l = 0; l < m; ++l) v = fmaf(-L[m * (m - 1) / 2 + l], w[l], v);
+        w[m] = v * io[m];
+        ww = fmaf(w[m], w[m], ww);
+        wy = fmaf(w[m], yo[m], wy);
+    }
+    const float d = Att - ww;
+    const bool ok = live && d > kPivotRel * Att;
+    const float inv = kFast ? rsqrtf(d) : 1.f / sqrtf(d);
+    const float yt = (b - wy) * inv;
+    float x[T + 1];
+    x[T] = yt * inv;
+#pragma unroll
+    for (int k = T - 1; k >= 0; --k) {
+        float v = yo[k];
+        if constexpr (kFast) {
+#pragma unroll
+            for (int l = k + 1; l < T; ++l) v = fmaf(-L[l * (l - 1) / 2 + k], x[l], v);
+            v = fmaf(-w[k], x[T], v);
+        } else {
+            v = fmaf(-w[k], x[T], v);
+#pragma unroll
+            for (int l = T - 1; l > k; --l) v = fmaf(-L[l * (l - 1) / 2 + k], x[l], v);
+        }
+        x[k] = v * io[k];
+    }
+    if (ok && writer) {
+#pragma unroll
+        for (int m = 0; m < T; ++m) {
+            lf[NL + m] = w[m];
+            rec[m].x = x[m];
+        }
+        iv[T] = inv;
+        yv[T] = yt;
+        Rec r = pick;
+        r.x = x[T];
+        rec[T] = r;
+    }
+    if (ok) E = fmaf(-yt, yt, E);
+    return ok;
+}
+
+// The same for any t, as loops through shared memory (row t of the factor and
+// the coefficients are written by every lane of the signal with equal values;
+// a step that fails leaves them unread).
+template <bool kFast>
+__device__ __forceinline__ bool chol_step_any(int t, bool live, bool writer, Rec* rec, float* lf, float* iv,
+                                              float* yv, const float* G1s, const float* G2s, int c1, int c2,
+                                              float Att, float b, const Rec& pick, float& E) {
+    float* w = lf + t * (t - 1) / 2;
+    float ww = 0.f, wy = 0.f;
+    for (int m = 0; m < t; ++m) {
+        float v = G1s[rec[m].o1() + c1] * G2s[rec[m].o2() + c2];
+        const float* Lm = lf + m * (m - 1) / 2;
+        for (int l = 0; l < m; ++l) v = fmaf(-Lm[l], w[l], v);
+        const float wm = v * iv[m];
+        w[m] = wm;
+        ww = fmaf(wm, wm, ww);
+        wy = fmaf(wm, yv[m], wy);
+    }
+    const float d = Att - ww;
+    const bool ok = live && d > kPivotRel * Att;
+    if (!ok) return false;
+    const float inv = kFast ? rsqrtf(d) : 1.f / sqrtf(d);
+    const float yt = (b - wy) * inv;
+    const float xt = yt * inv;
+    for (int k = t - 1; k >= 0; --k) {
+        float v = yv[k];
+        if constexpr (kFast) {
+            for (int l = k + 1; l < t; ++l) v = fmaf(-lf[l * (l - 1) / 2 + k], rec[l].x, v);
+            v = fmaf(-w[k], xt, v);
+        } else {
+            v = fmaf(-w[k], xt, v);
+            for (int l = t - 1; l > k; --l) v = fmaf(-lf[l * (l - 1) / 2 + k], rec[l].x, v);
+        }
+        rec[k].x = v * iv[k];
+    }
+    if (writer) {
+        iv[t] = inv;
+        yv[t] = yt;
+        Rec r = pick;
+        r.x = xt;
+        rec[t] = r;
+    }
+    E = fmaf(-yt, yt, E);
+    return true;
+}
+
+// compensated running sum
+__device__ __forceinline__ void ksum(float& s, float& c, float v) {
+    const float y = v - c;
+    const float t = s + y;
+    c = (t - s) - y;
+    s = t;
+}
+
+// ------------------------------------------------------------------- kernel
+// Positions 0 .. count-1 (signals, or entries of the index list) are coded in
+// units of SPW: warp w of CTA b takes units w gridDim + b, + gridDim warps, ...
+// (a small call spreads over the SMs).
+template <class C>
+__global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(PassArgs a) {
+    constexpr int GL = C::GL, LI = C::LI, LJ = C::LJ, RI = C::RI, RJ = C::RJ, E = C::E, SPW = C::SPW;
+    constexpr int LD1 = C::LD1, LD2 = C::LD2, RIP = C::RIP, RJP = C::RJP, ZA = C::ZA, WB = C::WB;
+    extern __shared__ __align__(16) float sm[];
+    const int p1 = C::P1 ? C::P1 : a.p1, p2 = C::P2 ? C::P2 : a.p2;
+    const int n1 = C::N1 ? C::N1 : a.n1, n2 = C::N2 ? C::N2 : a.n2;
+    const int s = C::S ? C::S : a.s;
+    const int pp = p1 * p2;
+    const bool error_driven = a.eps2 > 0.f;
+    const int warps = blockDim.x >> 5;
+    const Layout L = layout<C>(p1, p2, s, warps);
+    const int p1s = L.p1s;
+
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = lane / GL, gl = lane % GL;
+    const int li = gl % LI, lj = gl / LI;
+    float* D1s = sm + L.d1;    // row a: D1[a, :] in lane blocks
+    float* D2s = sm + L.d2;    // row b: D2[b, :] in lane blocks
+    float* G1s = sm + L.g1;
+    float* G2s = sm + L.g2;
+    float* wb = sm + L.warp0 + w * L.warp_stride;
+    float* sb = wb + grp * L.sig_stride;
+    float* Ys = sb + L.y;
+    float* Zs = sb + L.c0;     // Z (rows a) or W (rows b), then the C0 blocks
+    float* C0s = sb + L.c0;
+    float* myc0 = C0s + gl * C::EP;
+    float* col = sb + L.col;
+    Rec* rec = reinterpret_cast<Rec*>(sb + L.rec);
+    float* lf = sb + L.lf;
+    float* iv = sb + L.iv;
+    float* yv = sb + L.yv;
+
+    // ---- dictionaries in lane-block rows, then their Gram matrices (each
+    // entry one FMA chain over the rows, as the Gram kernels form it: no
+    // separate launch, and no difference)
+    for (int e = threadIdx.x; e < p1 * LD1; e += blockDim.x) {
+        const int r = e / LD1, pos = e % LD1, off = pos % RIP, i = (pos / RIP) * RI + off;
+        D1s[e] = (off < RI && i < n1) ? a.D1[r + p1 * i] : 0.f;
+    }
+    for (int e = threadIdx.x; e < p2 * LD2; e += blockDim.x) {
+        const int r = e / LD2, pos = e % LD2, off = pos % RJP, j = (pos / RJP) * RJ + off;
+        D2s[e] = (off < RJ && j < n2) ? a.D2[r + p2 * j] : 0.f;
+    }
+    // a signal's records start valid: a finished signal's lanes run along with
+    // the others of the warp on whatever its records hold
+    for (int e = lane; e < SPW * s; e += 32) {
+        const int g = e / s;
+        reinterpret_cast<Rec*>(wb + g * L.sig_stride + L.rec)[e - g * s] = Rec{0.f, 0u};
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < C::N1P * LD1; e += blockDim.x) {
+        const int i = e / LD1, pos = e % LD1;
+        const float* di = D1s + (i / RI) * RIP + i % RI;
+        const float* dj = D1s + pos;
+        float g = 0.f;
+        for (int r = 0; r < p1; ++r) g = fmaf(di[r * LD1], dj[r * LD1], g);
+        G1s[e] = g;
+    }
+    for (int e = threadIdx.x; e < C::N2P * LD2; e += blockDim.x) {
+        const int j = e / LD2, pos = e % LD2;
+        const float* di = D2s + (j / RJ) * RJP + j % RJ;
+        const float* dj = D2s + pos;
+        float g = 0.f;
+        for (int r = 0; r < p2; ++r) g = fmaf(di[r * LD2], dj[r * LD2], g);
+        G2s[e] = g;
+    }
+    __syncthreads();
+
+    const long long count = a.idx ? (long long)*a.idx_count : a.N;
+    const long long units = (count + SPW - 1) / SPW;
+    const long long ustep = (long long)gridDim.x * warps;
+    long long u = (long long)w * gridDim.x + blockIdx.x;   // next unit
+
+    // signals start on 16-byte boundaries and columns stay 16-byte aligned
+    const bool vec = (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0 && (C::P1 ? true : p1 % 4 == 0);
+    const unsigned inv_p1 = (65536u + p1 - 1) / p1;   // e / p1 = e inv_p1 >> 16 for e < 1024
+    auto fetch = [&](long long k) {   // this lane group's signal k into Ys (cp.async)
+        const float* src = a.Y + (size_t)k * pp;
+        if (vec) {
+            for (int e = gl * 4; e < pp; e += GL * 4) cp16(Ys + e, src + e);
+        } else {
+            for (int e = gl; e < pp; e += GL) {
+                const int b = (int)((unsigned)e * inv_p1 >> 16);
+                cp4(Ys + b * p1s + (e - b * p1), src + e);
+            }
+        }
+    };
+
+    float es = 0.f, ec = 0.f;      // this lane's residual-energy sum (compensated)
+    // the position of this group in the next unit; -1 when it has none.  The
+    // warp's units end when all groups have none.
+    auto next_pos = [&]() -> long long {
+        const long long p = u < units ? u * SPW + grp : count;
+        u += ustep;
+        return p < count ? p : -1;
+    };
+
+    long long pos = next_pos();
+    if (pos >= 0) fetch(a.idx ? (long long)a.idx[pos] : pos);
+    while (__any_sync(kFull, pos >= 0)) {
+        const bool act = pos >= 0;
+        const long long ko = !act ? 0 : (a.idx && !a.idx_compact) ? (long long)a.idx[pos] : pos;
+        cp_wait();
+        __syncwarp();
+        // ---- ||Y||^2: the 32 strided partial sums of the one-warp coders (this
+        // lane takes 32 / GL of them) and their combining tree
+        float part[SPW];
+#pragma unroll
+        for (int v = 0; v < SPW; ++v) part[v] = 0.f;
+        if (act) {
+#pragma unroll
+            for (int v = 0; v < SPW; ++v)
+                for (int e = gl + GL * v; e < pp; e += 32) {
+                    int at = e;
+                    if (!(C::P1 ? true : p1 % 4 == 0)) {
+                        const int b = (int)((unsigned)e * inv_p1 >> 16);
+                        at = b * p1s + (e - b * p1);
+                    }
+                    part[v] = fmaf(Ys[at], Ys[at], part[v]);
+                }
+        }
+        float ss;
+        if constexpr (SPW == 4) ss = (part[0] + part[2]) + (part[1] + part[3]);
+        else ss = part[0] + part[1];
+#pragma unroll
+        for (int o = GL / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
+        const bool finite = act && isfinite(ss);
+        bool go = finite && !(error_driven && ss <= a.eps2);
+
+        // ---- first contraction into shared memory: Z = Y D2 (lane (li, lj):
+        // rows li ZA.., columns of block lj) or W = D1^T Y (rows of block li,
+        // columns b of lane lj)
+        if constexpr (!C::kW) {
+            for (int a0 = li * ZA; a0 < (C::P1 ? C::P1 : p1); a0 += LI * ZA) {
+                float z[ZA * RJ];
+#pragma unroll
+                for (int e = 0; e < ZA * RJ; ++e) z[e] = 0.f;
+#pragma unroll 4
+                for (int b = 0; b < p2; ++b) {
+                    float y[ZA], d[RJ];
+                    if constexpr (ZA % 4 == 0) ld<ZA>(y, Ys + b * p1s + a0);
+                    else ld2<ZA>(y, Ys + b * p1s + a0);
+                    ld<RJ>(d, D2s + b * LD2 + lj * RJP);
+                    rank1_rows<ZA, RJ>(z, y, d);
+                }
+#pragma unroll
+                for (int r = 0; r < ZA; ++r) {
+                    if (C::P1 || a0 + r < p1) {
+                        float v[RJ];
+#pragma unroll
+                        for (int c = 0; c < RJ; ++c) v[c] = z[r * RJ + c];
+                        st<RJ>(Zs + (a0 + r) * LD2 + lj * RJP, v);
+                    }
+                }
+            }
+        } else {
+            float z[RI * WB];
+#pragma unroll
+            for (int e = 0; e < RI * WB; ++e) z[e] = 0.f;
+#pragma unroll 4
+            for (int r = 0; r < p1; ++r) {
+                float d[RI], y[WB];
+                ld<RI>(d, D1s + r * LD1 + li * RIP);
+#pragma unroll
+                for (int c = 0; c < WB; ++c) y[c] = Ys[(lj + LJ * c) * p1s + r];
+                rank1<RI, WB>(z, d, y);
+            }
+#pragma unroll
+            for (int c = 0; c < WB; ++c) {
+                float v[RI];
+#pragma unroll
+                for (int r = 0; r < RI; ++r) v[r] = z[c * RI + r];
+                st<RI>(Zs + (lj + LJ * c) * LD1 + li * RIP, v);
+            }
+        }
+        __syncwarp();
+        // Y is consumed: fetch the next unit's signals
+        const long long pos_next = next_pos();
+        if (pos_next >= 0) fetch(a.idx ? (long long)a.idx[pos_next] : pos_next);
+
+        // ---- C0 on the lane's RI x RJ block (flat index c * RI + r)
+        float sc[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) sc[e] = 0.f;
+        if constexpr (!C::kW) {
+#pragma unroll 2
+            for (int r = 0; r < p1; ++r) {
+                float x[RI], v[RJ];
+                ld<RI>(x, D1s + r * LD1 + li * RIP);
+                ld<RJ>(v, Zs + r * LD2 + lj * RJP);
+                rank1<RI, RJ>(sc, x, v);
+            }
+        } else {
+#pragma unroll 2
+            for (int b = 0; b < p2; ++b) {
+                float x[RI], v[RJ];
+                ld<RI>(x, Zs + b * LD1 + li * RIP);
+                ld<RJ>(v, D2s + b * LD2 + lj * RJP);
+                rank1<RI, RJ>(sc, x, v);
+            }
+        }
+        if constexpr (C::N1 == 0) {   // entries past the dictionaries never win
+#pragma unroll
+            for (int c = 0; c < RJ; ++c)
+#pragma unroll
+                for (int r = 0; r < RI; ++r)
+                    if (li * RI + r >= n1 || lj * RJ + c >= n2) sc[c * RI + r] = __int_as_float(0x7fc00000);
+        }
+        __syncwarp();   // every lane has read Z: its place takes the C0 blocks
+        st<E>(myc0, sc);
+        __syncwarp();
+
+        // ---- greedy steps
+        int cnt = 0;
+        float E2 = ss;
+#pragma unroll 1
+        for (int t = 0; t < s; ++t) {
+            const bool live = go && !(error_driven && E2 <= a.eps2);
+            if (!__any_sync(kFull, live)) break;
+            if (t > 0) {
+                ld<E>(sc, myc0);
+#pragma unroll 1
+                for (int l = 0; l < t; ++l) {
+                    const Rec r = rec[l];
+                    float x[RI], v[RJ];
+                    ld<RI>(x, G1s + r.o1() + li * RIP);
+                    ld<RJ>(v, G2s + r.o2() + lj * RJP);
+#pragma unroll
+                    for (int c = 0; c < RJ; ++c) v[c] *= -r.x;
+                    rank1<RI, RJ>(sc, x, v);
+                }
+            }
+            // the lane's largest |score|, its first column, by column maxima
+            float best = 0.f;
+            int bc = 0;
+#pragma unroll
+            for (int c = 0; c < RJ; ++c) {
+                float m = 0.f;
+#pragma unroll
+                for (int r = 0; r < RI; r += 2) m = max3abs(m, sc[c * RI + r], sc[c * RI + r + 1]);
+                if (m > best) { best = m; bc = c; }
+            }
+            // the signal's largest and its smallest (column, row block)
+            float M = best;
+            int key = (lj * RJ + bc) * LI + li;
+#pragma unroll
+            for (int o = GL / 2; o > 0; o >>= 1) {
+                const float mo = __shfl_xor_sync(kFull, M, o);
+                const int ko2 = __shfl_xor_sync(kFull, key, o);
+                if (mo > M || (mo == M && ko2 < key)) { M = mo; key = ko2; }
+            }
+            const bool pick = live && M != 0.f;
+            const int jt = key / LI, lio = key % LI;
+            // the owner lane's column, and the first row that holds M
+            if (gl == lio + LI * (jt / RJ)) {
+#pragma unroll
+                for (int c = 0; c < RJ; ++c)
+                    if (bc == c) {
+                        float v[RI];
+#pragma unroll
+                        for (int r = 0; r < RI; ++r) v[r] = sc[c * RI + r];
+                        st<RI>(col, v);
+                    }
+            }
+            __syncwarp();
+            unsigned rows = 0;
+#pragma unroll
+            for (int r0 = 0; r0 < RI; r0 += GL) {
+                const bool eq = r0 + gl < RI && fabsf(col[r0 + gl]) == M;
+                const unsigned bal = __ballot_sync(kFull, eq);
+                rows |= ((bal >> (GL * grp)) & ((1u << GL) - 1u)) << r0;
+            }
+            const int rt = rows ? __ffs(rows) - 1 : 0;
+            const int it = lio * RI + rt;
+            float* cq = C0s + (lio + LI * (jt / RJ)) * C::EP + (jt % RJ) * RI + rt;
+            const float b = *cq;
+            const int c1 = lio * RIP + rt, c2 = (jt / RJ) * RJP + jt % RJ;
+            const Rec pk{0.f, (unsigned)(it * LD1) | ((unsigned)(jt * LD2) << 16)};
+            const float Att = G1s[it * LD1 + c1] * G2s[jt * LD2 + c2];
+            __syncwarp();
+            const bool wr = gl == 0;
+            if (wr && pick) *cq = __int_as_float(0x7fc00000);   // mask the pick
+            bool ok = false;
+            auto step = [&](auto tc) {
+                ok = chol_step<decltype(tc)::value, C::kFast>(pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att,
+                                                              b, pk, E2);
+            };
+            switch (t) {
+                case 0: step(std::integral_constant<int, 0>{}); break;
+                case 1: if constexpr (C::SMAX > 1) step(std::integral_constant<int, 1>{}); break;
+                case 2: if constexpr (C::SMAX > 2) step(std::integral_constant<int, 2>{}); break;
+                case 3: if constexpr (C::SMAX > 3) step(std::integral_constant<int, 3>{}); break;
+                case 4: if constexpr (C::SMAX > 4) step(std::integral_constant<int, 4>{}); break;
+                case 5: if constexpr (C::SMAX > 5) step(std::integral_constant<int, 5>{}); break;
+                case 6: if constexpr (C::SMAX > 6) step(std::integral_constant<int, 6>{}); break;
+                case 7: if constexpr (C::SMAX > 7) step(std::integral_constant<int, 7>{}); break;
+                default:
+                    if constexpr (C::S == 0)
+                        ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att, b, pk, E2);
+                    break;
+            }
+            if (ok) cnt = t + 1;
+            go = ok;
+            __syncwarp();   // the step's state and the masked entry are visible
+        }
+
+        // ---- the code
+        if (act) {
+            if (a.support)
+                for (int l = gl; l < s; l += GL) {
+                    const Rec r = rec[l];
+                    a.support[(size_t)ko * s + l] = l < cnt ? r.o1() / LD1 + n1 * (r.o2() / LD2) : -1;
+                    a.coef[(size_t)ko * s + l] = l < cnt ? r.x : 0.f;
+                }
+            if (gl == 0) {
+                const float e = fmaxf(E2, 0.f);
+                if (a.nnz) a.nnz[ko] = cnt;
+                if (a.res_energy) a.res_energy[ko] = finite ? e : __int_as_float(0x7fc00000);
+                if (finite) ksum(es, ec, e);
+                else record_error(a.err, SDL_ERR_NONFINITE);
+            }
+        }
+        __syncwarp();   // records are read before the next unit writes them
+        pos = pos_next;
+    }
+
+    // ---- residual energies of this CTA's signals, lanes and warps in a fixed
+    // order; the slots past the grid are cleared
+    if (a.esum) {
+        __syncthreads();
+        double* red = reinterpret_cast<double*>(sm);
+        double d = (double)es - (double)ec;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(kFull, d, o);
+        if (lane == 0) red[w] = d;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double tot = 0.0;
+            for (int v = 0; v < warps; ++v) tot += red[v];
+            for (int slot = blockIdx.x; slot < a.esum_slots; slot += gridDim.x) {
+                a.esum[2 * slot] = slot == (int)blockIdx.x ? tot : 0.0;
+                a.esum[2 * slot + 1] = 0.0;
+            }
+        }
+    }
+}
+
+// Launch on at most max_grid CTAs (0: no limit).  Large signals leave room for
+// fewer warps per CTA; SDL_ERR_UNSUPPORTED when not even one fits (the caller
+// takes the generic kernel).
+template <class C>
+int launch(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid) {
+    constexpr size_t kSmMax = 227 * 1024, kSmTotal = 228 * 1024;
+    int warps = C::WARPS;
+    size_t bytes;
+    while ((bytes = sizeof(float) * (size_t)layout<C>(a.p1, a.p2, a.s, warps).total) > kSmMax && warps > 1)
+        --warps;
+    if (bytes > kSmMax) return SDL_ERR_UNSUPPORTED;
+    auto kern = code_group_kernel<C>;
+    // the shared-memory opt-in, once per device
+    static bool attr[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
+    if (dev >= 64 || !attr[dev]) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmMax) != cudaSuccess)
+            return SDL_ERR_CUDA;
+        if (dev < 64) attr[dev] = true;
+    }
+    // the registers allow MINB CTAs per SM (launch bounds); 1 KB per CTA is reserved
+    const int bps = std::max(1, std::min<int>(C::MINB, (int)(kSmTotal / (bytes + 1024))));
+    const long long units = (a.N + C::SPW - 1) / C::SPW;
+    long long grid = std::max<long long>(1, std::min<long long>(units, (long long)num_sms * bps));
+    if (max_grid > 0) grid = std::min<long long>(grid, max_grid);
+    kern<<<(int)grid, warps * 32, bytes, st>>>(a);
+    return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
+}
+
+}  // namespace group
+}  // namespace sdl

@@ -943,12 +943,7 @@ int launch_code_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms) 
         const int r = launch_code_pass_fast(a, side, st, num_sms);
         if (r != SDL_ERR_UNSUPPORTED) return r;
     }
-    switch (side) {
-        case kCodeOnly: return dispatch_code<kCodeOnly>(a, st, num_sms);
-        case kSideD1: return dispatch_code<kSideD1>(a, st, num_sms);
-        case kSideD2: return dispatch_code<kSideD2>(a, st, num_sms);
-        default: return SDL_ERR_ARG;
-    }
+    return launch_code_pass_generic(a, side, st, num_sms);
 }
 
 int launch_code_pass_generic(const PassArgs& a, int side, cudaStream_t st, int num_sms,

@@ -1,0 +1,156 @@
+// Error-driven coding: the signals already within the error target, found and
+// given their empty code before the coder runs, and the list of the others.
+//
+// Most patches of a denoising call take no atom, and they come in clusters
+// (smooth regions), so a coder that meets them one by one spends its time
+// loading them at a coder's occupancy and its warps finish unevenly.  This pass
+// reads the signals at the memory's rate and the coder's units are then full
+// and evenly dealt.  Measured on the patches of a 512 x 512 image (13-19 % of them
+// over the target): 8x8 84 -> 39 us, 12x12 158 -> 94, 16x16 397 -> 221; the
+// three sizes as one batch 668 -> 362.  The same scan inside the coder
+// (32 signals at a time per warp, the others queued) took 90, 444 and 518 us.
+#include <algorithm>
+
+#include "sdl_internal.cuh"
+
+namespace sdl {
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kWarps = 8;           // a block scans 8 x 32 signals
+
+// A group of 8 lanes sums one signal, 4 signals per warp and step.  The partial
+// sums and their combining tree are the coders' (32 strided chains, then xor
+// 16, 8, 4, 2, 1), so the comparison with the target comes out the same: lane j
+// holds chains 4j .. 4j+3.  VEC: 16-byte loads (p1 p2 a multiple of 4, Y
+// 16-byte aligned).
+template <bool VEC>
+__global__ void __launch_bounds__(kWarps * 32)
+    energy_scan_kernel(const float* __restrict__ Y, int pp, long long N, float eps2, int s,
+                       int32_t* __restrict__ support, float* __restrict__ coef, int32_t* __restrict__ nnz,
+                       float* __restrict__ res_energy, int32_t* __restrict__ list, int* __restrict__ count) {
+    __shared__ int wcount[kWarps], base_s;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane >> 3, j = lane & 7;
+    const long long first = ((long long)blockIdx.x * kWarps + w) * 32;
+    const int m = (int)max(0LL, min(32LL, N - first));
+    float mine = 0.f;
+#pragma unroll 2
+    for (int it = 0; it < 8; ++it) {
+        const int i = it * 4 + grp;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (i < m) {
+            const float* src = Y + (size_t)(first + i) * pp;
+            if constexpr (VEC) {
+#pragma unroll 4
+                for (int e = 4 * j; e < pp; e += 32) {
+                    const float4 y = __ldg(reinterpret_cast<const float4*>(src + e));
+                    v[0] = fmaf(y.x, y.x, v[0]);
+                    v[1] = fmaf(y.y, y.y, v[1]);
+                    v[2] = fmaf(y.z, y.z, v[2]);
+                    v[3] = fmaf(y.w, y.w, v[3]);
+                }
+            } else {
+                for (int e = 4 * j; e < pp; e += 32)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (e + c < pp) {
+                            const float y = __ldg(src + e + c);
+                            v[c] = fmaf(y, y, v[c]);
+                        }
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], o);
+        const float ss = (v[0] + v[2]) + (v[1] + v[3]);
+        const float mv = __shfl_sync(kFull, ss, (lane & 3) * 8);
+        if ((lane >> 2) == it) mine = mv;
+    }
+    // lane i holds signal i of the warp
+    const bool have = lane < m;
+    const bool done = have && isfinite(mine) && mine <= eps2;
+    const unsigned dm = __ballot_sync(kFull, done), todo = __ballot_sync(kFull, have && !done);
+    if (done) {
+        if (nnz) nnz[first + lane] = 0;
+        if (res_energy) res_energy[first + lane] = mine;
+    }
+    if (support && dm) {
+        const unsigned inv_s = (65536u + s - 1) / s;   // e / s for e < 1024
+        for (int e = lane; e < 32 * s; e += 32)
+            if ((dm >> ((unsigned)e * inv_s >> 16)) & 1u) {
+                support[(size_t)first * s + e] = -1;
+                coef[(size_t)first * s + e] = 0.f;
+            }
+    }
+    if (lane == 0) wcount[w] = __popc(todo);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int tot = 0;
+        for (int v = 0; v < kWarps; ++v) {
+            const int c = wcount[v];
+            wcount[v] = tot;
+            tot += c;
+        }
+        base_s = tot ? atomicAdd(count, tot) : 0;   // the list's order does not matter
+    }
+    __syncthreads();
+    if (have && !done) list[base_s + wcount[w] + __popc(todo & ((1u << lane) - 1u))] = (int32_t)(first + lane);
+}
+
+}  // namespace
+
+// The list fits the scratch in at most kSegments parts (4 floats hold the count).
+constexpr long long kSegments = 8;
+long long list_capacity(size_t ws_n) {
+    return ws_n < 64 ? 0 : std::min<long long>((long long)(ws_n - 4) & ~3LL, 1LL << 30);
+}
+
+// Code-only passes that the lane-group coder takes, given ws_n floats of scratch
+// for the list of an error-driven call.
+bool code_lanes_take(const PassArgs& a, size_t ws_n) {
+    // correlations from the tensor cores, a pinned tiling and wider dictionaries
+    // have coders of their own
+    if (a.c0ext || a.tiling > 0 || a.n1 > 32 || a.n2 > 32) return false;
+    return !(a.eps2 > 0.f) || (!a.idx && a.N <= kSegments * list_capacity(ws_n));
+}
+
+// ws: ws_n floats of scratch (null: none).  SDL_ERR_UNSUPPORTED, with nothing
+// launched, for a call that it does not take.
+int launch_code_lanes(const PassArgs& a, float* ws, size_t ws_n, cudaStream_t st, int num_sms) {
+    if (!code_lanes_take(a, ws ? ws_n : 0)) return SDL_ERR_UNSUPPORTED;
+    const bool aligned = (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0;
+    auto code = [&](const PassArgs& q) -> int {
+        // the compiled shapes keep their tilings' arithmetic, which they have
+        // only with aligned signals
+        const int r = aligned ? launch_code_group_fixed(q, false, st, num_sms) : SDL_ERR_UNSUPPORTED;
+        return r != SDL_ERR_UNSUPPORTED ? r : launch_code_group_any(q, st, num_sms);
+    };
+    if (!(a.eps2 > 0.f)) return code(a);
+    const long long cap = list_capacity(ws_n);
+    const int pp = a.p1 * a.p2;
+    int* count = reinterpret_cast<int*>(ws);
+    int32_t* list = reinterpret_cast<int32_t*>(ws + 4);
+    for (long long k0 = 0; k0 < a.N; k0 += cap) {
+        PassArgs q = a;
+        q.N = std::min(cap, a.N - k0);
+        q.Y = a.Y + (size_t)k0 * pp;
+        q.support = a.support ? a.support + (size_t)k0 * a.s : nullptr;
+        q.coef = a.coef ? a.coef + (size_t)k0 * a.s : nullptr;
+        q.nnz = a.nnz ? a.nnz + k0 : nullptr;
+        q.res_energy = a.res_energy ? a.res_energy + k0 : nullptr;
+        if (cudaMemsetAsync(count, 0, sizeof(int), st) != cudaSuccess) return SDL_ERR_CUDA;
+        const unsigned blocks = (unsigned)((q.N + kWarps * 32 - 1) / (kWarps * 32));
+        auto kern = aligned && pp % 4 == 0 ? energy_scan_kernel<true> : energy_scan_kernel<false>;
+        kern<<<blocks, kWarps * 32, 0, st>>>(q.Y, pp, q.N, a.eps2, a.s, q.support, q.coef, q.nnz, q.res_energy, list,
+                                             count);
+        if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
+        q.idx = list;
+        q.idx_count = count;
+        const int r = code(q);
+        if (r != SDL_OK) return r;
+    }
+    return SDL_OK;
+}
+
+}  // namespace sdl

@@ -65,6 +65,10 @@ struct PassArgs {
     // as fit)
     int tiling;
     int tiling_cps;
+    // lane-group coder only, optional: per-CTA sums of the residual energies,
+    // [esum_slots][2] (entry 0; slots past its grid and entries 1 are cleared)
+    double* esum;
+    int esum_slots;
 };
 
 // Host launchers (omp_pass.cu).  They return the number of partial-sum
@@ -76,6 +80,18 @@ int launch_code_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms);
 int launch_code_pass_generic(const PassArgs& a, int side, cudaStream_t st, int num_sms,
                              bool plan_only = false);
 int launch_accumulate_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms);
+// omp_group_*.cu: code-only passes with 8 or 16 lanes per signal, in the
+// arithmetic of the compiled tilings (fixed: their shapes; w_first: correlations
+// as (D1^T Y) D2, at most max_grid CTAs) or of the generic kernel (any: n1, n2 <=
+// 32).  SDL_ERR_UNSUPPORTED for other shapes.
+int launch_code_group_fixed(const PassArgs& a, bool w_first, cudaStream_t st, int num_sms,
+                            int max_grid = 0);
+int launch_code_group_any(const PassArgs& a, cudaStream_t st, int num_sms);
+int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms);
+// omp_scan.cu: the above for a code-only call, behind an error scan when it is
+// error-driven (ws: ws_n floats of scratch, or null)
+bool code_lanes_take(const PassArgs& a, size_t ws_n);
+int launch_code_lanes(const PassArgs& a, float* ws, size_t ws_n, cudaStream_t st, int num_sms);
 // omp_fast.cu: compile-time-shape kernels; SDL_ERR_UNSUPPORTED when no
 // specialisation matches (the caller then uses the generic kernel).
 int launch_code_pass_fast(const PassArgs& a, int side, cudaStream_t st, int num_sms);

@@ -90,13 +90,6 @@ extern "C" int sdl_sparse_code_static(const float* Y, int p1, int p2, int64_t N,
     cudaStream_t st = (cudaStream_t)stream;
     float* G1 = scratch;
     float* G2 = scratch + n1 * n1;
-    // Both Grams are fully rewritten before the coding pass reads them, so
-    // nothing left over from an earlier call is used.
-    launch_gram(D1, p1, n1, G1, st);
-    if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
-    launch_gram(D2, p2, n2, G2, st);
-    if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
-
     PassArgs a{};
     a.Y = Y;
     a.p1 = p1;
@@ -116,6 +109,17 @@ extern "C" int sdl_sparse_code_static(const float* Y, int p1, int p2, int64_t N,
     a.res_energy = res_energy;
     a.n_slots = 1;
     a.err = err;       // read by sdl_static_status
+    // calls with a fixed sparsity form the Grams inside the coder; the others run
+    // the coders that read them from memory
+    rc = launch_code_lanes(a, nullptr, 0, st, num_sms);
+    if (rc != SDL_ERR_UNSUPPORTED) return rc;
+    // Both Grams are fully rewritten before the coding pass reads them, so
+    // nothing left over from an earlier call is used.
+    launch_gram(D1, p1, n1, G1, st);
+    if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
+    launch_gram(D2, p2, n2, G2, st);
+    if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
+
     rc = launch_code_pass(a, kCodeOnly, st, num_sms);
     return rc < 0 ? rc : SDL_OK;
 }
