@@ -58,7 +58,8 @@ __global__ void reconstruct_patches_kernel(const int32_t* __restrict__ support,
         x = coef[k * s + lane];
     }
     const float mean = means[k];
-    for (int e = lane; e < pp; e += 32) {
+    for (int e0 = 0; e0 < pp; e0 += 32) {   // every lane stays in the loop: the picks travel by shuffles
+        const int e = min(e0 + lane, pp - 1);
         const int a = e % p, b = e / p;
         float v = mean;
         for (int l = 0; l < s; ++l) {
@@ -69,7 +70,7 @@ __global__ void reconstruct_patches_kernel(const int32_t* __restrict__ support,
                 v = fmaf(xl * D1[a + p * i], D2[b + p * j], v);
             }
         }
-        rec[(size_t)k * pp + e] = v;
+        if (e0 + lane < pp) rec[(size_t)k * pp + e] = v;
     }
 }
 
