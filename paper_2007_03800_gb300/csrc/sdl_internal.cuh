@@ -116,6 +116,11 @@ int launch_code_pass_variant(const PassArgs& a, int side, int shape_id, int ctas
 int launch_code_multi(const PassArgs* d_groups, const int* d_cta_begin, const int* d_shape, int G,
                       int total_ctas, size_t smem, int side, cudaStream_t st, int spread = 0);
 int multi_ctas_per_sm(size_t smem, int side);
+// accum.cu: partial sums of one side from given codes (a.in_support, a.in_coef),
+// up to 32 atoms and rows on that side; the residual energy with the given
+// dictionaries only if wanted.  Returns the slots written, or
+// SDL_ERR_UNSUPPORTED.  Needs no Gram matrices.
+int launch_accumulate_lanes(const PassArgs& a, int side, bool want_energy, cudaStream_t st, int num_sms);
 bool code_shape_supported(int p1, int p2, int n1, int n2, int s);
 // Upper bound of the partial-sum slots any pass may use for these sizes.
 int max_partial_slots(int num_sms);
