@@ -169,19 +169,33 @@ __global__ void topk_kernel(const float* __restrict__ Z, int ldz, long long N, i
         for (int e = 0; e < EQ; ++e) c += key[e] >= t ? 1 : 0;
         return (int)__reduce_add_sync(kFull, (unsigned)c);
     };
-    // largest threshold with at least kk keys >= it
-    auto threshold = [&](int kk) {
+    // largest threshold with at least kk keys >= it, or the first one met with
+    // exactly kk: then no key ties for the last place, and the set is the same
+    auto threshold = [&](int kk, bool& exact) {
         unsigned t = 0;
+        exact = false;
         for (int bit = 16; bit >= 0; --bit) {
             const unsigned c = t | (1u << bit);
-            if (count_ge(c) >= kk) t = c;
+            const int n = count_ge(c);
+            if (n >= kk) t = c;
+            if (n == kk) {
+                exact = true;
+                break;
+            }
         }
         return t;
     };
     // membership masks of the top-kk set (ties at the threshold by smaller q)
     auto select = [&](int kk) {
-        const unsigned t = threshold(kk);
+        bool exact;
+        const unsigned t = threshold(kk, exact);
         unsigned mask = 0;
+        if (exact) {
+#pragma unroll
+            for (int e = 0; e < EQ; ++e)
+                if (key[e] >= t) mask |= 1u << e;
+            return mask;
+        }
         int above = 0;
 #pragma unroll
         for (int e = 0; e < EQ; ++e) {
@@ -246,6 +260,7 @@ __global__ void __launch_bounds__(256) shortlist_omp_kernel(
     float* __restrict__ coef, int32_t* __restrict__ nnz, float* __restrict__ res_energy,
     int32_t* __restrict__ flag) {
     constexpr int PP = P1 * P2;
+    static_assert(N1 <= 32 && N2 <= 32, "one lane per atom, one bit per j");
     __shared__ float D1c[N1 * P1];       // column i contiguous
     __shared__ float D2r[P2 * N2];       // row b contiguous
     __shared__ float G1s[N1 * N1], G2s[N2 * N2];
@@ -356,21 +371,33 @@ __global__ void __launch_bounds__(256) shortlist_omp_kernel(
 #pragma unroll
         for (int m = 0; m < S; ++m)
             if (lane == m) myx = xs[m];
-        // fallback test over every pair not picked (lane takes q = lane + 32 e)
+        // fallback test over every pair not picked: lane = atom i (two lanes
+        // per atom, on alternate j, when N1 <= 16), its column of D1 and its
+        // factors -x_l G1[i, i_l] in registers; the maximum does not depend on
+        // the order of the pairs
         float ve = 0.f;
         if (cnt == S) {
-            for (int qq = lane; qq < N1 * N2; qq += 32) {
-                const int i = qq % N1, j = qq / N1;
-                bool picked = false;
+            constexpr int LJ = N1 <= 16 ? 2 : 1;
+            const int i = lane % (32 / LJ), j0 = lane / (32 / LJ);
+            if (i < N1) {
+                float d[P1], gx[S];
+                unsigned pm = 0;   // the picked j of this atom
 #pragma unroll
-                for (int l = 0; l < S; ++l) picked |= (si[l] == i && sj[l] == j);
-                if (picked) continue;
-                float sce = 0.f;
+                for (int a = 0; a < P1; ++a) d[a] = D1c[i * P1 + a];
 #pragma unroll
-                for (int a = 0; a < P1; ++a) sce = fmaf(D1c[i * P1 + a], Zs[a * N2 + j], sce);
+                for (int l = 0; l < S; ++l) {
+                    gx[l] = -xs[l] * G1s[i * N1 + si[l]];
+                    pm |= (si[l] == i ? 1u : 0u) << sj[l];
+                }
+#pragma unroll 4
+                for (int j = j0; j < N2; j += LJ) {
+                    float sce = 0.f;
 #pragma unroll
-                for (int l = 0; l < S; ++l) sce = fmaf(-xs[l] * G1s[i * N1 + si[l]], G2s[sj[l] * N2 + j], sce);
-                ve = fmaxf(ve, fabsf(sce));
+                    for (int a = 0; a < P1; ++a) sce = fmaf(d[a], Zs[a * N2 + j], sce);
+#pragma unroll
+                    for (int l = 0; l < S; ++l) sce = fmaf(gx[l], G2s[sj[l] * N2 + j], sce);
+                    if (!((pm >> j) & 1u)) ve = fmaxf(ve, fabsf(sce));
+                }
             }
         }
         const float maxe = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(ve)));
@@ -699,23 +726,64 @@ int sdl_mlp_gradients(sdl_mlp* m, const float* Y, const int32_t* support, int s,
     return SDL_OK;
 }
 
-// Scores of N signals (device FP32 N x n1n2), processed in chunks of max_batch.
+// Inference runs in chunks of this many signals: a 4096-signal chunk leaves
+// every SM one 128 x 128 tile per GEMM, so that nothing hides the epilogue's GELU
+// (23 us per chunk at 64 -> 512; 8 times the signals take ...), while the
+// activations and scores of a chunk still stay in L2.
+constexpr int64_t kInferChunk = 32768;
+
+static size_t infer_bytes(const sdl_mlp* m, int64_t rows) {
+    return (size_t)rows * (m->Kp + m->H) * sizeof(bf16) + 2 * 256;
+}
+
+// Grow the context's learned-coder workspace.
+static int learn_workspace(sdl_ctx* c, size_t need) {
+    if (need <= c->cap_learn) return SDL_OK;
+    if (c->learn) cudaFree(c->learn);
+    c->learn = nullptr;
+    c->cap_learn = 0;
+    if (cudaMalloc(&c->learn, need) != cudaSuccess) {
+        cudaGetLastError();
+        return SDL_ERR_WORKSPACE;
+    }
+    c->cap_learn = need;
+    return SDL_OK;
+}
+
+// Scores of `rows` signals (at most the rows that Xb and Hb hold).
+static int infer_rows(sdl_mlp* m, const float* Y, int64_t rows, bf16* Xb, bf16* Hb, float* scores,
+                      cudaStream_t st) {
+    sdl_ctx* c = m->ctx;
+    const int H = m->H, Kp = m->Kp, Q = m->Q, B = (int)rows;
+    prep_input_kernel<<<blocks_for(rows * 32, 256), 256, 0, st>>>(Y, B, m->P, Kp, Xb, Kp, nullptr, 0);
+    const int rc = tc_gemm(Xb, Kp, m->W1b, Kp, B, H, Kp, 1.f, m->b1, 1, nullptr, 0, 0, Hb, H, nullptr, 0, nullptr,
+                           0, c->err, st);
+    if (rc) return rc;
+    return tc_gemm(Hb, H, m->W2b, H, B, Q, H, 1.f, m->b2, 0, scores, Q, 0, nullptr, 0, nullptr, 0, nullptr, 0,
+                   c->err, st);
+}
+
+// Scores of N signals (device FP32 N x n1n2).
 int sdl_mlp_forward(sdl_mlp* m, const float* Y, int64_t N, float* scores, void* stream) {
     if (!m || (N > 0 && (!Y || !scores)) || N < 0) return SDL_ERR_ARG;
     DeviceGuard guard(m->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     sdl_ctx* c = m->ctx;
-    const int H = m->H, Kp = m->Kp, Q = m->Q;
+    // a call within the training batch uses the network's own buffers
+    bf16 *Xb = m->Xb, *Hb = m->Hb;
+    int64_t chunk = m->Bmax;
+    if (N > chunk) {
+        chunk = std::max<int64_t>(chunk, std::min<int64_t>(N, kInferChunk));
+        const int rc = learn_workspace(c, infer_bytes(m, chunk));
+        if (rc) return rc;
+        char* p = c->learn;
+        Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
+        Hb = carve<bf16>(p, (size_t)chunk * m->H);
+    }
     Trace tr(c, kMlp, st);
-    for (int64_t r0 = 0; r0 < N; r0 += m->Bmax) {
-        const int B = (int)std::min<int64_t>(m->Bmax, N - r0);
-        prep_input_kernel<<<blocks_for((long long)B * 32, 256), 256, 0, st>>>(
-            Y + (size_t)r0 * m->P, B, m->P, Kp, m->Xb, Kp, nullptr, 0);
-        int rc = tc_gemm(m->Xb, Kp, m->W1b, Kp, B, H, Kp, 1.f, m->b1, 1, nullptr, 0, 0, m->Hb, H,
-                         nullptr, 0, nullptr, 0, c->err, st);
-        if (!rc)
-            rc = tc_gemm(m->Hb, H, m->W2b, H, B, Q, H, 1.f, m->b2, 0, scores + (size_t)r0 * Q, Q, 0,
-                         nullptr, 0, nullptr, 0, nullptr, 0, c->err, st);
+    for (int64_t r0 = 0; r0 < N; r0 += chunk) {
+        const int64_t B = std::min<int64_t>(chunk, N - r0);
+        const int rc = infer_rows(m, Y + (size_t)r0 * m->P, B, Xb, Hb, scores + (size_t)r0 * m->Q, st);
         if (rc) return rc;
     }
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
@@ -756,24 +824,17 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     cudaStream_t st = (cudaStream_t)stream;
     const int k2 = k, Q = m->Q;     // the shortlist only: the fallback test scans every pair
     // workspace: scores of one chunk, candidates, Grams, scan buffers, index list
-    const long long chunk = m->Bmax;
+    const long long chunk = std::max<long long>(m->Bmax, std::min<long long>(N, kInferChunk));
     const int nblk = (int)((N + kScanBlock - 1) / kScanBlock);
     const long long m_s = std::min<long long>(N, std::max<long long>(kGuardMinSample, N / 16));
     const long long stride_s = N / m_s;
     const size_t need = sizeof(float) * (size_t)chunk * Q + sizeof(int32_t) * (size_t)N * k2 +
                         sizeof(float) * (size_t)(n1 * n1 + n2 * n2) + sizeof(int) * (nblk + 8) +
                         sizeof(int32_t) * (size_t)N + sizeof(int32_t) * (size_t)m_s +
-                        sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + 10 * 256;
-    if (need > c->cap_learn) {
-        if (c->learn) cudaFree(c->learn);
-        c->learn = nullptr;
-        c->cap_learn = 0;
-        if (cudaMalloc(&c->learn, need) != cudaSuccess) {
-            cudaGetLastError();
-            return SDL_ERR_WORKSPACE;
-        }
-        c->cap_learn = need;
-    }
+                        sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + 10 * 256 +
+                        infer_bytes(m, chunk);
+    int rc = learn_workspace(c, need);
+    if (rc) return rc;
     char* p = c->learn;
     float* scores = carve<float>(p, (size_t)chunk * Q);
     int32_t* cand = carve<int32_t>(p, (size_t)N * k2);
@@ -785,7 +846,8 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     float* plainE = carve<float>(p, (size_t)m_s);
     float* learnedE = res_energy ? res_energy : carve<float>(p, (size_t)N);
     int* cnt_s = carve<int>(p, 2);
-    int rc;
+    bf16* Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
+    bf16* Hb = carve<bf16>(p, (size_t)chunk * m->H);
     {
         Trace tr(c, kGram, st);
         launch_gram2(D1, p1, n1, G1, D2, p2, n2, G2, st);
@@ -793,7 +855,10 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     // 1. scores and shortlists, chunk by chunk
     for (int64_t r0 = 0; r0 < N; r0 += chunk) {
         const int B = (int)std::min<int64_t>(chunk, N - r0);
-        if ((rc = sdl_mlp_forward(m, Y + (size_t)r0 * p1 * p2, B, scores, stream))) return rc;
+        {
+            Trace tr(c, kMlp, st);
+            if ((rc = infer_rows(m, Y + (size_t)r0 * p1 * p2, B, Xb, Hb, scores, st))) return rc;
+        }
         Trace tr(c, kTopk, st);
         if (Q <= 256)
             topk_kernel<8><<<blocks_for((long long)B * 32, 256), 256, 0, st>>>(

@@ -48,15 +48,17 @@ using namespace sdl;
 namespace {
 
 constexpr int BM = 128, BK = 64, UMMA_K = 16;
-// shared-memory ring depth: as many stages as fit beside the epilogue's staging
-__host__ __device__ constexpr int stages_for(int BN) { return BN == 256 ? 4 : 6; }
 constexpr int kMaxTerms = 3;
-constexpr int kThreads = 192;
-constexpr int kEpiWarps = 4;
-constexpr int kStageLd = 33;                  // epilogue transpose row stride (floats)
-constexpr int kSlot = 4096;                   // one TMA output slot: 32 rows x 128 B
-constexpr int kEpiBytes = kEpiWarps * 2 * kSlot;   // both epilogue forms share this area
-static_assert(kEpiWarps * 32 * kStageLd * 4 <= kEpiBytes, "transpose staging must fit");
+// EW epilogue warps (4 or 16), each with its share of kEpiBytes: TMA output
+// slots of 32 rows x 128 B, or the 32 x 32 transpose staging of the other outputs
+constexpr int kSlot = 4096;
+__host__ __device__ constexpr int slots_for(int EW) { return EW == 4 ? 2 : 1; }
+__host__ __device__ constexpr int epi_bytes(int EW) { return EW * slots_for(EW) * kSlot; }
+// shared-memory ring depth: as many stages as fit beside the epilogue's staging
+__host__ __device__ constexpr int stages_for(int BN, int EW) {
+    return EW == 4 ? (BN == 256 ? 4 : 6) : (BN == 256 ? 3 : 5);
+}
+constexpr int threads_for(int EW) { return 64 + 32 * EW; }
 constexpr int TILE_A = BM * BK * 2;           // bytes
 constexpr long long kWaitCycles = 1ll << 31;  // about one second at 2 GHz
 
@@ -198,12 +200,28 @@ __device__ __forceinline__ void tmem_ld64(uint32_t ta, uint32_t (&v)[64]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kThreads, 1)
+// 32 columns of it (the 16-warp epilogue, at half the registers)
+__device__ __forceinline__ void tmem_ld32(uint32_t ta, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {"
+        "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, "
+        "%19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31 "
+        "}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+          "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
+          "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
+          "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(ta));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+template <int BN, int EW>
+__global__ void __launch_bounds__(threads_for(EW), 1)
     tc_gemm_kernel(const __grid_constant__ Maps maps, int terms, int M, int N, int K, Epi epi,
                    int* err) {
     constexpr int TILE_B = BN * BK * 2;
-    constexpr int STAGES = stages_for(BN);
+    constexpr int STAGES = stages_for(BN, EW), kEpiBytes = epi_bytes(EW);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~uintptr_t(1023));
@@ -212,7 +230,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     // epilogue area (1024-byte aligned): two TMA slots per warp, or the
     // transpose staging of the other outputs
     uint8_t* epi_area = sB + STAGES * TILE_B;
-    float* stage_all = reinterpret_cast<float*>(epi_area);
     uint64_t* full = reinterpret_cast<uint64_t*>(epi_area + kEpiBytes);
     uint64_t* empty = full + STAGES;
     uint64_t* acc_full = empty + STAGES;      // [2] MMA -> epilogue
@@ -235,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], kEpiWarps);
+            mbar_init(&acc_empty[b], EW);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -317,10 +334,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     } else {
-        // ---- epilogue warps
+        // ---- epilogue warps: 4 cover the 128 rows; with 16, four groups of 4
+        // take every fourth 32-column block (the activations' latency, and the
+        // row-by-row outputs, need more warps than the TMEM quarters)
+        constexpr int CB = EW == 4 ? 64 : 32;      // columns per TMEM load
+        constexpr int CSTEP = EW == 4 ? 64 : 128;
         const int quarter = warp & 3;              // TMEM lanes this warp may access
-        float* stage = stage_all + (warp - 2) * 32 * kStageLd;
-        uint8_t* slots = epi_area + (warp - 2) * 2 * kSlot;
+        const int cfirst = EW == 4 ? 0 : ((warp - 2) >> 2) * 32;
+        uint8_t* slots = epi_area + (warp - 2) * slots_for(EW) * kSlot;
+        float* stage = reinterpret_cast<float*>(slots);
+        // element (row, column) of the transpose staging, conflict-free both ways
+        auto sidx = [](int row, int column) { return row * 32 + (column ^ row); };
         int slot = 0;
         int i = 0;
         for (long long t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
@@ -333,18 +357,20 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int m0 = (int)(t / nt) * BM, n0 = (int)(t % nt) * BN;
             const int row0 = m0 + quarter * 32;    // first output row of this warp
             const int m = row0 + lane;
-            for (int c64 = 0; c64 < BN; c64 += 64) {
-                uint32_t v[64];
-                tmem_ld64(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + c64), v);
-                if (c64 + 64 == BN) {
-                    // the whole accumulator has been read: hand it back
+            for (int cb = cfirst; cb < BN; cb += CSTEP) {
+                uint32_t v[CB];
+                const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + cb);
+                if constexpr (EW == 4) tmem_ld64(ta, v);
+                else tmem_ld32(ta, v);
+                if (cb + CSTEP >= BN) {
+                    // this warp has read its part of the accumulator: hand it back
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[b]);
                 }
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int c0 = c64 + 32 * h;   // this 32-column block
+              for (int h = 0; h < CB / 32; ++h) {
+                const int c0 = cb + 32 * h;   // this 32-column block
                 float x[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
@@ -360,12 +386,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                             x[j] = 0.5f * x[j] * (1.f + erff(x[j] * 0.70710678118654752f));
                     }
                     if (n0 + c0 >= N || row0 >= M) continue;   // block wholly outside C
-                    // a slot is rewritten only after the store issued from it two
-                    // stores ago has read it
+                    // a slot is rewritten only after the store issued from it (one or
+                    // two stores ago) has read it
                     auto next_slot = [&]() {
                         uint8_t* buf = slots + slot * kSlot;
-                        slot ^= 1;
-                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        if constexpr (slots_for(EW) == 2) {
+                            slot ^= 1;
+                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        } else {
+                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        }
                         __syncwarp();
                         return buf;
                     };
@@ -408,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 auto store_rows = [&](float* dst, int ld, int accumulate) {
                     __syncwarp();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) stage[lane * kStageLd + j] = x[j];
+                    for (int j = 0; j < 32; ++j) stage[sidx(lane, j)] = x[j];
                     __syncwarp();
                     const int n = n0 + c0 + lane;
                     if (accumulate) {
@@ -423,12 +453,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                         for (int rr = 0; rr < 32; ++rr) {
                             const int mm = row0 + rr;
                             if (mm < M && n < N)
-                                dst[(size_t)mm * ld + n] = old[rr] + stage[rr * kStageLd + lane];
+                                dst[(size_t)mm * ld + n] = old[rr] + stage[sidx(rr, lane)];
                         }
                     } else {
+#pragma unroll 8
                         for (int rr = 0; rr < 32; ++rr) {
                             const int mm = row0 + rr;
-                            if (mm < M && n < N) dst[(size_t)mm * ld + n] = stage[rr * kStageLd + lane];
+                            if (mm < M && n < N) dst[(size_t)mm * ld + n] = stage[sidx(rr, lane)];
                         }
                     }
                 };
@@ -442,15 +473,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // gin block arrives through the transpose buffer
                     __syncwarp();
                     const int n = n0 + c0 + lane;
+#pragma unroll 16
                     for (int rr = 0; rr < 32; ++rr) {
                         const int mm = row0 + rr;
-                        stage[rr * kStageLd + lane] =
+                        stage[sidx(rr, lane)] =
                             (mm < M && n < N) ? epi.gin[(size_t)mm * epi.ldgin + n] : 0.f;
                     }
                     __syncwarp();
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
-                        const float u = stage[lane * kStageLd + j];
+                        const float u = stage[sidx(lane, j)];
                         const float Phi = 0.5f * (1.f + erff(u * 0.70710678118654752f));
                         const float phi = 0.3989422804014327f * expf(-0.5f * u * u);
                         x[j] *= Phi + u * phi;
@@ -460,14 +492,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (epi.Cb) {
                     __syncwarp();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) stage[lane * kStageLd + j] = x[j];
+                    for (int j = 0; j < 32; ++j) stage[sidx(lane, j)] = x[j];
                     __syncwarp();
                     const int n = n0 + c0 + lane;
                     for (int rr = 0; rr < 32; ++rr) {
                         const int mm = row0 + rr;
                         if (mm < M && n < N)
                             epi.Cb[(size_t)mm * epi.ldcb + n] =
-                                __float2bfloat16_rn(stage[rr * kStageLd + lane]);
+                                __float2bfloat16_rn(stage[sidx(rr, lane)]);
                     }
                 }
                 if (epi.Ct && m < M) {
@@ -528,10 +560,12 @@ int make_map(CUtensorMap* map, const void* ptr, int rows, int cols, int ld, int 
     return r == CUDA_SUCCESS ? SDL_OK : SDL_ERR_ARG;
 }
 
-constexpr size_t smem_bytes(int BN) {
-    return 1024 + (size_t)stages_for(BN) * (TILE_A + BN * BK * 2) + kEpiBytes + 256;
+constexpr size_t smem_bytes(int BN, int EW) {
+    return 1024 + (size_t)stages_for(BN, EW) * (TILE_A + BN * BK * 2) + epi_bytes(EW) + 256;
 }
-static_assert(smem_bytes(256) <= 232448 && smem_bytes(128) <= 232448, "shared memory per CTA");
+static_assert(smem_bytes(256, 4) <= 232448 && smem_bytes(128, 4) <= 232448 && smem_bytes(256, 16) <= 232448 &&
+                  smem_bytes(128, 16) <= 232448,
+              "shared memory per CTA");
 
 // output map: rows x cols matrix of 4-byte (f32) or 2-byte (bf16) elements,
 // row stride ld elements, 32 x 32 boxes swizzled to match the epilogue's slots
@@ -586,6 +620,9 @@ int cached_map(CUtensorMap* out, const MapKey& k, Encode encode) {
     c.map[slot] = *out;
     return SDL_OK;
 }
+
+// contraction length up to which the 16-warp epilogue is taken
+constexpr long long kShortK = 1024;
 
 int sm_count() {
     static int count[64] = {0};
@@ -666,13 +703,13 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
                   return make_out_map(m, Cb, M, N, ldcb, true);
               }) == SDL_OK;
     e.tma = tma ? 1 : 0;
-    auto launch = [&](auto kern, int BN) -> int {
-        const size_t bytes = smem_bytes(BN);
-        // the shared-memory opt-in is set once per device and tile width
-        static bool attr_set[2][64] = {};
+    auto launch = [&](auto kern, int BN, int EW) -> int {
+        const size_t bytes = smem_bytes(BN, EW);
+        // the shared-memory opt-in is set once per device and variant
+        static bool attr_set[4][64] = {};
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-        bool& done = attr_set[BN == 256][dev & 63];
+        bool& done = attr_set[(BN == 256) + 2 * (EW == 16)][dev & 63];
         if (!done || dev >= 64) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
                 cudaSuccess)
@@ -681,10 +718,14 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
         }
         const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
         const int grid = (int)std::min<long long>(tiles, sm_count());
-        kern<<<grid, kThreads, bytes, st>>>(maps, terms, M, N, K, e, err);
+        kern<<<grid, threads_for(EW), bytes, st>>>(maps, terms, M, N, K, e, err);
         return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
     };
-    return bn == 256 ? launch(tc_gemm_kernel<256>, 256) : launch(tc_gemm_kernel<128>, 128);
+    // 16 epilogue warps where a tile's epilogue outlasts its main loop: an
+    // activation, an output that leaves row by row, or a short contraction
+    const bool wide = act != 0 || !tma || (long long)K * terms <= kShortK;
+    if (bn == 256) return wide ? launch(tc_gemm_kernel<256, 16>, 256, 16) : launch(tc_gemm_kernel<256, 4>, 256, 4);
+    return wide ? launch(tc_gemm_kernel<128, 16>, 128, 16) : launch(tc_gemm_kernel<128, 4>, 128, 4);
 }
 
 int tc_gemm(const void* A, int lda, const void* B, int ldb, int M, int N, int K, float alpha,
