@@ -219,6 +219,9 @@ int sdl_destroy(sdl_ctx* c) {
     cudaFree(c->KT);
     cudaFree(c->C0);
     cudaFree(c->rescored);
+    for (cudaEvent_t e : c->side_ev)
+        if (e) cudaEventDestroy(e);
+    if (c->side) cudaStreamDestroy(c->side);
     for (auto& r : c->recs) {
         cudaEventDestroy(r.beg);
         cudaEventDestroy(r.end);

@@ -56,6 +56,10 @@ struct sdl_ctx {
         std::vector<float> log_cost;
     };
     std::vector<BatchTune> batch_tunes;
+    // second stream of a training batch (mlp.cu): the gradients that nothing
+    // waits for until the parameter update run beside the backward GEMMs
+    cudaStream_t side = nullptr;
+    cudaEvent_t side_ev[3] = {};
     // tracing: launch counters and (optionally) one event pair per launch
     struct Rec {
         int kind;

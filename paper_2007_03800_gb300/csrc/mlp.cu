@@ -58,75 +58,181 @@ __global__ void prep_input_kernel(const float* __restrict__ Y, long long N, int 
     }
 }
 
-// dz = (sigmoid(z) - t) * scale, loss terms softplus(z) - t z; one block per row
-__global__ void bce_kernel(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ sup,
-                           int s, int Q, float scale, bf16* __restrict__ dZ, int lddz,
-                           bf16* __restrict__ dZT, int lddt, float* __restrict__ lossp) {
-    __shared__ int ssup[32];
-    __shared__ float red[32];
-    const int b = blockIdx.x;
-    if (threadIdx.x < s) ssup[threadIdx.x] = sup[(size_t)b * s + threadIdx.x];
-    __syncthreads();
-    float acc = 0.f;
-    for (int q = threadIdx.x; q < Q; q += blockDim.x) {
-        float t = 0.f;
-        for (int l = 0; l < s; ++l) t = (ssup[l] == q) ? 1.f : t;
-        const float z = Z[(size_t)b * ldz + q];
-        acc += fmaxf(z, 0.f) - t * z + log1pf(expf(-fabsf(z)));
-        const float g = (1.f / (1.f + expf(-z)) - t) * scale;
-        const bf16 gb = __float2bfloat16_rn(g);
-        dZ[(size_t)b * lddz + q] = gb;
-        dZT[(size_t)q * lddt + b] = gb;
-    }
+// The same for a training batch, with the transposed copy: a block takes 32
+// signals, and both copies leave as coalesced rows (the norm, in the same order,
+// by one warp per signal).
+__global__ void __launch_bounds__(256) prep_batch_kernel(const float* __restrict__ Y, int N, int P, int Kp,
+                                                         bf16* __restrict__ X, bf16* __restrict__ XT, int ldt) {
+    __shared__ float inv_s[32];
+    __shared__ bf16 tile[32][66];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, k0 = blockIdx.x * 32;
+    for (int i = w; i < 32; i += 8) {
+        float ss = 0.f;
+        if (k0 + i < N) {
+            const float* y = Y + (size_t)(k0 + i) * P;
+            for (int e = lane; e < P; e += 32) ss = fmaf(y[e], y[e], ss);
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
+        if (lane == 0) inv_s[i] = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        lossp[b] = t;
+    for (int e0 = 0; e0 < Kp; e0 += 64) {
+        for (int t = threadIdx.x; t < 32 * 64; t += 256) {
+            const int i = t >> 6, e = e0 + (t & 63), k = k0 + i;
+            bf16 v = __float2bfloat16_rn(0.f);
+            if (k < N && e < P) v = __float2bfloat16_rn(Y[(size_t)k * P + e] * inv_s[i]);
+            if (k < N && e < Kp) X[(size_t)k * Kp + e] = v;
+            tile[i][t & 63] = v;
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < 32 * 64; t += 256) {
+            const int e = e0 + (t >> 5), k = k0 + (t & 31);
+            if (k < N && e < Kp) XT[(size_t)e * ldt + k] = tile[t & 31][t >> 5];
+        }
+        __syncthreads();
     }
 }
 
-// out[r] = sum_c M[r, c] (BF16 rows), one warp per row, fixed order
-__global__ void rowsum_kernel(const bf16* __restrict__ M, int ld, int R, int C,
-                              float* __restrict__ out) {
-    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (r >= R) return;
+// dz = (sigmoid(z) - t) * scale, loss terms softplus(z) - t z; a block takes 32
+// signals x 64 scores, so that dZ and its transpose leave as coalesced rows
+// (one block per signal wrote the transpose 2 bytes at a time: 29 us for a batch of
+// 4096 x 576).  lossp: one sum per (column block, signal).
+constexpr int kBceCols = 64;
+
+__global__ void __launch_bounds__(256)
+    bce_kernel(const float* __restrict__ Z, int ldz, const int32_t* __restrict__ sup, int s, int B, int Q,
+               float scale, bf16* __restrict__ dZ, int lddz, bf16* __restrict__ dZT, int lddt,
+               float* __restrict__ lossp) {
+    __shared__ unsigned long long hit[32];     // bit c: pair q0 + c is in the signal's support
+    __shared__ bf16 tile[32][kBceCols + 2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int b0 = blockIdx.x * 32, q0 = blockIdx.y * kBceCols;
+    if (threadIdx.x < 32) {
+        unsigned long long h = 0;
+        if (b0 + lane < B)
+            for (int l = 0; l < s; ++l) {
+                const int c = sup[(size_t)(b0 + lane) * s + l] - q0;
+                if (c >= 0 && c < kBceCols) h |= 1ull << c;
+            }
+        hit[lane] = h;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = w * 4 + r, b = b0 + i;
+        const unsigned long long h = hit[i];
+        float acc = 0.f;
+#pragma unroll
+        for (int c = lane; c < kBceCols; c += 32) {
+            const int q = q0 + c;
+            if (b < B && q < Q) {
+                const float t = (float)((h >> c) & 1ull);
+                const float z = Z[(size_t)b * ldz + q];
+                acc += fmaxf(z, 0.f) - t * z + log1pf(expf(-fabsf(z)));
+                const float g = (1.f / (1.f + expf(-z)) - t) * scale;
+                const bf16 gb = __float2bfloat16_rn(g);
+                dZ[(size_t)b * lddz + q] = gb;
+                tile[i][c] = gb;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if (lane == 0 && b < B) lossp[(size_t)blockIdx.y * B + b] = acc;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 32 * kBceCols; t += 256) {
+        const int q = q0 + (t >> 5), b = b0 + (t & 31);
+        if (b < B && q < Q) dZT[(size_t)q * lddt + b] = tile[t & 31][t >> 5];
+    }
+}
+
+// The bias gradients out[r] = sum_c M[r, c] of two BF16 matrices with the same
+// columns (one warp per row, fixed order), and in the last block the mean loss.
+__global__ void __launch_bounds__(256)
+    row_sums_kernel(const bf16* __restrict__ M1, int R1, float* __restrict__ out1, const bf16* __restrict__ M2,
+                    int R2, float* __restrict__ out2, int ld, int C, const float* __restrict__ lossp, int nloss,
+                    float scale, float* __restrict__ loss) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float part[8];
+        if (!loss) return;
+        float acc = 0.f;
+#pragma unroll 8
+        for (int i = threadIdx.x; i < nloss; i += 256) acc += lossp[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+        if (lane == 0) part[w] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float t = 0.f;
+            for (int v = 0; v < 8; ++v) t += part[v];
+            loss[0] = t * scale;
+        }
+        return;
+    }
+    int r = blockIdx.x * 8 + w;
+    const bf16* M = M1;
+    float* out = out1;
+    if (r >= R1) {
+        r -= R1;
+        M = M2;
+        out = out2;
+        if (r >= R2) return;
+    }
     float acc = 0.f;
-    for (int c = lane; c < C; c += 32) acc += __bfloat162float(M[(size_t)r * ld + c]);
+    const bf16* row = M + (size_t)r * ld;
+#pragma unroll 16
+    for (int c = lane; c < C; c += 32) acc += __bfloat162float(row[c]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
     if (lane == 0) out[r] = acc;
 }
 
-__global__ void sum_kernel(const float* __restrict__ x, int n, float scale, float* __restrict__ out) {
-    float acc = 0.f;
-    for (int i = threadIdx.x; i < n; i += 32) acc += x[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    if (threadIdx.x == 0) out[0] = acc * scale;
-}
+struct AdamJob {
+    float *p, *m, *v;
+    const float* g;
+    int rows, cols, blocks;  // 32 x 32 blocks
+    bf16 *pb, *pbT;          // BF16 copies (row-major, transposed) or null
+};
+struct AdamJobs {
+    AdamJob job[4];
+};
 
-// Adam on FP32 master weights; refresh the BF16 copy (and its transpose)
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, int rows, int cols,
-                            float lr, float beta1, float beta2, float eps, float bc1, float bc2,
-                            bf16* __restrict__ pb, bf16* __restrict__ pbT) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * cols) return;
-    const float gi = g[i];
-    const float mi = beta1 * m[i] + (1.f - beta1) * gi;
-    const float vi = beta2 * v[i] + (1.f - beta2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pn = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-    p[i] = pn;
-    const bf16 b = __float2bfloat16_rn(pn);
-    if (pb) pb[i] = b;
-    if (pbT) pbT[(size_t)(i % cols) * rows + i / cols] = b;
+// Adam on FP32 master weights for the four parameter arrays in one launch;
+// refreshes the BF16 copies (the transposed one through shared memory)
+__global__ void __launch_bounds__(256)
+    adam_kernel(const __grid_constant__ AdamJobs jobs, float lr, float beta1, float beta2, float eps, float bc1,
+                float bc2) {
+    __shared__ bf16 tile[32][34];
+    int blk = blockIdx.x, k = 0;
+    while (k < 3 && blk >= jobs.job[k].blocks) blk -= jobs.job[k++].blocks;
+    const AdamJob& q = jobs.job[k];
+    const int cb = (q.cols + 31) / 32, r0 = blk / cb * 32, c0 = blk % cb * 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = r0 + w + 8 * u, c = c0 + lane;
+        if (r >= q.rows || c >= q.cols) continue;
+        const size_t i = (size_t)r * q.cols + c;
+        const float gi = q.g[i];
+        const float mi = beta1 * q.m[i] + (1.f - beta1) * gi;
+        const float vi = beta2 * q.v[i] + (1.f - beta2) * gi * gi;
+        q.m[i] = mi;
+        q.v[i] = vi;
+        const float pn = q.p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        q.p[i] = pn;
+        const bf16 b = __float2bfloat16_rn(pn);
+        if (q.pb) q.pb[i] = b;
+        tile[w + 8 * u][lane] = b;
+    }
+    if (!q.pbT) return;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int c = c0 + w + 8 * u, r = r0 + lane;
+        if (c < q.cols && r < q.rows) q.pbT[(size_t)c * q.rows + r] = tile[lane][w + 8 * u];
+    }
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ p, int rows, int cols,
@@ -537,6 +643,14 @@ T* carve(char*& p, size_t n) {
     return r;
 }
 
+// The context's second stream and its events, made on first use.
+int side_stream(sdl_ctx* c) {
+    if (!c->side && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) return SDL_ERR_CUDA;
+    for (cudaEvent_t& e : c->side_ev)
+        if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return SDL_ERR_CUDA;
+    return SDL_OK;
+}
+
 int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
 }  // namespace
@@ -561,7 +675,8 @@ int sdl_mlp_create(sdl_ctx* c, int p1, int p2, int n1, int n2, int hidden, int m
     m->Bmax = max_batch;
     const size_t H = m->H, Kp = m->Kp, Q = m->Q, B = m->Bmax;
     const size_t nf = 4 * (H * Kp + H + Q * H + Q) + 1024;     // params, m, v, grads
-    const size_t bytes = (nf * 4 + (H * Kp + 2 * Q * H) * 2 + (2 * B * Kp + 2 * B * H + 2 * B * Q + B * H) * 2 +
+    const size_t nloss = B * ((Q + kBceCols - 1) / kBceCols);
+    const size_t bytes = (nf * 4 + nloss * 4 + (H * Kp + 2 * Q * H) * 2 + (2 * B * Kp + 2 * B * H + 2 * B * Q + B * H) * 2 +
                           (B * H + B * Q + B) * 4) + 64 * 256;
     if (cudaMalloc(&m->mem, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -583,7 +698,7 @@ int sdl_mlp_create(sdl_ctx* c, int p1, int p2, int n1, int n2, int hidden, int m
     m->Hb = carve<bf16>(p, B * H); m->HTb = carve<bf16>(p, H * B);
     m->dZb = carve<bf16>(p, B * Q); m->dZTb = carve<bf16>(p, Q * B);
     m->dPreTb = carve<bf16>(p, H * B);
-    m->pre = carve<float>(p, B * H); m->Z = carve<float>(p, B * Q); m->lossp = carve<float>(p, B);
+    m->pre = carve<float>(p, B * H); m->Z = carve<float>(p, B * Q); m->lossp = carve<float>(p, nloss);
     if ((size_t)(p - m->mem) > bytes) {
         cudaFree(m->mem);
         delete m;
@@ -652,46 +767,54 @@ static int mlp_batch(sdl_mlp* m, const float* Y, const int32_t* support, int s, 
                      float lr, float* loss_out, cudaStream_t st) {
     sdl_ctx* c = m->ctx;
     const int H = m->H, Kp = m->Kp, Q = m->Q, Bm = m->Bmax;
-    int rc;
+    int rc = side_stream(c);
+    if (rc) return rc;
     {
         Trace tr(c, kMlp, st);
-        prep_input_kernel<<<blocks_for((long long)B * 32, 256), 256, 0, st>>>(Y, B, m->P, Kp, m->Xb,
-                                                                             Kp, m->XTb, Bm);
+        prep_batch_kernel<<<blocks_for(B, 32), 256, 0, st>>>(Y, B, m->P, Kp, m->Xb, m->XTb, Bm);
         if ((rc = tc_gemm(m->Xb, Kp, m->W1b, Kp, B, H, Kp, 1.f, m->b1, 1, nullptr, 0, 0, m->Hb, H,
                           m->HTb, Bm, m->pre, H, c->err, st)))
             return rc;
         if ((rc = tc_gemm(m->Hb, H, m->W2b, H, B, Q, H, 1.f, m->b2, 0, m->Z, Q, 0, nullptr, 0,
                           nullptr, 0, nullptr, 0, c->err, st)))
             return rc;
-        bce_kernel<<<B, 256, 0, st>>>(m->Z, Q, support, s, Q, 1.f / (float)B, m->dZb, Q, m->dZTb,
-                                      Bm, m->lossp);
-        // dW2 = dZ^T H ; dPre = (dZ W2) * GELU'(pre) ; dW1 = dPre^T X
-        if ((rc = tc_gemm(m->dZTb, Bm, m->HTb, Bm, Q, H, B, 1.f, nullptr, 0, m->gW2, H, 0, nullptr,
-                          0, nullptr, 0, nullptr, 0, c->err, st)))
-            return rc;
-        if ((rc = tc_gemm(m->dZb, Q, m->W2Tb, Q, B, H, Q, 1.f, nullptr, 2, nullptr, 0, 0, nullptr,
-                          0, m->dPreTb, Bm, nullptr, 0, c->err, st, m->pre, H)))
-            return rc;
-        if ((rc = tc_gemm(m->dPreTb, Bm, m->XTb, Bm, H, Kp, B, 1.f, nullptr, 0, m->gW1, Kp, 0,
-                          nullptr, 0, nullptr, 0, nullptr, 0, c->err, st)))
-            return rc;
-        rowsum_kernel<<<blocks_for((long long)Q * 32, 256), 256, 0, st>>>(m->dZTb, Bm, Q, B, m->gb2);
-        rowsum_kernel<<<blocks_for((long long)H * 32, 256), 256, 0, st>>>(m->dPreTb, Bm, H, B, m->gb1);
-        if (loss_out) sum_kernel<<<1, 32, 0, st>>>(m->lossp, B, 1.f / (float)B, loss_out);
+        const dim3 bce(blocks_for(B, 32), blocks_for(Q, kBceCols));
+        bce_kernel<<<bce, 256, 0, st>>>(m->Z, Q, support, s, B, Q, 1.f / (float)B, m->dZb, Q, m->dZTb, Bm, m->lossp);
+        // dW2 = dZ^T H ; dPre = (dZ W2) * GELU'(pre) ; dW1 = dPre^T X.  dW2 (few
+        // tiles, a long K) runs beside dPre, which leaves it SMs, and the bias
+        // gradients beside dW1; everything joins `st` before the update.
+        auto step = [&](cudaError_t e) { return e == cudaSuccess; };
+        if (!step(cudaEventRecord(c->side_ev[0], st)) || !step(cudaStreamWaitEvent(c->side, c->side_ev[0], 0))) return SDL_ERR_CUDA;
+        rc = tc_gemm(m->dZTb, Bm, m->HTb, Bm, Q, H, B, 1.f, nullptr, 0, m->gW2, H, 0, nullptr, 0, nullptr, 0,
+                     nullptr, 0, c->err, c->side);
+        if (!rc)
+            rc = tc_gemm(m->dZb, Q, m->W2Tb, Q, B, H, Q, 1.f, nullptr, 2, nullptr, 0, 0, nullptr, 0, m->dPreTb, Bm,
+                         nullptr, 0, c->err, st, m->pre, H);
+        if (!step(cudaEventRecord(c->side_ev[1], st)) || !step(cudaStreamWaitEvent(c->side, c->side_ev[1], 0))) rc = SDL_ERR_CUDA;
+        if (!rc)
+            row_sums_kernel<<<blocks_for(Q + H, 8) + 1, 256, 0, c->side>>>(m->dZTb, Q, m->gb2, m->dPreTb, H, m->gb1, Bm,
+                                                                          B, m->lossp, B * (int)bce.y, 1.f / (float)B,
+                                                                          loss_out);
+        if (!rc)
+            rc = tc_gemm(m->dPreTb, Bm, m->XTb, Bm, H, Kp, B, 1.f, nullptr, 0, m->gW1, Kp, 0, nullptr, 0, nullptr, 0,
+                         nullptr, 0, c->err, st);
+        // the side stream joins whatever happened above
+        if (!step(cudaEventRecord(c->side_ev[2], c->side)) || !step(cudaStreamWaitEvent(st, c->side_ev[2], 0))) rc = SDL_ERR_CUDA;
+        if (rc) return rc;
     }
     if (update) {
         Trace tr(c, kAdam, st);
         m->step += 1;
         const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
         const float bc1 = 1.f - powf(b1, (float)m->step), bc2 = 1.f - powf(b2, (float)m->step);
-        adam_kernel<<<blocks_for((long long)H * Kp, 256), 256, 0, st>>>(
-            m->W1, m->gW1, m->mW1, m->vW1, H, Kp, lr, b1, b2, eps, bc1, bc2, m->W1b, nullptr);
-        adam_kernel<<<blocks_for(H, 256), 256, 0, st>>>(m->b1, m->gb1, m->mb1, m->vb1, 1, H, lr, b1,
-                                                         b2, eps, bc1, bc2, nullptr, nullptr);
-        adam_kernel<<<blocks_for((long long)Q * H, 256), 256, 0, st>>>(
-            m->W2, m->gW2, m->mW2, m->vW2, Q, H, lr, b1, b2, eps, bc1, bc2, m->W2b, m->W2Tb);
-        adam_kernel<<<blocks_for(Q, 256), 256, 0, st>>>(m->b2, m->gb2, m->mb2, m->vb2, 1, Q, lr, b1,
-                                                         b2, eps, bc1, bc2, nullptr, nullptr);
+        auto blocks = [](int rows, int cols) { return blocks_for(rows, 32) * blocks_for(cols, 32); };
+        const AdamJobs jobs = {{{m->W2, m->mW2, m->vW2, m->gW2, Q, H, blocks(Q, H), m->W2b, m->W2Tb},
+                                {m->W1, m->mW1, m->vW1, m->gW1, H, Kp, blocks(H, Kp), m->W1b, nullptr},
+                                {m->b1, m->mb1, m->vb1, m->gb1, 1, H, blocks(1, H), nullptr, nullptr},
+                                {m->b2, m->mb2, m->vb2, m->gb2, 1, Q, blocks(1, Q), nullptr, nullptr}}};
+        int total = 0;
+        for (const AdamJob& j : jobs.job) total += j.blocks;
+        adam_kernel<<<total, 256, 0, st>>>(jobs, lr, b1, b2, eps, bc1, bc2);
     }
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
 }

@@ -3,20 +3,20 @@
 // FP32 accumulation; t runs over 1 to 3 operand pairs summed into one
 // accumulator (the split-precision products of the correlation path).
 //
-// Blackwell path, persistent and warp-specialised (one CTA per SM, 192
-// threads):
+// Blackwell path, persistent and warp-specialised (one CTA per SM, 6 or 18
+// warps):
 //   warp 0  TMA producer: operand tiles by cp.async.bulk.tensor (128-byte
-//           swizzle) into a shared-memory ring of 6 stages (4 at BN = 256)
-//           guarded by mbarriers;
-//   warp 1  MMA issuer: one thread issues tcgen05.mma (128 x BN x 16, BN =
+//           swizzle) into a shared-memory ring of 3 to 9 stages guarded by
+//           mbarriers;
+//   warp 1  MMA issuer: one elected lane issues tcgen05.mma (128 x BN x 16, BN =
 //           256 when N is a multiple of 256 and the 256-wide tiles fill the
-//           SMs, else 128) into one of two
+//           SMs, 32 for a few tiles with a long K, else 128) into one of two
 //           BN-column FP32 accumulators in tensor memory (all 512 columns at
 //           BN = 256: the wider tile halves the operand bytes each FLOP needs
 //           from L2);
 //           tcgen05.commit releases ring stages and hands a finished
 //           accumulator to the epilogue;
-//   warps 2-5  epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
+//   warps 2-5 (or 2-17)  epilogue: tcgen05.ld of the accumulator (warp w reads TMEM
 //           lanes 32 (w % 4) .. +31 = output rows), bias / GELU / GELU'
 //           and the outputs.  The FP32 and BF16 row-major outputs leave by
 //           TMA: each warp writes its 32 x 32 block into one of two swizzled
@@ -24,8 +24,12 @@
 //           tensor reduce-add when accumulating), so the stores neither cost
 //           the warp an instruction per row nor wait on it.  The other
 //           outputs (transposed BF16, pre-activation, the GELU' product) go
-//           through a per-warp 32 x 33 shared-memory transpose as coalesced
-//           128-byte row segments.
+//           through a per-warp 32 x 32 shared-memory transpose (columns XORed
+//           with the row) as coalesced 128-byte row segments.
+// Measured (us): 32768 x 512 x 64 with GELU, 4 -> 16 epilogue warps 87 -> 35;
+// 4096 x 512 x 576 with GELU' and a transposed output 90 -> 20; 576 x 512 x 4096
+// (20 tiles) 32 -> 25 with the loops of warps 0 and 1 free of divisions and converged;
+// 512 x 144 x 4096 32 -> 20 with those and 128 x 32 tiles.
 // With two accumulators the epilogue of one tile overlaps the main loop of
 // the next.  Tiles are visited m-block-major, so CTAs running at the same
 // time share A rows and the whole of B in L2.
@@ -56,7 +60,7 @@ __host__ __device__ constexpr int slots_for(int EW) { return EW == 4 ? 2 : 1; }
 __host__ __device__ constexpr int epi_bytes(int EW) { return EW * slots_for(EW) * kSlot; }
 // shared-memory ring depth: as many stages as fit beside the epilogue's staging
 __host__ __device__ constexpr int stages_for(int BN, int EW) {
-    return EW == 4 ? (BN == 256 ? 4 : 6) : (BN == 256 ? 3 : 5);
+    return BN == 32 ? 9 : EW == 4 ? (BN == 256 ? 4 : 6) : (BN == 256 ? 3 : 5);
 }
 constexpr int threads_for(int EW) { return 64 + 32 * EW; }
 constexpr int TILE_A = BM * BK * 2;           // bytes
@@ -113,6 +117,7 @@ __device__ __forceinline__ bool mbar_test(uint32_t a, uint32_t parity) {
 // bounded wait; false on timeout or when *fail is set by another role
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* fail) {
     const uint32_t a = saddr(b);
+    if (mbar_test(a, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
         if (mbar_test(a, parity)) return true;
@@ -161,6 +166,13 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// one lane of a converged warp (the branch on it keeps the warp's loop variables
+// in uniform registers, which the tensor instructions take their operands from)
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
 }
 // K-major operand tile, 128-byte swizzle: rows of 128 B, 8-row groups 1024 B apart
 __device__ __forceinline__ uint64_t smem_desc(const void* p) {
@@ -268,56 +280,68 @@ __global__ void __launch_bounds__(threads_for(EW), 1)
     const uint32_t tmem = *tslot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer
-            long long g = 0;   // k-blocks issued so far (ring position)
-            for (long long t = blockIdx.x; t < tiles && !*fail; t += gridDim.x) {
-                const int m0 = (int)(t / nt) * BM, n0 = (int)(t % nt) * BN;
-                for (int ks = 0; ks < ksteps; ++ks) {
-                    const int s = (int)(g % STAGES);
-                    const long long use = g / STAGES;
-                    if (use > 0 && !mbar_wait(&empty[s], (uint32_t)((use - 1) & 1), fail)) break;
-                    const int term = ks / nk, kb = ks - term * nk;
-                    mbar_arrive_tx(&full[s], TILE_A + TILE_B);
-                    tma_load_2d(sA + s * TILE_A, &maps.a[term], kb * BK, m0, &full[s]);
-                    tma_load_2d(sB + s * TILE_B, &maps.b[term], kb * BK, n0, &full[s]);
-                    ++g;
+        // ---- TMA producer.  The warp loops converged and one elected lane
+        // issues; stage and phase are counted along, without divisions: this
+        // loop's latency is the pace of a k-block whenever the MMAs are short
+        long long issued = 0;   // k-blocks issued so far
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;   // the same in every lane: the loops end together
+        for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+            const int m0 = (int)(t / nt) * BM, n0 = (int)(t % nt) * BN;
+            for (int term = 0; term < terms && ok; ++term) {
+                for (int kb = 0; kb < nk; ++kb) {
+                    // on a fresh barrier the wait for the other parity passes at once
+                    ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], ph ^ 1u, fail));
+                    if (!ok) break;
+                    if (elect_one()) {
+                        mbar_arrive_tx(&full[s], TILE_A + TILE_B);
+                        tma_load_2d(sA + s * TILE_A, &maps.a[term], kb * BK, m0, &full[s]);
+                        tma_load_2d(sB + s * TILE_B, &maps.b[term], kb * BK, n0, &full[s]);
+                    }
+                    ++issued;
+                    if (++s == STAGES) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
             }
-            if (*fail) {
-                // let the copies in flight land before shared memory is released
-                for (long long h = g - STAGES > 0 ? g - STAGES : 0; h < g; ++h)
-                    mbar_drain(&full[h % STAGES], (uint32_t)((h / STAGES) & 1));
-            }
+        }
+        if (lane == 0 && *fail) {
+            // let the copies in flight land before shared memory is released
+            for (long long h = issued - STAGES > 0 ? issued - STAGES : 0; h < issued; ++h)
+                mbar_drain(&full[h % STAGES], (uint32_t)((h / STAGES) & 1));
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---- MMA issuer
-            const uint32_t idesc = instr_desc<BN>();
-            long long g = 0;
-            int i = 0;   // local tile counter
-            for (long long t = blockIdx.x; t < tiles && !*fail; t += gridDim.x, ++i) {
-                const int b = i & 1, use_b = i >> 1;
-                if (use_b > 0 && !mbar_wait(&acc_empty[b], (uint32_t)((use_b - 1) & 1), fail)) break;
+        // ---- MMA issuer (converged, one elected lane)
+        const uint32_t idesc = instr_desc<BN>();
+        const uint64_t ad0 = smem_desc(sA), bd0 = smem_desc(sB);   // addresses count in 16 bytes
+        int s = 0;
+        uint32_t ph = 0;
+        int i = 0;   // local tile counter
+        bool ok = true;   // the same in every lane
+        for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
+            const int b = i & 1, use_b = i >> 1;
+            if (use_b > 0) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[b], (uint32_t)((use_b - 1) & 1), fail));
+                if (!ok) break;
+            }
+            tc_fence_after();
+            const uint32_t acc_addr = tmem + (uint32_t)(b * BN);
+            for (int ks = 0; ks < ksteps; ++ks) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, fail));
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t acc_addr = tmem + (uint32_t)(b * BN);
-                bool ok = true;
-                for (int ks = 0; ks < ksteps; ++ks, ++g) {
-                    const int s = (int)(g % STAGES);
-                    if (!mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1), fail)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
+                const uint64_t as = ad0 + (uint32_t)(s * (TILE_A >> 4)), bs = bd0 + (uint32_t)(s * (TILE_B >> 4));
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                        const uint64_t ad = smem_desc(sA + s * TILE_A + kk * UMMA_K * 2);
-                        const uint64_t bd = smem_desc(sB + s * TILE_B + kk * UMMA_K * 2);
+                        const uint64_t ad = as + kk * (UMMA_K * 2 >> 4);
+                        const uint64_t bd = bs + kk * (UMMA_K * 2 >> 4);
                         const uint32_t accum = (ks > 0 || kk > 0) ? 1u : 0u;
                         asm volatile(
                             "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                                acc_addr),
+                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc_addr),
                             "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
                             : "memory");
                     }
@@ -325,20 +349,25 @@ __global__ void __launch_bounds__(threads_for(EW), 1)
                         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
                         "[%0];" ::"r"(saddr(&empty[s]))
                         : "memory");
+                    if (ks + 1 == ksteps)
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                saddr(&acc_full[b]))
+                            : "memory");
                 }
-                if (!ok) break;
-                asm volatile(
-                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                        saddr(&acc_full[b]))
-                    : "memory");
+                __syncwarp();
+                if (++s == STAGES) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
         }
     } else {
         // ---- epilogue warps: 4 cover the 128 rows; with 16, four groups of 4
         // take every fourth 32-column block (the activations' latency, and the
         // row-by-row outputs, need more warps than the TMEM quarters)
-        constexpr int CB = EW == 4 ? 64 : 32;      // columns per TMEM load
-        constexpr int CSTEP = EW == 4 ? 64 : 128;
+        constexpr int CB = EW == 4 && BN >= 64 ? 64 : 32;      // columns per TMEM load
+        constexpr int CSTEP = EW == 4 ? CB : 128;
         const int quarter = warp & 3;              // TMEM lanes this warp may access
         const int cfirst = EW == 4 ? 0 : ((warp - 2) >> 2) * 32;
         uint8_t* slots = epi_area + (warp - 2) * slots_for(EW) * kSlot;
@@ -360,7 +389,7 @@ __global__ void __launch_bounds__(threads_for(EW), 1)
             for (int cb = cfirst; cb < BN; cb += CSTEP) {
                 uint32_t v[CB];
                 const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * BN + cb);
-                if constexpr (EW == 4) tmem_ld64(ta, v);
+                if constexpr (CB == 64) tmem_ld64(ta, v);
                 else tmem_ld32(ta, v);
                 if (cb + CSTEP >= BN) {
                     // this warp has read its part of the accumulator: hand it back
@@ -564,7 +593,7 @@ constexpr size_t smem_bytes(int BN, int EW) {
     return 1024 + (size_t)stages_for(BN, EW) * (TILE_A + BN * BK * 2) + epi_bytes(EW) + 256;
 }
 static_assert(smem_bytes(256, 4) <= 232448 && smem_bytes(128, 4) <= 232448 && smem_bytes(256, 16) <= 232448 &&
-                  smem_bytes(128, 16) <= 232448,
+                  smem_bytes(128, 16) <= 232448 && smem_bytes(32, 4) <= 232448,
               "shared memory per CTA");
 
 // output map: rows x cols matrix of 4-byte (f32) or 2-byte (bf16) elements,
@@ -623,6 +652,8 @@ int cached_map(CUtensorMap* out, const MapKey& k, Encode encode) {
 
 // contraction length up to which the 16-warp epilogue is taken
 constexpr long long kShortK = 1024;
+// and from which a GEMM with few output tiles takes 128 x 32 ones
+constexpr int kThinK = 1024;
 
 int sm_count() {
     static int count[64] = {0};
@@ -651,7 +682,12 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
     // to fill the SMs, else 128 x 128 (a small output with a long K, such as a
     // weight gradient, keeps twice the CTAs busy)
     const long long mb = (M + BM - 1) / BM;
-    const int bn = (N % 256 == 0 && mb * (N / 256) >= sm_count()) ? 256 : 128;
+    // and 128 x 32 tiles for a long K with few 128 x 128 ones (the weight gradient
+    // of 512 x 144 has 8): more CTAs, and a k-block is 20 KB instead of 32.  Cutting K
+    // instead would fill the SMs better but change the order of the sums.
+    const bool thin = terms == 1 && act == 0 && C && !Cb && !Ct && !pre && K >= kThinK &&
+                      mb * ((N + 127) / 128) <= sm_count() / 16;
+    const int bn = thin ? 32 : (N % 256 == 0 && mb * (N / 256) >= sm_count()) ? 256 : 128;
     Maps maps;
     std::memset(&maps, 0, sizeof(maps));
     int rc;
@@ -706,10 +742,10 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
     auto launch = [&](auto kern, int BN, int EW) -> int {
         const size_t bytes = smem_bytes(BN, EW);
         // the shared-memory opt-in is set once per device and variant
-        static bool attr_set[4][64] = {};
+        static bool attr_set[5][64] = {};
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-        bool& done = attr_set[(BN == 256) + 2 * (EW == 16)][dev & 63];
+        bool& done = attr_set[BN == 32 ? 4 : (BN == 256) + 2 * (EW == 16)][dev & 63];
         if (!done || dev >= 64) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
                 cudaSuccess)
@@ -723,6 +759,7 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
     };
     // 16 epilogue warps where a tile's epilogue outlasts its main loop: an
     // activation, an output that leaves row by row, or a short contraction
+    if (bn == 32) return launch(tc_gemm_kernel<32, 4>, 32, 4);
     const bool wide = act != 0 || !tma || (long long)K * terms <= kShortK;
     if (bn == 256) return wide ? launch(tc_gemm_kernel<256, 16>, 256, 16) : launch(tc_gemm_kernel<256, 4>, 256, 4);
     return wide ? launch(tc_gemm_kernel<128, 16>, 128, 16) : launch(tc_gemm_kernel<128, 4>, 128, 4);
