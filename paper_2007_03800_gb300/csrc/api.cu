@@ -129,6 +129,42 @@ int prepare_tc_pass(sdl_ctx* c, PassArgs& a, bool fill_y, cudaStream_t st) {
     return SDL_OK;
 }
 
+// Partial-sum slots of a learning pass that runs as the lane-group coder followed
+// by the ordered sums (compiled shapes, fixed sparsity, aligned signals, no tiling
+// pinned), or 0: the fused kernels.  Two launches instead of one pay off from
+// about 2.1M correlations on: an iteration (us, split / fused) at 8x8 x 4000 78 / 75,
+// x 16000 95 / 99, x 64000 169 / 202; at 12x12 x 2000 94 / 88, x 4000 97 / 100,
+// x 64000 332 / 421; at 16x16 x 1000 110 / 101, x 4000 130 / 137, x 64000 688 / 987.
+constexpr long long kSplitPairs = 2100000;
+int split_pass_slots(const PassArgs& a, bool tc, int num_sms) {
+    if (a.N * a.n1 * a.n2 < kSplitPairs) return 0;
+    if (tc || a.tiling > 0 || a.eps2 > 0.f || a.N < 1 || (reinterpret_cast<uintptr_t>(a.Y) & 15u)) return 0;
+    return std::max(0, ordered_slots(a, num_sms));
+}
+
+// One such pass: codes to the caller's arrays (both passes: the second rewrites
+// them), residual energies to the slots of part_d, sums to those of part_f.
+int split_pass(sdl_ctx* c, const PassArgs& a0, int side, int slots, int32_t* support, float* coef, int32_t* nnz,
+               cudaStream_t st) {
+    PassArgs a = a0;
+    a.support = support;
+    a.coef = coef;
+    a.nnz = nnz;
+    a.esum = c->part_d;
+    a.esum_slots = slots;
+    int rc;
+    {
+        Trace tr(c, side == kSideD1 ? kCodeD1 : kCodeD2, st);
+        rc = launch_code_group_fixed(a, side == kSideD2, st, c->num_sms, slots);
+    }
+    if (rc != SDL_OK) return rc;
+    a.in_support = support;
+    a.in_coef = coef;
+    Trace tr(c, side == kSideD1 ? kAccD1 : kAccD2, st);
+    rc = launch_accumulate_ordered(a, side, st, c->num_sms);
+    return rc == SDL_OK ? slots : rc;
+}
+
 // reduce -> solve for one dictionary side, using the partial sums in slots.
 int finish_update(sdl_ctx* c, int slots, int side, float* D, int p1, int p2, int64_t N, int n1,
                   int n2, double* objective_out, double* rmse_out, cudaStream_t st,
@@ -349,30 +385,32 @@ int sdl_iterate(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, float* D1
     cudaStream_t st = (cudaStream_t)stream;
     const float eps2 = eps > 0.f ? eps * eps : 0.f;
 
-    // steps 1-2: code with (D1, D2) accumulating P, B1; solve for D1
-    grams(c, D1, p1, n1, D2, p2, n2, st);
     PassArgs a = base_args(c, Y, p1, p2, N, D1, n1, D2, n2, s);
     a.eps2 = eps2;
     const bool tc = (c->prec & SDL_PREC_BF16_CORR) != 0;
+    const int ordered = split_pass_slots(a, tc, c->num_sms);
+    // one coding pass with its sums: the number of partial-sum slots
+    auto code_side = [&](int side) -> int {
+        if (ordered > 0) return split_pass(c, a, side, ordered, support, coef, nnz, st);
+        Trace tr(c, side == kSideD1 ? kCodeD1 : kCodeD2, st);
+        return launch_code_pass(a, side, st, c->num_sms);
+    };
+
+    // steps 1-2: code with (D1, D2) accumulating P, B1; solve for D1
+    if (ordered <= 0) grams(c, D1, p1, n1, D2, p2, n2, st);
     if (tc && (rc = prepare_tc_pass(c, a, true, st)) != SDL_OK) return rc;
-    int slots;
-    {
-        Trace tr(c, kCodeD1, st);
-        slots = launch_code_pass(a, kSideD1, st, c->num_sms);
-    }
+    int slots = code_side(kSideD1);
     if (slots < 0) return slots;
     // the solve also refreshes G1 for the new D1
-    rc = finish_update(c, slots, kSideD1, D1, p1, p2, N, n1, n2, nullptr, rmse_out, st, c->G1);
+    rc = finish_update(c, slots, kSideD1, D1, p1, p2, N, n1, n2, nullptr, rmse_out, st,
+                       ordered > 0 ? nullptr : c->G1);
     if (rc != SDL_OK) return rc;
     // steps 3-4: code with the new D1 accumulating M, B2; solve for D2
     a.support = support;
     a.coef = coef;
     a.nnz = nnz;
     if (tc && (rc = prepare_tc_pass(c, a, false, st)) != SDL_OK) return rc;   // new D1
-    {
-        Trace tr(c, kCodeD2, st);
-        slots = launch_code_pass(a, kSideD2, st, c->num_sms);
-    }
+    slots = code_side(kSideD2);
     if (slots < 0) return slots;
     rc = finish_update(c, slots, kSideD2, D2, p1, p2, N, n1, n2, nullptr,
                        rmse_out ? rmse_out + 1 : nullptr, st);

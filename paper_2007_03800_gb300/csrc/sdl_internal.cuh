@@ -121,6 +121,11 @@ int multi_ctas_per_sm(size_t smem, int side);
 // dictionaries only if wanted.  Returns the slots written, or
 // SDL_ERR_UNSUPPORTED.  Needs no Gram matrices.
 int launch_accumulate_lanes(const PassArgs& a, int side, bool want_energy, cudaStream_t st, int num_sms);
+// accum_ordered.cu: the sums of a fused coding pass at a compiled shape from codes
+// already written (a.in_support, a.in_coef; Y 16-byte aligned), in the fused
+// pass's order, to ordered_slots(a) slots (a negative error for other shapes)
+int ordered_slots(const PassArgs& a, int num_sms);
+int launch_accumulate_ordered(const PassArgs& a, int side, cudaStream_t st, int num_sms);
 bool code_shape_supported(int p1, int p2, int n1, int n2, int s);
 // Upper bound of the partial-sum slots any pass may use for these sizes.
 int max_partial_slots(int num_sms);
