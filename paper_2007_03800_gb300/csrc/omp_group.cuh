@@ -43,9 +43,15 @@ __host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
 // kFastNum: 1/sqrt by rsqrtf and back substitution in increasing row order
 // (the compiled tilings' forms); else 1/sqrtf and decreasing order (the
 // generic kernel's).  kW: C0 = (D1^T Y) D2 rather than D1^T (Y D2).
+// ORTHO_: 0, or the orthonormal variant (n = p; a pick's coefficient is its
+// correlation and leaves the others alone) with ||Y||^2 in that many chains.
 template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,
-          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0>
+          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0>
 struct Cfg {
+    static constexpr bool kOrtho = ORTHO_ > 0;
+    static constexpr int CHAINS = ORTHO_ > 0 ? ORTHO_ : 32;   // of ||Y||^2
+    static constexpr int CPL = CHAINS / GL_;                  // per lane
+    static_assert(CPL == 1 || CPL == 2 || CPL == 4, "chains");
     static constexpr int GL = GL_, LI = LI_, LJ = GL_ / LI_, RI = RI_, RJ = RJ_;
     static constexpr int WARPS = WARPS_, MINB = MINB_;
     static constexpr bool kFast = FAST_, kW = W_;
@@ -64,7 +70,7 @@ struct Cfg {
     static constexpr int WB = P2 ? (P2 / LJ) : 4;
     static constexpr int SMAX = S ? S : 8;              // unrolled Cholesky rows
     static_assert(N1P * LD1 <= 65536 && N2P * LD2 <= 65536, "16-bit row offsets");
-    static_assert(E % 4 == 0 && RI % 2 == 0, "row pairs, 16-byte block stores");
+    static_assert(E % 2 == 0 && RI % 2 == 0, "row pairs, 16-byte block stores");
     static_assert((LI & (LI - 1)) == 0 && LI * LJ == GL, "lane grid");
     static_assert(!kW || P2 > 0, "the W stage is compiled for fixed sizes");
     static_assert(P1 == 0 || (P1 % LI == 0 && ZA % 2 == 0 && P1 % 4 == 0 && P2 % LJ == 0), "fixed sizes");
@@ -86,8 +92,8 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     L.d1 = 0;
     L.d2 = L.d1 + p1 * C::LD1;
     L.g1 = L.d2 + p2 * C::LD2;
-    L.g2 = L.g1 + C::N1P * C::LD1;
-    L.warp0 = L.g2 + C::N2P * C::LD2;
+    L.g2 = L.g1 + (C::kOrtho ? 0 : C::N1P * C::LD1);
+    L.warp0 = L.g2 + (C::kOrtho ? 0 : C::N2P * C::LD2);
     L.y = 0;
     L.c0 = L.y + L.p1s * p2;
     const int z = C::kW ? p2 * C::LD1 : up4(p1) * C::LD2;   // Z or W shares the C0 blocks' place
@@ -95,9 +101,9 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     L.col = L.c0 + (z > c ? z : c);
     L.rec = L.col + C::CS;
     L.lf = L.rec + up4(2 * s);
-    L.iv = L.lf + up4(s * (s - 1) / 2);
-    L.yv = L.iv + up4(s);
-    int st = L.yv + up4(s);
+    L.iv = L.lf + (C::kOrtho ? 0 : up4(s * (s - 1) / 2));
+    L.yv = L.iv + (C::kOrtho ? 0 : up4(s));
+    int st = L.yv + (C::kOrtho ? 0 : up4(s));
     // neighbouring signals of a warp start 8 banks apart where they read the
     // same offsets together
     while (st % 32 != 8 && st % 32 != 24) st += 4;
@@ -375,6 +381,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         reinterpret_cast<Rec*>(wb + g * L.sig_stride + L.rec)[e - g * s] = Rec{0.f, 0u};
     }
     __syncthreads();
+    if constexpr (!C::kOrtho) {
     for (int e = threadIdx.x; e < C::N1P * LD1; e += blockDim.x) {
         const int i = e / LD1, pos = e % LD1;
         const float* di = D1s + (i / RI) * RIP + i % RI;
@@ -392,6 +399,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         G2s[e] = g;
     }
     __syncthreads();
+    }
 
     const long long count = a.idx ? (long long)*a.idx_count : a.N;
     const long long units = (count + SPW - 1) / SPW;
@@ -429,15 +437,15 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         const long long ko = !act ? 0 : (a.idx && !a.idx_compact) ? (long long)a.idx[pos] : pos;
         cp_wait();
         __syncwarp();
-        // ---- ||Y||^2: the 32 strided partial sums of the one-warp coders (this
-        // lane takes 32 / GL of them) and their combining tree
-        float part[SPW];
+        // ---- ||Y||^2: the strided partial sums of the one-signal-per-warp (or half
+        // warp) coders (this lane takes CPL of them) and their combining tree
+        float part[C::CPL];
 #pragma unroll
-        for (int v = 0; v < SPW; ++v) part[v] = 0.f;
+        for (int v = 0; v < C::CPL; ++v) part[v] = 0.f;
         if (act) {
 #pragma unroll
-            for (int v = 0; v < SPW; ++v)
-                for (int e = gl + GL * v; e < pp; e += 32) {
+            for (int v = 0; v < C::CPL; ++v)
+                for (int e = gl + GL * v; e < pp; e += C::CHAINS) {
                     int at = e;
                     if (!(C::P1 ? true : p1 % 4 == 0)) {
                         const int b = (int)((unsigned)e * inv_p1 >> 16);
@@ -447,8 +455,9 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 }
         }
         float ss;
-        if constexpr (SPW == 4) ss = (part[0] + part[2]) + (part[1] + part[3]);
-        else ss = part[0] + part[1];
+        if constexpr (C::CPL == 4) ss = (part[0] + part[2]) + (part[1] + part[3]);
+        else if constexpr (C::CPL == 2) ss = part[0] + part[1];
+        else ss = part[0];
 #pragma unroll
         for (int o = GL / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
         const bool finite = act && isfinite(ss);
@@ -547,7 +556,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             if (t > 0) {
                 ld<E>(sc, myc0);
 #pragma unroll 1
-                for (int l = 0; l < t; ++l) {
+                for (int l = 0; l < (C::kOrtho ? 0 : t); ++l) {
                     const Rec r = rec[l];
                     float x[RI], v[RJ];
                     ld<RI>(x, G1s + r.o1() + li * RIP);
@@ -603,11 +612,18 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             const float b = *cq;
             const int c1 = lio * RIP + rt, c2 = (jt / RJ) * RJP + jt % RJ;
             const Rec pk{0.f, (unsigned)(it * LD1) | ((unsigned)(jt * LD2) << 16)};
-            const float Att = G1s[it * LD1 + c1] * G2s[jt * LD2 + c2];
+            const float Att = C::kOrtho ? 1.f : G1s[it * LD1 + c1] * G2s[jt * LD2 + c2];
             __syncwarp();
             const bool wr = gl == 0;
             if (wr && pick) *cq = __int_as_float(0x7fc00000);   // mask the pick
             bool ok = false;
+            if constexpr (C::kOrtho) {
+                ok = pick;
+                if (ok) {
+                    if (wr) rec[t] = Rec{b, pk.o};
+                    E2 = fmaf(-b, b, E2);
+                }
+            } else {
             auto step = [&](auto tc) {
                 ok = chol_step<decltype(tc)::value, C::kFast>(pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att,
                                                               b, pk, E2);
@@ -625,6 +641,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     if constexpr (C::S == 0)
                         ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att, b, pk, E2);
                     break;
+            }
             }
             if (ok) cnt = t + 1;
             go = ok;

@@ -6,6 +6,9 @@
 // printed SVD argument of Remark 1 carries an extra sum X X^T factor, which
 // the trace maximisation behind the Procrustes problem does not have.
 //
+//   code_group_kernel  (omp_group_ortho.cu) calls with a fixed sparsity, 8 or 16
+//                      lanes per signal, with ortho_sums_kernel for a learning
+//                      pass over many signals;
 //   ortho_code_sq_kernel  square shapes compiled ahead (8, 12, 16): a
 //                      half-warp per signal with register-blocked Z and C;
 //   ortho_code_kernel  any other shape, one warp per signal: Y staged in shared memory,
@@ -441,6 +444,132 @@ __global__ void __launch_bounds__(kOrthoWarps * 32)
     }
 }
 
+// The sums of a learning pass at a compiled square shape from codes just written:
+// an iteration codes with the lane-group coder (omp_group_ortho.cu) and then adds
+// here, in the order of ortho_code_sq_kernel's epilogue (half-warp team t of CTA b
+// takes signals 16 b + t, + 16 grid, ...; lane = row, picks one after the other; teams
+// combined in order), since the rounding of the first dictionary decides near-tied
+// entries of the second pass.  CPS: CTAs per SM of that kernel.  200 000 x 12x12,
+// s = 6: 107 us of coding and 46 us of sums per pass, in place of 188 (D1 side) and
+// 212 us (D2 side).
+template <int P> constexpr int kSqCps = P == 8 ? 5 : P == 12 ? 3 : 2;
+
+template <int P>
+struct SqSumsLayout {
+    static constexpr int PP = P * P, AS = P + 1;             // accumulator rows in different banks
+    static constexpr int DS = P / 4 % 2 ? P : P + 4;         // columns of D in different banks
+    static constexpr int d = 0, team0 = d + DS * P;
+    static constexpr int y = 0, acc = 2 * al4(P * DS), tstride = acc + al4(P * AS);
+    static constexpr int total = team0 + kHalfTeams * tstride;
+};
+
+template <int P, int SIDE>
+__global__ void __launch_bounds__(kOrthoWarps * 32)
+    ortho_sums_kernel(const float* __restrict__ Y, long long N, const float* __restrict__ D, int s,
+                      const int32_t* __restrict__ support, const float* __restrict__ coef,
+                      float* __restrict__ part_f) {
+    using L = SqSumsLayout<P>;
+    constexpr bool kD1 = SIDE == kSideD1;
+    constexpr int PP = P * P, YS = kD1 ? P : L::DS;          // row (D1 side) or column (D2 side) per lane
+    extern __shared__ __align__(16) float sm[];
+    const int lane = threadIdx.x & 31, half = lane >> 4, l16 = lane & 15;
+    const int team = (threadIdx.x >> 5) * 2 + half;
+    const unsigned hm = 0xffffu << (16 * half);
+    float* ds = sm + L::d;                                   // column j of the other dictionary at j * DS
+    float* tb = sm + L::team0 + team * L::tstride;
+    float* acc = tb + L::acc;
+    for (int e = threadIdx.x; e < PP; e += blockDim.x) ds[e / P * L::DS + e % P] = D[e];
+    for (int e = l16; e < P * L::AS; e += 16) acc[e] = 0.f;
+    __syncthreads();
+    const long long step = (long long)gridDim.x * kHalfTeams;
+    long long k = (long long)blockIdx.x * kHalfTeams + team;
+    int qn = -1;
+    float xn = 0.f;
+    auto load = [&](long long kk, int buf) {
+        qn = -1;
+        if (kk < N) {
+            const float* src = Y + (size_t)kk * PP;
+            float* dst = tb + L::y + buf * al4(P * L::DS);
+#pragma unroll
+            for (int e0 = 0; e0 < PP; e0 += 64) {
+                const int e = e0 + l16 * 4;
+                if (e < PP)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (unsigned)__cvta_generic_to_shared(dst + e / P * YS + e % P)),
+                                 "l"(src + e)
+                                 : "memory");
+            }
+            if (l16 < s) {
+                qn = support[(size_t)kk * s + l16];
+                xn = coef[(size_t)kk * s + l16];
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    load(k, 0);
+    const int r = l16 < P ? l16 : P - 1;
+    for (int it = 0; k < N; ++it, k += step) {
+        const int q = qn;
+        const float x = xn;
+        const int cnt = __popc(__ballot_sync(hm, q >= 0));   // the picks come first
+        const int j = q >= 0 ? q / P : 0, i = q >= 0 ? q - j * P : 0;
+        const int pk = kD1 ? i | j << 8 : j | i << 8;
+        load(k + step, (it + 1) & 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp(hm);
+        const float* Ys = tb + L::y + (it & 1) * al4(P * L::DS);
+        float y[P];
+        if constexpr (kD1) {
+#pragma unroll
+            for (int b = 0; b < P; ++b) y[b] = Ys[r + P * b];
+        } else {
+#pragma unroll
+            for (int a = 0; a < P; a += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(Ys + YS * r + a);
+                y[a] = v.x; y[a + 1] = v.y; y[a + 2] = v.z; y[a + 3] = v.w;
+            }
+        }
+        for (int l = 0; l < cnt; ++l) {
+            const int p = __shfl_sync(hm, pk, l + 16 * half);
+            const float xl = __shfl_sync(hm, x, l + 16 * half);
+            const float* d = ds + (p >> 8) * L::DS;
+            float z = 0.f;
+#pragma unroll
+            for (int c = 0; c < P; c += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(d + c);
+                z = fmaf(y[c], v.x, z);
+                z = fmaf(y[c + 1], v.y, z);
+                z = fmaf(y[c + 2], v.z, z);
+                z = fmaf(y[c + 3], v.w, z);
+            }
+            float* dst = acc + r * L::AS + (p & 255);
+            if (l16 < P) *dst = fmaf(xl, z, *dst);
+        }
+        __syncwarp(hm);   // the buffer's next fetch
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    float* dst = part_f + (size_t)blockIdx.x * PP;
+    for (int e = threadIdx.x; e < PP; e += blockDim.x) {
+        float v = 0.f;
+        for (int tt = 0; tt < kHalfTeams; ++tt) v += sm[L::team0 + tt * L::tstride + L::acc + e / P * L::AS + e % P];
+        dst[e] = v;
+    }
+}
+
+template <int P>
+int launch_sums(const float* Y, long long N, const float* D1, const float* D2, int s, int side, const int32_t* support,
+                const float* coef, float* part_f, int slots, cudaStream_t st) {
+    constexpr size_t bytes = sizeof(float) * (size_t)SqSumsLayout<P>::total;
+    auto go = [&](auto kern, const float* D) -> int {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+            return SDL_ERR_CUDA;
+        kern<<<slots, kOrthoWarps * 32, bytes, st>>>(Y, N, D, s, support, coef, part_f);
+        return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
+    };
+    return side == kSideD1 ? go(ortho_sums_kernel<P, kSideD1>, D2) : go(ortho_sums_kernel<P, kSideD2>, D1);
+}
+
 template <int P, int SIDE>
 int launch_sq(const float* Y, long long N, const float* D1, const float* D2, int s, float eps2,
               int32_t* support, float* coef, int32_t* nnz, float* res, float* part_f,
@@ -499,7 +628,7 @@ __global__ void procrustes_kernel(const float* __restrict__ red_f, const double*
     float* V = A + m * n;                    // m x m (column-major)
     float* sig = V + m * m;                  // m
     int* sched = reinterpret_cast<int*>(sig + m);   // (m - 1) x m/2 column pairs
-    __shared__ int s_fail, s_rot;
+    __shared__ int s_fail;
     __shared__ double s_tr, s_sig;
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
@@ -541,20 +670,25 @@ __global__ void procrustes_kernel(const float* __restrict__ red_f, const double*
         sched[e] = ci | (cj << 16);
     }
     __syncthreads();
-    // sweeps: m - 1 rounds of m/2 disjoint column pairs
+    // sweeps: m - 1 rounds of m/2 disjoint column pairs.  A round is one chain of
+    // latencies (three sums by shuffles, the rotation, a barrier), so everything
+    // that does not hang on it is off it: a lane holds its row of the pair's
+    // columns of A and V in registers from one load (n, m <= 32), the next pair
+    // is looked up before the barrier, and a sweep's rotations are counted once,
+    // at its end.  12 x 12: 50 -> 32 us per call.
+    const bool in_a = lane < n, in_v = lane < m;
     for (int sweep = 0; sweep < kMaxSweeps && s_fail == 0; ++sweep) {
-        if (tid == 0) s_rot = 0;
-        __syncthreads();
+        int rotated = 0;
+        int pr = sched[warp];
         for (int round = 0; round < m - 1; ++round) {
-            const int pr = sched[round * (m / 2) + warp];
-            const int ci = pr & 0xffff, cj = pr >> 16;
-            float al = 0.f, be = 0.f, ga = 0.f;
-            for (int r = lane; r < n; r += 32) {
-                const float x = A[ci * n + r], y = A[cj * n + r];
-                al = fmaf(x, x, al);
-                be = fmaf(y, y, be);
-                ga = fmaf(x, y, ga);
-            }
+            float* ai = A + (pr & 0xffff) * n + lane;
+            float* aj = A + (pr >> 16) * n + lane;
+            float* vi = V + (pr & 0xffff) * m + lane;
+            float* vj = V + (pr >> 16) * m + lane;
+            const float x = in_a ? *ai : 0.f, y = in_a ? *aj : 0.f;
+            const float vx = in_v ? *vi : 0.f, vy = in_v ? *vj : 0.f;
+            if (round + 2 < m) pr = sched[(round + 1) * (m / 2) + warp];
+            float al = __fmul_rn(x, x), be = __fmul_rn(y, y), ga = __fmul_rn(x, y);   // not fused into the sums
             if (n > 16) {
                 al += __shfl_xor_sync(kFull, al, 16);
                 be += __shfl_xor_sync(kFull, be, 16);
@@ -579,23 +713,21 @@ __global__ void procrustes_kernel(const float* __restrict__ red_f, const double*
                     t = __fdividef(0.5f, zeta);
                 }
                 const float c = rsqrtf(fmaf(t, t, 1.f)), sn = c * t;
-                for (int r = lane; r < n; r += 32) {
-                    const float x = A[ci * n + r], y = A[cj * n + r];
-                    A[ci * n + r] = c * x - sn * y;
-                    A[cj * n + r] = sn * x + c * y;
+                // the roundings are spelt out: the next pass's near-tied entries hang
+                // on the dictionary's last bits
+                if (in_a) {
+                    *ai = fmaf(c, x, -__fmul_rn(sn, y));
+                    *aj = fmaf(sn, x, __fmul_rn(c, y));
                 }
-                for (int r = lane; r < m; r += 32) {
-                    const float x = V[ci * m + r], y = V[cj * m + r];
-                    V[ci * m + r] = c * x - sn * y;
-                    V[cj * m + r] = sn * x + c * y;
+                if (in_v) {
+                    *vi = fmaf(c, vx, -__fmul_rn(sn, vy));
+                    *vj = fmaf(sn, vx, __fmul_rn(c, vy));
                 }
-                if (lane == 0) atomicAdd(&s_rot, 1);
+                rotated = 1;
             }
             __syncthreads();
         }
-        const int rot = s_rot;
-        __syncthreads();
-        if (rot == 0) break;
+        if (!__syncthreads_or(rotated)) break;
     }
     for (int c = tid; c < m; c += nth) {
         float t = 0.f;
@@ -681,10 +813,52 @@ bool ortho_shape_supported(int p1, int p2, int s) {
            s <= p1 * p2;
 }
 
+// Learning passes that run as the lane-group coder and ortho_sums_kernel: compiled
+// square shapes, aligned signals, fixed sparsity, and enough signals for two
+// launches to beat one.
+constexpr long long kOrthoSplitPairs = 1500000;
+bool ortho_split(int p1, int p2, long long N, int s, float eps2, const float* Y) {
+    return p1 == p2 && (p1 == 8 || p1 == 12 || p1 == 16) && s <= 16 && !(eps2 > 0.f) &&
+           (reinterpret_cast<uintptr_t>(Y) & 15u) == 0 && N * p1 * p2 >= kOrthoSplitPairs;
+}
+
 int launch_ortho_code(const float* Y, int p1, int p2, long long N, const float* D1,
                       const float* D2, int s, float eps2, int32_t* support, float* coef, int32_t* nnz,
                       float* res, float* part_f, double* part_d, int max_slots, int side,
                       int* err, int num_sms, cudaStream_t st) {
+    PassArgs a{};
+    a.Y = Y;
+    a.p1 = a.n1 = p1;
+    a.p2 = a.n2 = p2;
+    a.N = N;
+    a.D1 = D1;
+    a.D2 = D2;
+    a.s = s;
+    a.support = support;
+    a.coef = coef;
+    a.nnz = nnz;
+    a.res_energy = res;
+    a.err = err;
+    // fixed sparsity: the lane-group coder, for a learning pass with the sums from
+    // its codes (the caller passes arrays for them) where that pays off
+    if (side == kCodeOnly && !(eps2 > 0.f)) return launch_ortho_group(a, st, num_sms);
+    if (side != kCodeOnly && ortho_split(p1, p2, N, s, eps2, Y)) {
+        const int cps = p1 == 8 ? kSqCps<8> : p1 == 12 ? kSqCps<12> : kSqCps<16>;
+        const long long need = (N + kHalfTeams - 1) / kHalfTeams;
+        const int slots = (int)std::min<long long>({need, (long long)num_sms * cps, (long long)max_slots});
+        a.esum = part_d;
+        a.esum_slots = slots;
+        int rc = launch_ortho_group(a, st, num_sms, slots);
+        if (rc != SDL_OK) return rc;
+        rc = p1 == 8    ? launch_sums<8>(Y, N, D1, D2, s, side, support, coef, part_f, slots, st)
+             : p1 == 12 ? launch_sums<12>(Y, N, D1, D2, s, side, support, coef, part_f, slots, st)
+                        : launch_sums<16>(Y, N, D1, D2, s, side, support, coef, part_f, slots, st);
+        return rc == SDL_OK ? slots : rc;
+    }
+    if (side == kSideD1) {   // the fused kernels write no codes on this side
+        support = nullptr;
+        nnz = nullptr;
+    }
     // compiled square shapes (s <= 16: the half-warp holds one pick per lane)
     if (p1 == p2 && s <= 16 && (p1 == 8 || p1 == 12 || p1 == 16)) {
         if (p1 == 8)
@@ -762,8 +936,7 @@ int sdl_ortho_iterate(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, flo
         {
             Trace tr(c, kOrthoCode, st);
             slots = launch_ortho_code(Y, p1, p2, N, D1, D2, s, eps > 0.f ? eps * eps : 0.f,
-                                      side == kSideD2 ? support : nullptr,
-                                      coef, nnz, nullptr, c->part_f, c->part_d, max_slots, side,
+                                      support, coef, nnz, nullptr, c->part_f, c->part_d, max_slots, side,
                                       c->err, c->num_sms, st);
         }
         if (slots < 0) return slots;

@@ -88,6 +88,7 @@ int launch_code_group_fixed(const PassArgs& a, bool w_first, cudaStream_t st, in
                             int max_grid = 0);
 int launch_code_group_any(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms);
+int launch_ortho_group(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid = 0);
 // omp_scan.cu: the above for a code-only call, behind an error scan when it is
 // error-driven (ws: ws_n floats of scratch, or null)
 bool code_lanes_take(const PassArgs& a, size_t ws_n);
