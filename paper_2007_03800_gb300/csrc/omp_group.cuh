@@ -203,15 +203,15 @@ struct alignas(8) Rec {
 // One greedy step's Cholesky row T and the coefficients of the T + 1 picks
 // (every lane of the signal holds the same values; `writer` stores them).
 // Returns false (state untouched) when the pick is degenerate or !live.
-template <int T, bool kFast>
+// gram(r): the product of the Gram entries of the new pick and pick r.
+template <int T, bool kFast, class Gram>
 __device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, float* lf, float* iv, float* yv,
-                                          const float* G1s, const float* G2s, int c1, int c2, float Att,
-                                          float b, const Rec& pick, float& E) {
+                                          Gram gram, float Att, float b, const Rec& pick, float& E) {
     constexpr int NL = T * (T - 1) / 2;
     float L[NL > 0 ? up4(NL) : 1], io[T > 0 ? up4(T) : 1], yo[T > 0 ? up4(T) : 1], am[T > 0 ? T : 1];
     if constexpr (T > 0) {
 #pragma unroll
-        for (int m = 0; m < T; ++m) am[m] = G1s[rec[m].o1() + c1] * G2s[rec[m].o2() + c2];
+        for (int m = 0; m < T; ++m) am[m] = gram(rec[m]);
 #pragma unroll
         for (int k = 0; k < NL; k += 4) {
             const float4 t = *reinterpret_cast<const float4*>(lf + k);
@@ -275,14 +275,13 @@ __device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, floa
 // The same for any t, as loops through shared memory (row t of the factor and
 // the coefficients are written by every lane of the signal with equal values;
 // a step that fails leaves them unread).
-template <bool kFast>
+template <bool kFast, class Gram>
 __device__ __forceinline__ bool chol_step_any(int t, bool live, bool writer, Rec* rec, float* lf, float* iv,
-                                              float* yv, const float* G1s, const float* G2s, int c1, int c2,
-                                              float Att, float b, const Rec& pick, float& E) {
+                                              float* yv, Gram gram, float Att, float b, const Rec& pick, float& E) {
     float* w = lf + t * (t - 1) / 2;
     float ww = 0.f, wy = 0.f;
     for (int m = 0; m < t; ++m) {
-        float v = G1s[rec[m].o1() + c1] * G2s[rec[m].o2() + c2];
+        float v = gram(rec[m]);
         const float* Lm = lf + m * (m - 1) / 2;
         for (int l = 0; l < m; ++l) v = fmaf(-Lm[l], w[l], v);
         const float wm = v * iv[m];
@@ -624,9 +623,9 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     E2 = fmaf(-b, b, E2);
                 }
             } else {
+            auto gram = [&](const Rec& r) { return G1s[r.o1() + c1] * G2s[r.o2() + c2]; };
             auto step = [&](auto tc) {
-                ok = chol_step<decltype(tc)::value, C::kFast>(pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att,
-                                                              b, pk, E2);
+                ok = chol_step<decltype(tc)::value, C::kFast>(pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
             };
             switch (t) {
                 case 0: step(std::integral_constant<int, 0>{}); break;
@@ -639,7 +638,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 case 7: if constexpr (C::SMAX > 7) step(std::integral_constant<int, 7>{}); break;
                 default:
                     if constexpr (C::S == 0)
-                        ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, G1s, G2s, c1, c2, Att, b, pk, E2);
+                        ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
                     break;
             }
             }

@@ -133,6 +133,10 @@ int max_partial_slots(int num_sms);
 // tmod3_fast.cu: three-mode coding pass specialised at compile time for the
 // compiled shapes (SDL_ERR_UNSUPPORTED otherwise or for a Y not 16-byte
 // aligned); returns the partial-sum slots written (mode 1-3) or 0 (mode 0)
+// tmod3_group.cu: the same shapes without partial sums (no Gram matrices needed)
+int launch_code3_group(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, long long N, const float* D1,
+                       const float* D2, const float* D3, int s, int32_t* support, float* coef, int32_t* nnz,
+                       float* res, int* err, int num_sms, cudaStream_t st);
 int launch_code3_fast(int mode, const float* Y, int p1, int p2, int p3, int n1, int n2, int n3,
                       long long N, const float* D1, const float* D2, const float* D3,
                       const float* G1, const float* G2, const float* G3, int s, int32_t* support,
