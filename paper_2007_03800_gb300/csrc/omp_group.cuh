@@ -46,17 +46,21 @@ __host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
 // ORTHO_: 0, or the orthonormal variant (n = p; a pick's coefficient is its
 // correlation and leaves the others alone) with ||Y||^2 in that many chains.
 template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,
-          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0>
+          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0, int CHAINS_ = 32>
 struct Cfg {
     static constexpr bool kOrtho = ORTHO_ > 0;
-    static constexpr int CHAINS = ORTHO_ > 0 ? ORTHO_ : 32;   // of ||Y||^2
-    static constexpr int CPL = CHAINS / GL_;                  // per lane
-    static_assert(CPL == 1 || CPL == 2 || CPL == 4, "chains");
+    static constexpr int CHAINS = ORTHO_ > 0 ? ORTHO_ : CHAINS_;   // of ||Y||^2 (128: four warps' worth)
+    static constexpr int CPL = CHAINS / GL_;                       // per lane
+    // a group of 64 lanes is a team of two warps that meet at a named barrier
+    static constexpr int TW = GL_ > 32 ? GL_ / 32 : 1;
+    static constexpr int XS = TW > 1 ? 16 : 0;                     // exchange slots between them
+    static_assert(CHAINS == 128 || CPL == 1 || CPL == 2 || CPL == 4, "chains");
+    static_assert(TW == 1 || CHAINS == 128, "a team's chains");
     static constexpr int GL = GL_, LI = LI_, LJ = GL_ / LI_, RI = RI_, RJ = RJ_;
     static constexpr int WARPS = WARPS_, MINB = MINB_;
     static constexpr bool kFast = FAST_, kW = W_;
     static constexpr int P1 = P1_, P2 = P2_, N1 = N1_, N2 = N2_, S = S_;
-    static constexpr int SPW = 32 / GL;                 // signals per warp
+    static constexpr int SPW = GL < 32 ? 32 / GL : 1;   // signals per warp (or team)
     static constexpr int N1P = LI * RI, N2P = LJ * RJ;
     static constexpr int RIP = up4(RI), RJP = up4(RJ);  // padded block lengths (16-byte loads)
     static constexpr int LD1 = LI * RIP, LD2 = LJ * RJP;
@@ -68,7 +72,7 @@ struct Cfg {
     // rows per lane and block of the Z stage (Y D2), columns of the W stage
     static constexpr int ZA = P1 ? (P1 / LI) : 4;
     static constexpr int WB = P2 ? (P2 / LJ) : 4;
-    static constexpr int SMAX = S ? S : 8;              // unrolled Cholesky rows
+    static constexpr int SMAX = S ? S : TW > 1 ? 10 : 8;   // unrolled Cholesky rows
     static_assert(N1P * LD1 <= 65536 && N2P * LD2 <= 65536, "16-bit row offsets");
     static_assert(E % 2 == 0 && RI % 2 == 0, "row pairs, 16-byte block stores");
     static_assert((LI & (LI - 1)) == 0 && LI * LJ == GL, "lane grid");
@@ -81,8 +85,8 @@ struct Cfg {
 struct Layout {
     int p1s;       // row stride of a staged signal's columns (p1 rounded up to 4)
     int d1, d2, g1, g2, warp0;
-    int y, c0, col, rec, lf, iv, yv, sig_stride;   // per signal
-    int warp_stride, total;
+    int y, c0, col, xs, rec, lf, iv, yv, sig_stride;   // per signal
+    int total;
 };
 
 template <class C>
@@ -99,7 +103,8 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     const int z = C::kW ? p2 * C::LD1 : up4(p1) * C::LD2;   // Z or W shares the C0 blocks' place
     const int c = C::GL * C::EP;
     L.col = L.c0 + (z > c ? z : c);
-    L.rec = L.col + C::CS;
+    L.xs = L.col + C::CS;
+    L.rec = L.xs + C::XS;
     L.lf = L.rec + up4(2 * s);
     L.iv = L.lf + (C::kOrtho ? 0 : up4(s * (s - 1) / 2));
     L.yv = L.iv + (C::kOrtho ? 0 : up4(s));
@@ -108,8 +113,7 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     // same offsets together
     while (st % 32 != 8 && st % 32 != 24) st += 4;
     L.sig_stride = st;
-    L.warp_stride = C::SPW * st;
-    L.total = L.warp0 + warps * L.warp_stride;
+    L.total = L.warp0 + warps * 32 / C::GL * st;
     return L;
 }
 
@@ -317,6 +321,42 @@ __device__ __forceinline__ bool chol_step_any(int t, bool live, bool writer, Rec
     return true;
 }
 
+// G (row i: the products with every position of a lane-block row) of the
+// dictionary whose rows are d, by the whole CTA; wide ones in 4 x 4 blocks
+// (128 atoms x 64 rows: a plain loop reads two words per multiply-add)
+template <int R, int RP, int NP, int LD>
+__device__ __forceinline__ void gram(const float* d, int p, float* G) {
+    if constexpr (R % 4 == 0 && NP >= 64) {
+        for (int e = threadIdx.x; e < NP / 4 * (LD / 4); e += blockDim.x) {
+            const int i0 = e / (LD / 4) * 4, pos = e % (LD / 4) * 4;
+            const float* di = d + i0 / R * RP + i0 % R;
+            float g[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) g[k] = 0.f;
+#pragma unroll 2
+            for (int r = 0; r < p; ++r) {
+                float x[4], y[4];
+                ld<4>(x, d + r * LD + pos);
+                ld<4>(y, di + r * LD);
+                rank1<4, 4>(g, x, y);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float v[4] = {g[4 * k], g[4 * k + 1], g[4 * k + 2], g[4 * k + 3]};
+                st<4>(G + (i0 + k) * LD + pos, v);
+            }
+        }
+    } else {
+        for (int e = threadIdx.x; e < NP * LD; e += blockDim.x) {
+            const int i = e / LD, pos = e % LD;
+            const float* di = d + i / R * RP + i % R;
+            float g = 0.f;
+            for (int r = 0; r < p; ++r) g = fmaf(di[r * LD], d[r * LD + pos], g);
+            G[e] = g;
+        }
+    }
+}
+
 // compensated running sum
 __device__ __forceinline__ void ksum(float& s, float& c, float v) {
     const float y = v - c;
@@ -339,19 +379,27 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
     const int s = C::S ? C::S : a.s;
     const int pp = p1 * p2;
     const bool error_driven = a.eps2 > 0.f;
-    const int warps = blockDim.x >> 5;
+    constexpr int TW = C::TW;
+    const int warps = blockDim.x >> 5, workers = warps / TW;
     const Layout L = layout<C>(p1, p2, s, warps);
     const int p1s = L.p1s;
 
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = lane / GL, gl = lane % GL;
+    const int grp = GL < 32 ? lane / GL : 0, gl = threadIdx.x % GL;
+    const int worker = threadIdx.x / (32 * TW);   // warp or team
     const int li = gl % LI, lj = gl / LI;
     float* D1s = sm + L.d1;    // row a: D1[a, :] in lane blocks
     float* D2s = sm + L.d2;    // row b: D2[b, :] in lane blocks
     float* G1s = sm + L.g1;
     float* G2s = sm + L.g2;
-    float* wb = sm + L.warp0 + w * L.warp_stride;
-    float* sb = wb + grp * L.sig_stride;
+    float* sb = sm + L.warp0 + (threadIdx.x / GL) * L.sig_stride;
+    // the lanes of a signal (and the other signals of its warp) meet
+    auto sync = [&]() {
+        if constexpr (TW == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(32 * TW) : "memory");
+    };
+    // whether any signal of the warp (the one of the team, whose lanes agree) goes on
+    auto any = [&](bool v) { return TW == 1 ? __any_sync(kFull, v) != 0 : v; };
     float* Ys = sb + L.y;
     float* Zs = sb + L.c0;     // Z (rows a) or W (rows b), then the C0 blocks
     float* C0s = sb + L.c0;
@@ -375,35 +423,18 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
     }
     // a signal's records start valid: a finished signal's lanes run along with
     // the others of the warp on whatever its records hold
-    for (int e = lane; e < SPW * s; e += 32) {
-        const int g = e / s;
-        reinterpret_cast<Rec*>(wb + g * L.sig_stride + L.rec)[e - g * s] = Rec{0.f, 0u};
-    }
+    for (int l = gl; l < s; l += GL) rec[l] = Rec{0.f, 0u};
     __syncthreads();
     if constexpr (!C::kOrtho) {
-    for (int e = threadIdx.x; e < C::N1P * LD1; e += blockDim.x) {
-        const int i = e / LD1, pos = e % LD1;
-        const float* di = D1s + (i / RI) * RIP + i % RI;
-        const float* dj = D1s + pos;
-        float g = 0.f;
-        for (int r = 0; r < p1; ++r) g = fmaf(di[r * LD1], dj[r * LD1], g);
-        G1s[e] = g;
-    }
-    for (int e = threadIdx.x; e < C::N2P * LD2; e += blockDim.x) {
-        const int j = e / LD2, pos = e % LD2;
-        const float* di = D2s + (j / RJ) * RJP + j % RJ;
-        const float* dj = D2s + pos;
-        float g = 0.f;
-        for (int r = 0; r < p2; ++r) g = fmaf(di[r * LD2], dj[r * LD2], g);
-        G2s[e] = g;
-    }
-    __syncthreads();
+        gram<RI, RIP, C::N1P, LD1>(D1s, p1, G1s);
+        gram<RJ, RJP, C::N2P, LD2>(D2s, p2, G2s);
+        __syncthreads();
     }
 
     const long long count = a.idx ? (long long)*a.idx_count : a.N;
     const long long units = (count + SPW - 1) / SPW;
-    const long long ustep = (long long)gridDim.x * warps;
-    long long u = (long long)w * gridDim.x + blockIdx.x;   // next unit
+    const long long ustep = (long long)gridDim.x * workers;
+    long long u = (long long)worker * gridDim.x + blockIdx.x;   // next unit
 
     // signals start on 16-byte boundaries and columns stay 16-byte aligned
     const bool vec = (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0 && (C::P1 ? true : p1 % 4 == 0);
@@ -431,11 +462,11 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
 
     long long pos = next_pos();
     if (pos >= 0) fetch(a.idx ? (long long)a.idx[pos] : pos);
-    while (__any_sync(kFull, pos >= 0)) {
+    while (any(pos >= 0)) {
         const bool act = pos >= 0;
         const long long ko = !act ? 0 : (a.idx && !a.idx_compact) ? (long long)a.idx[pos] : pos;
         cp_wait();
-        __syncwarp();
+        sync();
         // ---- ||Y||^2: the strided partial sums of the one-signal-per-warp (or half
         // warp) coders (this lane takes CPL of them) and their combining tree
         float part[C::CPL];
@@ -454,11 +485,37 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 }
         }
         float ss;
-        if constexpr (C::CPL == 4) ss = (part[0] + part[2]) + (part[1] + part[3]);
-        else if constexpr (C::CPL == 2) ss = part[0] + part[1];
-        else ss = part[0];
+        if constexpr (C::CHAINS == 128) {
+            // four warps' sums, added in order; chain GL v + gl belongs to lane
+            // (GL v + gl) % 32 of warp (GL v + gl) / 32
+            float ws[4];
 #pragma unroll
-        for (int o = GL / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
+            for (int v = 0; v < 4; ++v) {
+                if constexpr (GL == 16) ws[v] = part[2 * v] + part[2 * v + 1];
+                else if constexpr (GL == 32) ws[v] = part[v];
+                else ws[v] = part[v / 2];
+#pragma unroll
+                for (int o = GL < 32 ? GL / 2 : 16; o > 0; o >>= 1) ws[v] += __shfl_xor_sync(kFull, ws[v], o);
+            }
+            if constexpr (TW > 1) {   // this warp has warps w % 2 and w % 2 + 2
+                const int h = w % TW;
+                float* xs = sb + L.xs + 8;
+                if (lane == 0) {
+                    xs[h] = ws[0];
+                    xs[h + 2] = ws[2];
+                }
+                sync();
+#pragma unroll
+                for (int v = 0; v < 4; ++v) ws[v] = xs[v];
+            }
+            ss = ((ws[0] + ws[1]) + ws[2]) + ws[3];
+        } else {
+            if constexpr (C::CPL == 4) ss = (part[0] + part[2]) + (part[1] + part[3]);
+            else if constexpr (C::CPL == 2) ss = part[0] + part[1];
+            else ss = part[0];
+#pragma unroll
+            for (int o = GL / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
+        }
         const bool finite = act && isfinite(ss);
         bool go = finite && !(error_driven && ss <= a.eps2);
 
@@ -508,7 +565,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 st<RI>(Zs + (lj + LJ * c) * LD1 + li * RIP, v);
             }
         }
-        __syncwarp();
+        sync();
         // Y is consumed: fetch the next unit's signals
         const long long pos_next = next_pos();
         if (pos_next >= 0) fetch(a.idx ? (long long)a.idx[pos_next] : pos_next);
@@ -541,18 +598,22 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 for (int r = 0; r < RI; ++r)
                     if (li * RI + r >= n1 || lj * RJ + c >= n2) sc[c * RI + r] = __int_as_float(0x7fc00000);
         }
-        __syncwarp();   // every lane has read Z: its place takes the C0 blocks
+        sync();   // every lane has read Z: its place takes the C0 blocks
         st<E>(myc0, sc);
-        __syncwarp();
+        sync();
 
         // ---- greedy steps
         int cnt = 0;
         float E2 = ss;
+        float* masked = nullptr;
 #pragma unroll 1
         for (int t = 0; t < s; ++t) {
             const bool live = go && !(error_driven && E2 <= a.eps2);
-            if (!__any_sync(kFull, live)) break;
+            if (!any(live)) break;
             if (t > 0) {
+                // the last pick leaves the search: its owner masks it here, after
+                // every lane has read the entry
+                if (masked) *masked = __int_as_float(0x7fc00000);
                 ld<E>(sc, myc0);
 #pragma unroll 1
                 for (int l = 0; l < (C::kOrtho ? 0 : t); ++l) {
@@ -579,10 +640,20 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             float M = best;
             int key = (lj * RJ + bc) * LI + li;
 #pragma unroll
-            for (int o = GL / 2; o > 0; o >>= 1) {
+            for (int o = GL < 32 ? GL / 2 : 16; o > 0; o >>= 1) {
                 const float mo = __shfl_xor_sync(kFull, M, o);
                 const int ko2 = __shfl_xor_sync(kFull, key, o);
                 if (mo > M || (mo == M && ko2 < key)) { M = mo; key = ko2; }
+            }
+            if constexpr (TW > 1) {   // two slots per parity of t: no barrier before their next use
+                float* xs = sb + L.xs + 4 * (t & 1);
+                if (lane == 0) *reinterpret_cast<float2*>(xs + 2 * (w % TW)) = make_float2(M, __int_as_float(key));
+                sync();
+                const float4 v = *reinterpret_cast<const float4*>(xs);
+                const int k0 = __float_as_int(v.y), k1 = __float_as_int(v.w);
+                const bool first = v.x > v.z || (v.x == v.z && k0 < k1);
+                M = first ? v.x : v.z;
+                key = first ? k0 : k1;
             }
             const bool pick = live && M != 0.f;
             const int jt = key / LI, lio = key % LI;
@@ -597,13 +668,15 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                         st<RI>(col, v);
                     }
             }
-            __syncwarp();
+            sync();
             unsigned rows = 0;
 #pragma unroll
             for (int r0 = 0; r0 < RI; r0 += GL) {
-                const bool eq = r0 + gl < RI && fabsf(col[r0 + gl]) == M;
+                constexpr int GW = GL < 32 ? GL : 32;
+                const int r = r0 + lane % GW;
+                const bool eq = r < RI && fabsf(col[r]) == M;
                 const unsigned bal = __ballot_sync(kFull, eq);
-                rows |= ((bal >> (GL * grp)) & ((1u << GL) - 1u)) << r0;
+                rows |= ((bal >> (GW * grp)) & (unsigned)((1ull << GW) - 1ull)) << r0;
             }
             const int rt = rows ? __ffs(rows) - 1 : 0;
             const int it = lio * RI + rt;
@@ -612,9 +685,8 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             const int c1 = lio * RIP + rt, c2 = (jt / RJ) * RJP + jt % RJ;
             const Rec pk{0.f, (unsigned)(it * LD1) | ((unsigned)(jt * LD2) << 16)};
             const float Att = C::kOrtho ? 1.f : G1s[it * LD1 + c1] * G2s[jt * LD2 + c2];
-            __syncwarp();
             const bool wr = gl == 0;
-            if (wr && pick) *cq = __int_as_float(0x7fc00000);   // mask the pick
+            masked = pick && gl == lio + LI * (jt / RJ) ? cq : nullptr;
             bool ok = false;
             if constexpr (C::kOrtho) {
                 ok = pick;
@@ -636,6 +708,18 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 case 5: if constexpr (C::SMAX > 5) step(std::integral_constant<int, 5>{}); break;
                 case 6: if constexpr (C::SMAX > 6) step(std::integral_constant<int, 6>{}); break;
                 case 7: if constexpr (C::SMAX > 7) step(std::integral_constant<int, 7>{}); break;
+                case 8:
+                    if constexpr (C::SMAX > 8) {
+                        step(std::integral_constant<int, 8>{});
+                        break;
+                    }
+                    [[fallthrough]];
+                case 9:
+                    if constexpr (C::SMAX > 9) {
+                        step(std::integral_constant<int, 9>{});
+                        break;
+                    }
+                    [[fallthrough]];
                 default:
                     if constexpr (C::S == 0)
                         ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
@@ -644,7 +728,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             }
             if (ok) cnt = t + 1;
             go = ok;
-            __syncwarp();   // the step's state and the masked entry are visible
+            sync();   // the step's state is visible
         }
 
         // ---- the code
@@ -663,7 +747,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 else record_error(a.err, SDL_ERR_NONFINITE);
             }
         }
-        __syncwarp();   // records are read before the next unit writes them
+        sync();   // records are read before the next unit writes them
         pos = pos_next;
     }
 
@@ -696,8 +780,8 @@ int launch(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid) {
     constexpr size_t kSmMax = 227 * 1024, kSmTotal = 228 * 1024;
     int warps = C::WARPS;
     size_t bytes;
-    while ((bytes = sizeof(float) * (size_t)layout<C>(a.p1, a.p2, a.s, warps).total) > kSmMax && warps > 1)
-        --warps;
+    while ((bytes = sizeof(float) * (size_t)layout<C>(a.p1, a.p2, a.s, warps).total) > kSmMax && warps > C::TW)
+        warps -= C::TW;
     if (bytes > kSmMax) return SDL_ERR_UNSUPPORTED;
     auto kern = code_group_kernel<C>;
     // the shared-memory opt-in, once per device

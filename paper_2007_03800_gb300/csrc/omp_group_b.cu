@@ -10,7 +10,7 @@ int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms) {
     if (n1 <= 24 && n2 <= 32) return group::launch<group::Cfg<16, 4, 6, 8, 8, 2, false, false>>(a, st, num_sms, 0);
     if (n1 <= 32 && n2 <= 24) return group::launch<group::Cfg<16, 4, 8, 6, 8, 2, false, false>>(a, st, num_sms, 0);
     if (n1 <= 32 && n2 <= 32) return group::launch<group::Cfg<16, 4, 8, 8, 8, 2, false, false>>(a, st, num_sms, 0);
-    return SDL_ERR_UNSUPPORTED;
+    return launch_code_group_cols(a, st, num_sms);
 }
 
 }  // namespace sdl

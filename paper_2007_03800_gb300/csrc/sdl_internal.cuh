@@ -82,12 +82,13 @@ int launch_code_pass_generic(const PassArgs& a, int side, cudaStream_t st, int n
 int launch_accumulate_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms);
 // omp_group_*.cu: code-only passes with 8 or 16 lanes per signal, in the
 // arithmetic of the compiled tilings (fixed: their shapes; w_first: correlations
-// as (D1^T Y) D2, at most max_grid CTAs) or of the generic kernel (any: n1, n2 <=
-// 32).  SDL_ERR_UNSUPPORTED for other shapes.
+// as (D1^T Y) D2, at most max_grid CTAs) or of the generic kernel (any: n1 <= 32,
+// n2 <= 128).  SDL_ERR_UNSUPPORTED for other shapes.
 int launch_code_group_fixed(const PassArgs& a, bool w_first, cudaStream_t st, int num_sms,
                             int max_grid = 0);
 int launch_code_group_any(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms);
+int launch_code_group_cols(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_ortho_group(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid = 0);
 // omp_scan.cu: the above for a code-only call, behind an error scan when it is
 // error-driven (ws: ws_n floats of scratch, or null)
