@@ -46,8 +46,18 @@ __host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
 // ORTHO_: 0, or the orthonormal variant (n = p; a pick's coefficient is its
 // correlation and leaves the others alone) with ||Y||^2 in that many chains.
 template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,
-          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0, int CHAINS_ = 32>
+          int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0, int CHAINS_ = 32,
+          bool TM_ = false>
 struct Cfg {
+    // the C0 blocks live in tensor memory instead of shared memory: they are read
+    // back whole every step, at a bandwidth of its own, and leave the shared memory
+    // to more signals in flight (one signal per warp or team, 8 x 8 blocks)
+    static constexpr bool kTM = TM_;
+    static constexpr int TUSED = kTM ? WARPS_ / 4 * RI_ * RJ_ : 0;
+    static constexpr int TCOLS = TUSED <= 64 ? TUSED : TUSED <= 128 ? 128 : TUSED <= 256 ? 256 : 512;   // of a CTA
+    static_assert(!kTM || (GL_ >= 32 && RI_ == 8 && RJ_ == 8 && WARPS_ % 4 == 0 && (TCOLS & (TCOLS - 1)) == 0 &&
+                           TCOLS >= 32 && TCOLS * MINB_ <= 512),
+                  "tensor memory");
     static constexpr bool kOrtho = ORTHO_ > 0;
     static constexpr int CHAINS = ORTHO_ > 0 ? ORTHO_ : CHAINS_;   // of ||Y||^2 (128: four warps' worth)
     static constexpr int CPL = CHAINS / GL_;                       // per lane
@@ -68,7 +78,7 @@ struct Cfg {
     // lane stride of the C0 blocks: an odd multiple of 4 floats, so that the 8
     // lanes of a 128-bit load phase hit distinct banks
     static constexpr int EP = (up4(E) / 4) % 2 ? up4(E) : up4(E) + 4;
-    static constexpr int CS = up4(RI);                  // the winning column's read-back buffer
+    static constexpr int CS = kTM ? 2 * RI : up4(RI);   // the winning column's read-back buffer (and its C0)
     // rows per lane and block of the Z stage (Y D2), columns of the W stage
     static constexpr int ZA = P1 ? (P1 / LI) : 4;
     static constexpr int WB = P2 ? (P2 / LJ) : 4;
@@ -101,7 +111,7 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     L.y = 0;
     L.c0 = L.y + L.p1s * p2;
     const int z = C::kW ? p2 * C::LD1 : up4(p1) * C::LD2;   // Z or W shares the C0 blocks' place
-    const int c = C::GL * C::EP;
+    const int c = C::kTM ? 0 : C::GL * C::EP;
     L.col = L.c0 + (z > c ? z : c);
     L.xs = L.col + C::CS;
     L.rec = L.xs + C::XS;
@@ -113,7 +123,7 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     // same offsets together
     while (st % 32 != 8 && st % 32 != 24) st += 4;
     L.sig_stride = st;
-    L.total = L.warp0 + warps * 32 / C::GL * st;
+    L.total = L.warp0 + warps * 32 / C::GL * st + (C::kTM ? 4 : 0);   // (the tensor-memory address)
     return L;
 }
 
@@ -194,6 +204,32 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sptr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ------------------------------------------------------------ tensor memory
+// Each warp reaches the 32 TMEM lanes of its quarter (warp % 4); thread = lane,
+// columns hold its floats.
+__device__ __forceinline__ void tm_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tm_ld8(unsigned ta, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(ta));
+}
+__device__ __forceinline__ void tm_st8(unsigned ta, const float* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(v[0]), "f"(v[1]),
+                 "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "r"(ta)
+                 : "memory");
+}
+__device__ __forceinline__ void tm_ld32(unsigned ta, float* v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+          "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]),
+          "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]),
+          "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])
+        : "r"(ta));
+}
 
 // One pick of a signal: its coefficient, and the offsets of its rows of G1
 // (low half) and G2 (high half) in shared memory, one 8-byte load.
@@ -431,6 +467,22 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         __syncthreads();
     }
 
+    // tensor memory of the CTA, and this warp's place in it
+    unsigned tbase = 0, tmine = 0;
+    unsigned* tslot = reinterpret_cast<unsigned*>(sm + L.total - 4);
+    if constexpr (C::kTM) {
+        if (w == 0) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sptr(tslot)),
+                         "r"(C::TCOLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tbase = *static_cast<volatile unsigned*>(tslot);
+        tmine = tbase + ((unsigned)(w % 4) << 21) + (unsigned)(w / 4 * E);
+    }
+
     const long long count = a.idx ? (long long)*a.idx_count : a.N;
     const long long units = (count + SPW - 1) / SPW;
     const long long ustep = (long long)gridDim.x * workers;
@@ -599,8 +651,14 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     if (li * RI + r >= n1 || lj * RJ + c >= n2) sc[c * RI + r] = __int_as_float(0x7fc00000);
         }
         sync();   // every lane has read Z: its place takes the C0 blocks
-        st<E>(myc0, sc);
-        sync();
+        if constexpr (C::kTM) {
+#pragma unroll
+            for (int e = 0; e < E; e += 8) tm_st8(tmine + e, sc + e);
+            tm_wait_st();
+        } else {
+            st<E>(myc0, sc);
+            sync();
+        }
 
         // ---- greedy steps
         int cnt = 0;
@@ -613,8 +671,16 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             if (t > 0) {
                 // the last pick leaves the search: its owner masks it here, after
                 // every lane has read the entry
-                if (masked) *masked = __int_as_float(0x7fc00000);
-                ld<E>(sc, myc0);
+                if constexpr (C::kTM) {
+                    __syncwarp();
+                    static_assert(!C::kTM || E == 64, "block");
+                    tm_ld32(tmine, sc);
+                    tm_ld32(tmine + 32, sc + (C::kTM ? 32 : 0));
+                    tm_wait_ld();
+                } else {
+                    if (masked) *masked = __int_as_float(0x7fc00000);
+                    ld<E>(sc, myc0);
+                }
 #pragma unroll 1
                 for (int l = 0; l < (C::kOrtho ? 0 : t); ++l) {
                     const Rec r = rec[l];
@@ -658,7 +724,22 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             const bool pick = live && M != 0.f;
             const int jt = key / LI, lio = key % LI;
             // the owner lane's column, and the first row that holds M
-            if (gl == lio + LI * (jt / RJ)) {
+            const int owner = lio + LI * (jt / RJ);
+            const bool owner_warp = TW == 1 || w % TW == owner / 32;
+            float c8[8];   // tensor memory: the C0 values of that column
+            if constexpr (C::kTM) {
+                if (owner_warp) {
+                    __syncwarp();
+                    tm_ld8(tmine + jt % RJ * RI, c8);
+                    tm_wait_ld();
+                    if (gl == owner)
+#pragma unroll
+                        for (int r = 0; r < RI; r += 4)
+                            *reinterpret_cast<float4*>(col + RI + r) =
+                                make_float4(c8[r], c8[r + 1], c8[r + 2], c8[r + 3]);
+                }
+            }
+            if (gl == owner) {
 #pragma unroll
                 for (int c = 0; c < RJ; ++c)
                     if (bc == c) {
@@ -680,13 +761,23 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             }
             const int rt = rows ? __ffs(rows) - 1 : 0;
             const int it = lio * RI + rt;
-            float* cq = C0s + (lio + LI * (jt / RJ)) * C::EP + (jt % RJ) * RI + rt;
+            float* cq = C::kTM ? col + RI + rt : C0s + owner * C::EP + (jt % RJ) * RI + rt;
             const float b = *cq;
+            if constexpr (C::kTM) {   // the pick leaves the search: masked in its owner's lane
+                if (owner_warp && pick) {
+                    __syncwarp();
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        if (gl == owner && r == rt) c8[r] = __int_as_float(0x7fc00000);
+                    tm_st8(tmine + jt % RJ * RI, c8);
+                    tm_wait_st();
+                }
+            }
             const int c1 = lio * RIP + rt, c2 = (jt / RJ) * RJP + jt % RJ;
             const Rec pk{0.f, (unsigned)(it * LD1) | ((unsigned)(jt * LD2) << 16)};
             const float Att = C::kOrtho ? 1.f : G1s[it * LD1 + c1] * G2s[jt * LD2 + c2];
             const bool wr = gl == 0;
-            masked = pick && gl == lio + LI * (jt / RJ) ? cq : nullptr;
+            masked = pick && gl == owner ? cq : nullptr;
             bool ok = false;
             if constexpr (C::kOrtho) {
                 ok = pick;
@@ -749,6 +840,15 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         }
         sync();   // records are read before the next unit writes them
         pos = pos_next;
+    }
+
+    if constexpr (C::kTM) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (w == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(C::TCOLS) : "memory");
+        }
     }
 
     // ---- residual energies of this CTA's signals, lanes and warps in a fixed

@@ -1,4 +1,4 @@
-"""The lane-group coder (code-only calls with n1, n2 <= 32) at the edges of its
+"""The lane-group coder (code-only calls with n1 <= 32, n2 <= 128) at the edges of its
 tiles: ragged dictionaries in each compiled tile, counts that leave units of a
 warp partly empty, sparsities past the unrolled Cholesky rows, signals so large
 that a CTA holds fewer warps, error-driven calls (scan and list), and signals
@@ -29,6 +29,12 @@ SHAPES = [  # p1, p2, n1, n2, s, N
     (8, 8, 16, 16, 12, 40),
     (32, 32, 16, 16, 4, 23),     # 1024-entry signals
     (2, 64, 5, 27, 3, 30),       # the longest side
+    (8, 16, 16, 40, 4, 61),      # 16 x 64 pairs: 16 lanes
+    (16, 24, 31, 64, 6, 45),     # 32 x 64: one warp per signal
+    (9, 30, 15, 100, 5, 40),     # 16 x 128
+    (12, 40, 25, 97, 12, 37),    # 32 x 128: teams of two warps, tensor memory, past the unrolled rows
+    (16, 64, 32, 128, 10, 331),  # the same with its sizes fixed
+    (16, 64, 32, 128, 1, 1),
 ]
 
 
