@@ -86,12 +86,19 @@ __device__ __forceinline__ void reduce_body(const float* __restrict__ part_f,
                 sum[u] = t;
             }
         }
-        for (; c < n_slots; c += kReduceWarps) {
-            const float y = part_f[(size_t)c * nf + e] - comp[0];
-            const float t = sum[0] + y;
-            comp[0] = (t - sum[0]) - y;
-            sum[0] = t;
-        }
+        // what is left (fewer than kReduceIlp slots), loaded together and added in order
+        float v[kReduceIlp];
+#pragma unroll
+        for (int u = 0; u < kReduceIlp; ++u)
+            v[u] = c + u * kReduceWarps < n_slots ? part_f[(size_t)(c + u * kReduceWarps) * nf + e] : 0.f;
+#pragma unroll
+        for (int u = 0; u < kReduceIlp; ++u)
+            if (c + u * kReduceWarps < n_slots) {
+                const float y = v[u] - comp[0];
+                const float t = sum[0] + y;
+                comp[0] = (t - sum[0]) - y;
+                sum[0] = t;
+            }
     }
     float wsum = 0.f;
 #pragma unroll
@@ -311,10 +318,252 @@ __device__ __forceinline__ void block_product(int m, int nu, int kn, Lf lf, Rf r
         }
 }
 
-// kLarge: the n > 32 instantiation (the 8 x 4 register Gauss-Jordan and the
-// blocked products); the n <= 32 one stays small, since each solve runs once
-// from a cold instruction cache.
-template <bool kLarge>
+// The same for n <= 32 (p <= 64), where the one CTA is bound by latency alone:
+// every global load is issued before anything waits for one (the used atoms are
+// gathered from shared memory), the elimination runs on two warps with 4 x 4
+// contiguous blocks (a pivot costs two 16-byte reads, one reciprocal and a 64-thread
+// barrier; its row, column and the pivot itself go through the same multiply-add
+// as the rest), and the objective and its FP64 arithmetic are formed only for a
+// caller that wants them.  Every value takes the operations of the general form in
+// their order.  SM cycles by phase at n = 24, p = 12 in the general form: loads
+// 5800, elimination 12270, D* 1610, objective 3290, norms 1140, scaling 2780, end 2240;
+// the kernel went from 22 to 8.4 us there and from 26 to 10.3 us at n = 32.
+constexpr int kSmallLd = 36;       // row stride of the small matrices (16-byte rows)
+constexpr int kSmallP = kMaxP;
+
+__device__ __forceinline__ void solve_small_body(const float* __restrict__ red_f, const double* __restrict__ red_d,
+                                                 float* D, int p, int n, float* __restrict__ norms,
+                                                 double inv_count, double* objective_out, double* rmse_out,
+                                                 int* err, float* G_out) {
+    __shared__ __align__(16) float Praw[32 * kSmallLd], A[32 * kSmallLd];   // P as given; P_u, then its inverse
+    __shared__ __align__(16) float Bc[kSmallP * kSmallLd], X[kSmallP * kSmallLd], Dn[kSmallP * kSmallLd];
+    __shared__ __align__(16) float rc[2][2][32];                            // pivot row | column, two buffers
+    __shared__ float nrm[32], d0[32];
+    __shared__ int idx[32], s_nu, s_fail;
+    __shared__ double s_red[kSolveThreadsSmall / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NW = kSolveThreadsSmall / 32;
+    const float* P = red_f;
+    const float* B = red_f + n * n;
+    // ---- all loads first: rows to warps, columns to lanes
+    {
+        float pv[32 / NW], bv[kSmallP / NW], dv[32 / NW][2];
+#pragma unroll
+        for (int u = 0; u < 32 / NW; ++u) {
+            const int r = warp + NW * u;
+            pv[u] = r < n && lane < n ? P[r * n + lane] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kSmallP / NW; ++u) {
+            const int r = warp + NW * u;
+            bv[u] = r < p && lane < n ? B[r * n + lane] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 32 / NW; ++u)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = warp + NW * u, r = lane + 32 * h;
+                dv[u][h] = c < n && r < p ? D[r + p * c] : 0.f;
+            }
+        if (tid == 0) s_fail = 0;
+#pragma unroll
+        for (int u = 0; u < 32 / NW; ++u) Praw[(warp + NW * u) * kSmallLd + lane] = pv[u];
+#pragma unroll
+        for (int u = 0; u < kSmallP / NW; ++u) X[(warp + NW * u) * kSmallLd + lane] = bv[u];   // B as given
+#pragma unroll
+        for (int u = 0; u < 32 / NW; ++u)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = warp + NW * u, r = lane + 32 * h;
+                Dn[r * kSmallLd + c] = dv[u][h];
+            }
+    }
+    __syncthreads();
+    // ---- used atoms (every warp finds them; warp 0 writes)
+    const float diag = lane < n ? Praw[lane * kSmallLd + lane] : 0.f;
+    const unsigned used = __ballot_sync(0xffffffffu, lane < n && diag > 0.f);
+    const int nu = __popc(used);
+    // the lane-th used atom (mostly all are used)
+    const int mine = nu == n ? lane : (int)__fns(used, 0, lane + 1);
+    if (warp == 0) {
+        const unsigned bad = __ballot_sync(0xffffffffu, lane < n && !isfinite(diag));
+        if (lane < nu) {
+            idx[lane] = mine;
+            d0[lane] = Praw[mine * kSmallLd + mine];
+        }
+        if (lane == 0) {
+            s_nu = nu;
+            if (bad) s_fail = SDL_ERR_NONFINITE;
+        }
+    }
+    int bad = 0;
+    {
+        const int c = lane < nu ? mine : 0;
+#pragma unroll
+        for (int u = 0; u < 32 / NW; ++u) {
+            const int r = warp + NW * u;
+            const int rr = __shfl_sync(0xffffffffu, mine, r);
+            const float v = r < nu && lane < nu ? Praw[rr * kSmallLd + c] : 0.f;
+            A[r * kSmallLd + lane] = v;
+            if (!isfinite(v)) bad = 1;
+        }
+        for (int r = warp; r < p; r += NW) {
+            const float v = lane < nu ? X[r * kSmallLd + c] : 0.f;
+            Bc[r * kSmallLd + lane] = v;
+            if (!isfinite(v)) bad = 1;
+        }
+    }
+    if (bad) s_fail = SDL_ERR_NONFINITE;
+    __syncthreads();
+
+    // ---- 1. Gauss-Jordan inverse of P_u, two warps: thread (ti, tj) of an 8 x 8
+    // grid owns rows 4 ti.. and columns 4 tj..
+    if (tid < 64 && s_fail == 0) {
+        const int ti = tid >> 3, tj = tid & 7;
+        float a[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float4 v = *reinterpret_cast<const float4*>(A + (4 * ti + r) * kSmallLd + 4 * tj);
+            a[r][0] = v.x; a[r][1] = v.y; a[r][2] = v.z; a[r][3] = v.w;
+        }
+        // row (register row q of its owners) and column of pivot k to buffer k & 1
+        auto publish = [&](int k, auto qc) {
+            constexpr int q = decltype(qc)::value;
+            if (ti == k >> 2) {
+                *reinterpret_cast<float4*>(&rc[k & 1][0][4 * tj]) = make_float4(a[q][0], a[q][1], a[q][2], a[q][3]);
+            }
+            if (tj == k >> 2) {
+                *reinterpret_cast<float4*>(&rc[k & 1][1][4 * ti]) = make_float4(a[0][q], a[1][q], a[2][q], a[3][q]);
+            }
+        };
+        publish(0, std::integral_constant<int, 0>{});
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        bool ok = true;
+        for (int k0 = 0; k0 < nu && ok; k0 += 4) {
+            unrolled_for<0, 4>([&](auto qc) {
+                constexpr int q = decltype(qc)::value;
+                const int k = k0 + q;
+                if (k >= nu || !ok) return;
+                const float4 rv = *reinterpret_cast<const float4*>(&rc[k & 1][0][4 * tj]);
+                const float4 cv = *reinterpret_cast<const float4*>(&rc[k & 1][1][4 * ti]);
+                const float piv = rc[k & 1][1][k];
+                if (!(piv > kSolvePivotRel * d0[k])) {
+                    ok = false;
+                    return;
+                }
+                const float inv = 1.f / piv;
+                const bool rk = ti == k >> 2, ck = tj == k >> 2;
+                float nf[4] = {-(cv.x * inv), -(cv.y * inv), -(cv.z * inv), -(cv.w * inv)};
+                float w[4] = {rv.x, rv.y, rv.z, rv.w};
+                // the pivot's row is row * inv, its column -column * inv, itself inv
+                if (rk) {
+                    nf[q] = inv;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) a[q][c] = 0.f;
+                }
+                if (ck) {
+                    w[q] = 1.f;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) a[r][q] = 0.f;
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) a[r][c] = fmaf(nf[r], w[c], a[r][c]);
+                if (k + 1 < nu) publish(k + 1, std::integral_constant<int, (q + 1) % 4>{});
+                asm volatile("bar.sync 1, 64;" ::: "memory");
+            });
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            *reinterpret_cast<float4*>(A + (4 * ti + r) * kSmallLd + 4 * tj) =
+                make_float4(a[r][0], a[r][1], a[r][2], a[r][3]);
+        if (!ok && tid == 0) s_fail = SDL_ERR_SINGULAR;
+    }
+    __syncthreads();
+    const bool ok_inv = s_fail == 0;
+    const bool want = objective_out || rmse_out;
+    double part = 0.0;
+    if (ok_inv) {
+        // ---- 2. D* rows: one chain per entry
+        for (int r = warp; r < p; r += NW)
+            if (lane < nu) {
+                float x = 0.f;
+#pragma unroll 8
+                for (int k = 0; k < nu; ++k) x = fmaf(Bc[r * kSmallLd + k], A[k * kSmallLd + lane], x);
+                X[r * kSmallLd + lane] = x;
+            }
+        __syncthreads();
+        // ---- 3. objective change (see solve_body)
+        if (want) {
+            for (int r = warp; r < p; r += NW)
+                if (lane < nu) {
+                    float w = -2.f * Bc[r * kSmallLd + lane];
+                    const float* prow = Praw + mine * kSmallLd;
+#pragma unroll 4
+                    for (int k = 0; k < nu; ++k)
+                        w = fmaf(prow[idx[k]], Dn[r * kSmallLd + idx[k]] + X[r * kSmallLd + k], w);
+                    part += (double)(X[r * kSmallLd + lane] - Dn[r * kSmallLd + mine]) * (double)w;
+                }
+        }
+        // ---- 4. column norms of D*
+        if (warp == 0 && lane < nu) {
+            float ss = 0.f;
+#pragma unroll 8
+            for (int r = 0; r < p; ++r) ss = fmaf(X[r * kSmallLd + lane], X[r * kSmallLd + lane], ss);
+            const float nr = sqrtf(ss);
+            nrm[lane] = nr;
+            if (!(nr > 0.f) || !isfinite(nr)) s_fail = SDL_ERR_SINGULAR;
+        }
+    }
+    if (want) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        if (lane == 0) s_red[warp] = part;
+    }
+    __syncthreads();
+    const bool ok = s_fail == 0;
+    if (warp == 0 && lane < n) {
+        const bool on = (used >> lane) & 1u;
+        norms[lane] = ok && on ? nrm[__popc(used & ((1u << lane) - 1u))] : 1.f;
+    }
+    if (ok) {
+        if (lane < nu) {
+            const float nr = nrm[lane];
+            for (int r = warp; r < p; r += NW) {
+                const float v = X[r * kSmallLd + lane] / nr;
+                Dn[r * kSmallLd + mine] = v;
+                D[r + p * mine] = v;
+            }
+        }
+        if (G_out) {
+            __syncthreads();
+            for (int i = warp; i < n; i += NW)
+                if (lane < n) {
+                    float g = 0.f;
+#pragma unroll 4
+                    for (int r = 0; r < p; ++r) g = fmaf(Dn[r * kSmallLd + i], Dn[r * kSmallLd + lane], g);
+                    G_out[i * n + lane] = g;
+                }
+        }
+    }
+    if (tid == 0) {
+        if (!ok) record_error(err, s_fail);
+        if (want) {
+            double change = 0.0;
+            for (int w = 0; w < NW; ++w) change += s_red[w];
+            const double before = red_d[0];
+            const double after = ok ? before + change : before;
+            if (objective_out) {
+                objective_out[0] = before;
+                objective_out[1] = after;
+            }
+            if (rmse_out) rmse_out[0] = sqrt(fmax(after, 0.0) * inv_count);
+        }
+    }
+}
+
+// n > 32: the 8 x 4 register Gauss-Jordan and the blocked products.
 __device__ __forceinline__ void solve_body(const float* __restrict__ red_f,
                                            const double* __restrict__ red_d, float* D, int p,
                                            int n, float* __restrict__ norms, double inv_count,
@@ -393,16 +642,9 @@ __device__ __forceinline__ void solve_body(const float* __restrict__ red_f,
     if (s_fail == 0) {
         bool ok;
         bool regs = false;
-        if constexpr (kLarge) {
-            if (nth == kSolveThreads && nu <= 128) {
-                ok = gj_inverse_regs<16, 32, 8, 4>(A, lda, nu, d0, A2);
-                regs = true;
-            }
-        } else {
-            if (nth == kSolveThreadsSmall && nu <= 32) {
-                ok = gj_inverse_regs<16, 16, 2, 2>(A, lda, nu, d0, A2);
-                regs = true;
-            }
+        if (nth == kSolveThreads && nu <= 128) {
+            ok = gj_inverse_regs<16, 32, 8, 4>(A, lda, nu, d0, A2);
+            regs = true;
         }
         if (!regs) {
             // any other size: in place through shared memory, the saved pivot
@@ -445,9 +687,8 @@ __device__ __forceinline__ void solve_body(const float* __restrict__ red_f,
     if (ok_inv) {
         // 2. D* rows: D*[a][c] = sum_k B[a][k] P_u^{-1}[k][c].  Few entries
         //    (p nu <= 2 threads): one chain per thread; else 4 x 4 blocks
-        const bool blocked = kLarge && nth == kSolveThreads && p * nu > 2 * nth;
-        if constexpr (kLarge) {
-            if (blocked)
+        const bool blocked = nth == kSolveThreads && p * nu > 2 * nth;
+        if (blocked) {
             block_product<16, 32>(
                 p, nu, nu, [&](int a, int k) { return Bc[a * lda + k]; },
                 [&](int k, int c) { return Ain[k * lda + c]; }, [](int, int) { return 0.f; },
@@ -475,8 +716,7 @@ __device__ __forceinline__ void solve_body(const float* __restrict__ red_f,
             __syncthreads();
             Pu = A;
         }
-        if constexpr (kLarge) {
-            if (blocked)
+        if (blocked) {
             block_product<16, 32>(
                 p, nu, nu, [&](int a, int k) { return Dn[a * lda + idx[k]] + X[a * lda + k]; },
                 [&](int k, int c) { return Pu[c * lda + k]; },
@@ -544,21 +784,27 @@ __device__ __forceinline__ void solve_body(const float* __restrict__ red_f,
 }
 
 template <bool kLarge>
-__global__ void __launch_bounds__(kSolveThreads)
+__global__ void __launch_bounds__(kLarge ? kSolveThreads : kSolveThreadsSmall)
     solve_kernel(const float* __restrict__ red_f, const double* __restrict__ red_d, float* D, int p,
                  int n, float* __restrict__ norms, double inv_count, double* objective_out,
                  double* rmse_out, int* err, float* G_out, int keep_p) {
-    solve_body<kLarge>(red_f, red_d, D, p, n, norms, inv_count, objective_out, rmse_out, err,
-                       G_out, keep_p);
+    if constexpr (kLarge)
+        solve_body(red_f, red_d, D, p, n, norms, inv_count, objective_out, rmse_out, err, G_out, keep_p);
+    else
+        solve_small_body(red_f, red_d, D, p, n, norms, inv_count, objective_out, rmse_out, err, G_out);
 }
 
 // One CTA per problem.
 template <bool kLarge>
-__global__ void __launch_bounds__(kSolveThreads) solve_multi_kernel(const SolveDesc* __restrict__ d,
-                                                                    int* err) {
+__global__ void __launch_bounds__(kLarge ? kSolveThreads : kSolveThreadsSmall)
+    solve_multi_kernel(const SolveDesc* __restrict__ d, int* err) {
     const SolveDesc q = d[blockIdx.x];
-    solve_body<kLarge>(q.red_f, q.red_d, q.D, q.p, q.n, q.norms, q.inv_count, q.objective_out, q.rmse_out,
-               err, q.G_out, q.keep_p);
+    if constexpr (kLarge)
+        solve_body(q.red_f, q.red_d, q.D, q.p, q.n, q.norms, q.inv_count, q.objective_out, q.rmse_out, err, q.G_out,
+                   q.keep_p);
+    else
+        solve_small_body(q.red_f, q.red_d, q.D, q.p, q.n, q.norms, q.inv_count, q.objective_out, q.rmse_out, err,
+                         q.G_out);
 }
 
 // FP64 version of solve_kernel (precision extension): the same steps with
@@ -794,13 +1040,15 @@ int launch_multi_update_kernels(int which, const void* d_desc, int G, int blocks
                 static_cast<const ReduceDesc*>(d_desc), G);
             break;
         case 2:
+            solve_multi_kernel<false><<<G, kSolveThreadsSmall, 0, st>>>(static_cast<const SolveDesc*>(d_desc), err);
+            break;
         case 4: {
-            // 4: some problem has n > 32
-            auto kern = which == 4 ? solve_multi_kernel<true> : solve_multi_kernel<false>;
+            // some problem has n > 32
+            auto kern = solve_multi_kernel<true>;
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
                 cudaSuccess)
                 return SDL_ERR_CUDA;
-            kern<<<G, which == 4 ? kSolveThreads : kSolveThreadsSmall, smem, st>>>(
+            kern<<<G, kSolveThreads, smem, st>>>(
                 static_cast<const SolveDesc*>(d_desc), err);
             break;
         }
@@ -851,14 +1099,19 @@ int launch_solve64(const float* red_f, const double* red_d, float* D, int p, int
 int launch_solve(const float* red_f, const double* red_d, float* D, int p, int n, float* norms,
                  double inv_count, double* objective_out, double* rmse_out, int* err,
                  cudaStream_t st, float* G_out) {
+    if (n <= 32) {
+        solve_kernel<false><<<1, kSolveThreadsSmall, 0, st>>>(red_f, red_d, D, p, n, norms, inv_count, objective_out,
+                                                              rmse_out, err, G_out, 0);
+        return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
+    }
     // keep a copy of P in shared memory for the objective term when it fits
     int keep_p = 0;
     const size_t bytes = solve_smem_bytes(p, n, &keep_p);
-    auto kern = n > 32 ? solve_kernel<true> : solve_kernel<false>;
+    auto kern = solve_kernel<true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
         cudaSuccess)
         return SDL_ERR_CUDA;
-    kern<<<1, n > 32 ? kSolveThreads : kSolveThreadsSmall, bytes, st>>>(red_f, red_d, D, p, n, norms, inv_count, objective_out,
+    kern<<<1, kSolveThreads, bytes, st>>>(red_f, red_d, D, p, n, norms, inv_count, objective_out,
                                             rmse_out, err, G_out, keep_p);
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
 }
