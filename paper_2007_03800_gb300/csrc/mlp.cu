@@ -39,9 +39,8 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// x = vec(Y_k)/||Y_k|| as BF16 rows (zero padded to Kp), optional transposed copy
-__global__ void prep_input_kernel(const float* __restrict__ Y, long long N, int P, int Kp,
-                                  bf16* __restrict__ X, int ldx, bf16* __restrict__ XT, int ldt) {
+// x = vec(Y_k)/||Y_k|| as BF16 rows (zero padded to Kp)
+__global__ void prep_input_kernel(const float* __restrict__ Y, long long N, int P, int Kp, bf16* __restrict__ X) {
     const long long k = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (k >= N) return;
@@ -53,8 +52,47 @@ __global__ void prep_input_kernel(const float* __restrict__ Y, long long N, int 
     const float inv = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
     for (int e = lane; e < Kp; e += 32) {
         const bf16 v = __float2bfloat16_rn(e < P ? y[e] * inv : 0.f);
-        X[(size_t)k * ldx + e] = v;
-        if (XT) XT[(size_t)e * ldt + k] = v;
+        X[(size_t)k * Kp + e] = v;
+    }
+}
+
+// The same rows for inference when p1 p2 is a multiple of 4 and Y is 16-byte aligned: 8 lanes
+// per signal, 16-byte loads and 8-byte stores, the norm in the same 32 chains and
+// order (lane j holds chains 4j .. 4j + 3); one square root per four signals.
+// 32 768 x 64: 7.4 us, 13 with a warp per signal (latency of 4-byte loads and of one
+// root per signal).
+__global__ void __launch_bounds__(256) prep_rows_kernel(const float* __restrict__ Y, long long N, int P, int Kp,
+                                                        bf16* __restrict__ X) {
+    const int lane = threadIdx.x & 31, j = lane & 7;
+    const long long k = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * 4 + (lane >> 3);
+    const float* src = Y + (size_t)k * P;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (k < N) {
+#pragma unroll 4
+        for (int e = 4 * j; e < P; e += 32) {
+            const float4 y = *reinterpret_cast<const float4*>(src + e);
+            v[0] = fmaf(y.x, y.x, v[0]);
+            v[1] = fmaf(y.y, y.y, v[1]);
+            v[2] = fmaf(y.z, y.z, v[2]);
+            v[3] = fmaf(y.w, y.w, v[3]);
+        }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] += __shfl_xor_sync(kFull, v[c], o);
+    const float ss = (v[0] + v[2]) + (v[1] + v[3]);
+    const float inv = ss > 0.f ? 1.f / sqrtf(ss) : 0.f;
+    if (k < N) {
+#pragma unroll 4
+        for (int e = 4 * j; e < Kp; e += 32) {
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e < P) y = *reinterpret_cast<const float4*>(src + e);   // still in L1
+            const __nv_bfloat162 a = __floats2bfloat162_rn(y.x * inv, y.y * inv);
+            const __nv_bfloat162 b = __floats2bfloat162_rn(y.z * inv, y.w * inv);
+            *reinterpret_cast<uint2*>(X + (size_t)k * Kp + e) =
+                make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b));
+        }
     }
 }
 
@@ -323,7 +361,7 @@ __global__ void topk_kernel(const float* __restrict__ Z, int ldz, long long N, i
     const unsigned m2 = k2 > k1 ? select(k2) & ~m1 : 0u;   // no check set: one bisection
     int base = 0;
     int32_t* o = out + (size_t)k * k2;
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0; pass < (k2 > k1 ? 2 : 1); ++pass) {
         const unsigned msk = pass == 0 ? m1 : m2;
         if (pass == 1) base = k1;
         int written = 0;
@@ -540,15 +578,21 @@ __global__ void count_flags_kernel(const int32_t* __restrict__ flag, long long N
 }
 
 __global__ void scan_counts_kernel(int* __restrict__ blockcnt, int nblocks, int* __restrict__ total) {
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int b = 0; b < nblocks; ++b) {
-            const int c = blockcnt[b];
-            blockcnt[b] = run;
-            run += c;
+    // one warp, 32 counts at a time
+    int run = 0;
+    for (int b0 = 0; b0 < nblocks; b0 += 32) {
+        const int b = b0 + (int)threadIdx.x;
+        const int c = b < nblocks ? blockcnt[b] : 0;
+        int s = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, s, o);
+            if ((int)threadIdx.x >= o) s += v;
         }
-        total[0] = run;
+        if (b < nblocks) blockcnt[b] = run + s - c;
+        run += __shfl_sync(kFull, s, 31);
     }
+    if (threadIdx.x == 0) total[0] = run;
 }
 
 __global__ void write_index_kernel(const int32_t* __restrict__ flag, long long N,
@@ -594,6 +638,7 @@ __global__ void __launch_bounds__(kGuardThreads)
                  int32_t* __restrict__ n_fallback, float* __restrict__ guard_out) {
     __shared__ double sp[kGuardThreads / 32], sl[kGuardThreads / 32];
     double a = 0.0, b = 0.0;
+#pragma unroll 4
     for (int r = threadIdx.x; r < m; r += blockDim.x) {
         a += (double)plainE[r];
         b += (double)learnedE[idx[r]];
@@ -851,7 +896,7 @@ int sdl_mlp_gradients(sdl_mlp* m, const float* Y, const int32_t* support, int s,
 
 // Inference runs in chunks of this many signals: a 4096-signal chunk leaves
 // every SM one 128 x 128 tile per GEMM, so that nothing hides the epilogue's GELU
-// (23 us per chunk at 64 -> 512; 8 times the signals take ...), while the
+// (23 us per chunk at 64 -> 512; 8 times the signals take 36 us), while the
 // activations and scores of a chunk still stay in L2.
 constexpr int64_t kInferChunk = 32768;
 
@@ -878,7 +923,10 @@ static int infer_rows(sdl_mlp* m, const float* Y, int64_t rows, bf16* Xb, bf16* 
                       cudaStream_t st) {
     sdl_ctx* c = m->ctx;
     const int H = m->H, Kp = m->Kp, Q = m->Q, B = (int)rows;
-    prep_input_kernel<<<blocks_for(rows * 32, 256), 256, 0, st>>>(Y, B, m->P, Kp, Xb, Kp, nullptr, 0);
+    if (m->P % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0)
+        prep_rows_kernel<<<blocks_for(rows * 8, 256), 256, 0, st>>>(Y, B, m->P, Kp, Xb);
+    else
+        prep_input_kernel<<<blocks_for(rows * 32, 256), 256, 0, st>>>(Y, B, m->P, Kp, Xb);
     const int rc = tc_gemm(Xb, Kp, m->W1b, Kp, B, H, Kp, 1.f, m->b1, 1, nullptr, 0, 0, Hb, H, nullptr, 0, nullptr,
                            0, c->err, st);
     if (rc) return rc;
