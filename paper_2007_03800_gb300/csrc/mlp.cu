@@ -377,188 +377,6 @@ __global__ void topk_kernel(const float* __restrict__ Z, int ldz, long long N, i
     }
 }
 
-// ---------------------------------------------------------------- shortlist OMP
-// fallback test: a signal whose final residual correlates with some
-// unselected pair more strongly than this fraction of its weakest greedy
-// score is coded again by the full coder
-constexpr float kCheckMargin = 0.7f;
-template <int B, int E, class F>
-__device__ __forceinline__ void sfor(F&& f) {
-    if constexpr (B < E) {
-        f(std::integral_constant<int, B>{});
-        sfor<B + 1, E>(f);
-    }
-}
-
-// 2D-OMP restricted to the k1 shortlisted pairs (lane l owns candidate l),
-// the same greedy rule, Cholesky and energy identity as the full coder.
-// Fallback test: after the last pick, the residual's correlation with every
-// pair not picked, C0 - sum_l x_l G1[:, i_l] G2[j_l, :]; if one exceeds
-// kCheckMargin x the weakest pick's score at its step, plain 2D-OMP might
-// have taken a pair the shortlist missed: the signal is flagged.
-template <int P1, int P2, int N1, int N2, int S>
-__global__ void __launch_bounds__(256) shortlist_omp_kernel(
-    const float* __restrict__ Y, long long N, const float* __restrict__ D1,
-    const float* __restrict__ D2, const float* __restrict__ G1, const float* __restrict__ G2,
-    const int32_t* __restrict__ cand, int k1, int k2, int32_t* __restrict__ support,
-    float* __restrict__ coef, int32_t* __restrict__ nnz, float* __restrict__ res_energy,
-    int32_t* __restrict__ flag) {
-    constexpr int PP = P1 * P2;
-    static_assert(N1 <= 32 && N2 <= 32, "one lane per atom, one bit per j");
-    __shared__ float D1c[N1 * P1];       // column i contiguous
-    __shared__ float D2r[P2 * N2];       // row b contiguous
-    __shared__ float G1s[N1 * N1], G2s[N2 * N2];
-    __shared__ float Ysh[8][PP];
-    __shared__ float Zsh[8][P1 * N2];
-    for (int e = threadIdx.x; e < N1 * P1; e += blockDim.x) D1c[e] = D1[e];
-    for (int e = threadIdx.x; e < P2 * N2; e += blockDim.x) {
-        const int b = e / N2, j = e % N2;
-        D2r[e] = D2[b + P2 * j];
-    }
-    for (int e = threadIdx.x; e < N1 * N1; e += blockDim.x) G1s[e] = G1[e];
-    for (int e = threadIdx.x; e < N2 * N2; e += blockDim.x) G2s[e] = G2[e];
-    __syncthreads();
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* Ys = Ysh[w];
-    float* Zs = Zsh[w];
-    const long long stride = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long k = (long long)blockIdx.x * (blockDim.x >> 5) + w; k < N; k += stride) {
-        float ss = 0.f;
-        for (int e = lane; e < PP; e += 32) {
-            const float v = Y[(size_t)k * PP + e];
-            Ys[e] = v;
-            ss = fmaf(v, v, ss);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(kFull, ss, o);
-        __syncwarp();
-        for (int e = lane; e < P1 * N2; e += 32) {
-            const int a = e / N2, j = e % N2;
-            float z = 0.f;
-#pragma unroll
-            for (int b = 0; b < P2; ++b) z = fmaf(Ys[a + P1 * b], D2r[b * N2 + j], z);
-            Zs[e] = z;
-        }
-        __syncwarp();
-        // lane's shortlist candidate
-        const int q = lane < k1 ? cand[(size_t)k * k2 + lane] : -1;
-        const int ci = q >= 0 ? q % N1 : 0, cj = q >= 0 ? q / N1 : 0;
-        float c0 = 0.f;
-#pragma unroll
-        for (int a = 0; a < P1; ++a) c0 = fmaf(D1c[ci * P1 + a], Zs[a * N2 + cj], c0);
-        if (q < 0) c0 = __int_as_float(0x7fc00000);
-        int si[S], sj[S];
-        float xs[S], yv[S], Lrow[S], Lcol[S];
-#pragma unroll
-        for (int m = 0; m < S; ++m) {
-            si[m] = 0; sj[m] = 0; xs[m] = 0.f; yv[m] = 0.f; Lrow[m] = 0.f; Lcol[m] = 0.f;
-        }
-        float myinvd = 0.f, myy = 0.f, myx = 0.f;
-        int myi = 0, myj = 0, cnt = 0;
-        float E2 = ss, weakest = INFINITY;
-        bool go = isfinite(ss);
-        sfor<0, S>([&](auto tc) {
-            constexpr int t = decltype(tc)::value;
-            if (!go) return;
-            float sc = c0;
-#pragma unroll
-            for (int l = 0; l < t; ++l)
-                sc = fmaf(-xs[l] * G1s[ci * N1 + si[l]], G2s[sj[l] * N2 + cj], sc);
-            const float v = fabsf(sc);
-            const float vv = (v == v) ? v : 0.f;             // masked / padding lanes: NaN
-            const unsigned M = __reduce_max_sync(kFull, __float_as_uint(vv));
-            if (M == 0u) { go = false; return; }
-            const unsigned cq = (__float_as_uint(vv) == M && q >= 0) ? (unsigned)q : 0xffffffffu;
-            const unsigned qs = __reduce_min_sync(kFull, cq);
-            const int owner = __ffs(__ballot_sync(kFull, (unsigned)q == qs)) - 1;
-            const float b = __shfl_sync(kFull, c0, owner);
-            if (lane == owner) c0 = __int_as_float(0x7fc00000);
-            const int it = (int)(qs % N1), jt = (int)(qs / N1);
-            float r = 0.f;
-            if (lane < t) r = G1s[it * N1 + myi] * G2s[jt * N2 + myj];
-            const float Att = G1s[it * N1 + it] * G2s[jt * N2 + jt];
-            float ww = 0.f, wy = 0.f;
-#pragma unroll
-            for (int m = 0; m < t; ++m) {
-                const float wm = __shfl_sync(kFull, r * myinvd, m);
-                r = fmaf(-Lrow[m], wm, r);
-                ww = fmaf(wm, wm, ww);
-                wy = fmaf(wm, yv[m], wy);
-                if (lane == t) Lrow[m] = wm;
-                if (lane == m) Lcol[t] = wm;
-            }
-            const float d = Att - ww;
-            if (!(d > kPivotRel * Att)) { go = false; return; }
-            const float inv = rsqrtf(d);
-            const float yt = (b - wy) * inv;
-            yv[t] = yt;
-            si[t] = it;
-            sj[t] = jt;
-            if (lane == t) {
-                Lrow[t] = d * inv;
-                myinvd = inv;
-                myy = yt;
-                myi = it;
-                myj = jt;
-            }
-            float rb = myy;
-#pragma unroll
-            for (int kk = t; kk >= 0; --kk) {
-                const float xk = __shfl_sync(kFull, rb * myinvd, kk);
-                rb = fmaf(-Lcol[kk], xk, rb);
-                xs[kk] = xk;
-            }
-            E2 = fmaf(-yt, yt, E2);
-            weakest = fminf(weakest, __uint_as_float(M));
-            cnt = t + 1;
-        });
-#pragma unroll
-        for (int m = 0; m < S; ++m)
-            if (lane == m) myx = xs[m];
-        // fallback test over every pair not picked: lane = atom i (two lanes
-        // per atom, on alternate j, when N1 <= 16), its column of D1 and its
-        // factors -x_l G1[i, i_l] in registers; the maximum does not depend on
-        // the order of the pairs
-        float ve = 0.f;
-        if (cnt == S) {
-            constexpr int LJ = N1 <= 16 ? 2 : 1;
-            const int i = lane % (32 / LJ), j0 = lane / (32 / LJ);
-            if (i < N1) {
-                float d[P1], gx[S];
-                unsigned pm = 0;   // the picked j of this atom
-#pragma unroll
-                for (int a = 0; a < P1; ++a) d[a] = D1c[i * P1 + a];
-#pragma unroll
-                for (int l = 0; l < S; ++l) {
-                    gx[l] = -xs[l] * G1s[i * N1 + si[l]];
-                    pm |= (si[l] == i ? 1u : 0u) << sj[l];
-                }
-#pragma unroll 4
-                for (int j = j0; j < N2; j += LJ) {
-                    float sce = 0.f;
-#pragma unroll
-                    for (int a = 0; a < P1; ++a) sce = fmaf(d[a], Zs[a * N2 + j], sce);
-#pragma unroll
-                    for (int l = 0; l < S; ++l) sce = fmaf(gx[l], G2s[sj[l] * N2 + j], sce);
-                    if (!((pm >> j) & 1u)) ve = fmaxf(ve, fabsf(sce));
-                }
-            }
-        }
-        const float maxe = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(ve)));
-        const bool fb = !isfinite(ss) || (cnt == S && maxe > kCheckMargin * weakest);
-        if (lane < S) {
-            support[(size_t)k * S + lane] = lane < cnt ? myi + N1 * myj : -1;
-            coef[(size_t)k * S + lane] = lane < cnt ? myx : 0.f;
-        }
-        if (lane == 0) {
-            nnz[k] = cnt;
-            if (res_energy) res_energy[k] = fmaxf(E2, 0.f);
-            flag[k] = fb ? 1 : 0;
-        }
-        __syncwarp();
-    }
-}
-
 // ---------------------------------------------------------------- compaction
 constexpr int kScanBlock = 1024;
 
@@ -965,16 +783,30 @@ int sdl_mlp_forward(sdl_mlp* m, const float* Y, int64_t N, float* scores, void* 
 // ------------------------------------------------------------ learned coder
 namespace {
 
-template <int P1, int P2, int N1, int N2, int S>
-int launch_shortlist(const float* Y, long long N, const float* D1, const float* D2, const float* G1,
-                     const float* G2, const int32_t* cand, int k1, int k2, int32_t* support,
-                     float* coef, int32_t* nnz, float* res, int32_t* flag, int num_sms,
-                     cudaStream_t st) {
-    const long long need = (N + 7) / 8;
-    const int grid = (int)std::max<long long>(1, std::min<long long>(need, (long long)num_sms * 8));
-    shortlist_omp_kernel<P1, P2, N1, N2, S><<<grid, 256, 0, st>>>(Y, N, D1, D2, G1, G2, cand, k1, k2,
-                                                                  support, coef, nnz, res, flag);
-    return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
+// 2D-OMP on the shortlists and the fallback flags
+int launch_shortlist(const float* Y, int p1, int p2, long long N, const float* D1, int n1, const float* D2, int n2,
+                     int s, const int32_t* cand, int k1, int k2, int32_t* support, float* coef, int32_t* nnz,
+                     float* res, int32_t* flag, int num_sms, cudaStream_t st) {
+    PassArgs a{};
+    a.Y = Y;
+    a.p1 = p1;
+    a.p2 = p2;
+    a.N = N;
+    a.D1 = D1;
+    a.D2 = D2;
+    a.n1 = n1;
+    a.n2 = n2;
+    a.s = s;
+    a.support = support;
+    a.coef = coef;
+    a.nnz = nnz;
+    a.res_energy = res;
+    a.n_slots = 1;
+    a.cand = cand;
+    a.cand_k = k1;
+    a.cand_ld = k2;
+    a.flag = flag;
+    return launch_code_group_short(a, st, num_sms);
 }
 
 }  // namespace
@@ -994,13 +826,13 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     DeviceGuard guard(c->device);
     cudaStream_t st = (cudaStream_t)stream;
     const int k2 = k, Q = m->Q;     // the shortlist only: the fallback test scans every pair
-    // workspace: scores of one chunk, candidates, Grams, scan buffers, index list
+    // workspace: scores of one chunk, candidates, scan buffers, index list
     const long long chunk = std::max<long long>(m->Bmax, std::min<long long>(N, kInferChunk));
     const int nblk = (int)((N + kScanBlock - 1) / kScanBlock);
     const long long m_s = std::min<long long>(N, std::max<long long>(kGuardMinSample, N / 16));
     const long long stride_s = N / m_s;
     const size_t need = sizeof(float) * (size_t)chunk * Q + sizeof(int32_t) * (size_t)N * k2 +
-                        sizeof(float) * (size_t)(n1 * n1 + n2 * n2) + sizeof(int) * (nblk + 8) +
+                        sizeof(int) * (nblk + 8) +
                         sizeof(int32_t) * (size_t)N + sizeof(int32_t) * (size_t)m_s +
                         sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + 10 * 256 +
                         infer_bytes(m, chunk);
@@ -1009,8 +841,6 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     char* p = c->learn;
     float* scores = carve<float>(p, (size_t)chunk * Q);
     int32_t* cand = carve<int32_t>(p, (size_t)N * k2);
-    float* G1 = carve<float>(p, (size_t)n1 * n1);
-    float* G2 = carve<float>(p, (size_t)n2 * n2);
     int* blockcnt = carve<int>(p, nblk + 8);
     int32_t* idx = carve<int32_t>(p, (size_t)N);
     int32_t* idx_s = carve<int32_t>(p, (size_t)m_s);
@@ -1019,10 +849,6 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     int* cnt_s = carve<int>(p, 2);
     bf16* Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
     bf16* Hb = carve<bf16>(p, (size_t)chunk * m->H);
-    {
-        Trace tr(c, kGram, st);
-        launch_gram2(D1, p1, n1, G1, D2, p2, n2, G2, st);
-    }
     // 1. scores and shortlists, chunk by chunk
     for (int64_t r0 = 0; r0 < N; r0 += chunk) {
         const int B = (int)std::min<int64_t>(chunk, N - r0);
@@ -1044,12 +870,8 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     // 2. 2D-OMP on the shortlists, with the fallback test
     {
         Trace tr(c, kShortlist, st);
-        rc = shape_a ? launch_shortlist<12, 12, 24, 24, 6>(Y, N, D1, D2, G1, G2, cand, k, k2, support,
-                                                          coef, nnz, learnedE, fallback,
-                                                          c->num_sms, st)
-                     : launch_shortlist<8, 8, 16, 16, 4>(Y, N, D1, D2, G1, G2, cand, k, k2, support,
-                                                        coef, nnz, learnedE, fallback, c->num_sms,
-                                                        st);
+        rc = launch_shortlist(Y, p1, p2, N, D1, n1, D2, n2, s_max, cand, k, k2, support, coef, nnz, learnedE, fallback,
+                              c->num_sms, st);
         if (rc) return rc;
     }
     // 3. compact the flagged signals (fixed order) and re-code them with the full coder
@@ -1063,8 +885,6 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     a.N = N;
     a.D1 = D1;
     a.D2 = D2;
-    a.G1 = G1;
-    a.G2 = G2;
     a.n1 = n1;
     a.n2 = n2;
     a.s = s_max;
@@ -1144,17 +964,7 @@ extern "C" int sdl_sparse_code_shortlist(sdl_ctx* c, const float* Y, int p1, int
     if (!Y || !cand || !support || !coef || !nnz || !flag) return SDL_ERR_ARG;
     DeviceGuard guard(c->device);
     cudaStream_t st = (cudaStream_t)stream;
-    int rc = ctx_workspace(c, p1, p2, n1, n2);
-    if (rc) return rc;
-    {
-        Trace tr(c, kGram, st);
-        launch_gram2(D1, p1, n1, c->G1, D2, p2, n2, c->G2, st);
-    }
     Trace tr(c, kShortlist, st);
-    return shape_a ? launch_shortlist<12, 12, 24, 24, 6>(Y, N, D1, D2, c->G1, c->G2, cand, k1, k2,
-                                                         support, coef, nnz, res_energy, flag,
-                                                         c->num_sms, st)
-                   : launch_shortlist<8, 8, 16, 16, 4>(Y, N, D1, D2, c->G1, c->G2, cand, k1, k2,
-                                                       support, coef, nnz, res_energy, flag,
-                                                       c->num_sms, st);
+    return launch_shortlist(Y, p1, p2, N, D1, n1, D2, n2, s_max, cand, k1, k2, support, coef, nnz, res_energy, flag,
+                            c->num_sms, st);
 }

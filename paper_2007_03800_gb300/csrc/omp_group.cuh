@@ -47,23 +47,32 @@ __host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
 // correlation and leaves the others alone) with ||Y||^2 in that many chains.
 template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,
           int P2_ = 0, int N1_ = 0, int N2_ = 0, int S_ = 0, int ORTHO_ = 0, int CHAINS_ = 32,
-          bool TM_ = false>
+          bool TM_ = false, bool SHORT_ = false>
 struct Cfg {
     // the C0 blocks live in tensor memory instead of shared memory: they are read
     // back whole every step, at a bandwidth of its own, and leave the shared memory
     // to more signals in flight (one signal per warp or team, 8 x 8 blocks)
     static constexpr bool kTM = TM_;
-    static constexpr int TUSED = kTM ? WARPS_ / 4 * RI_ * RJ_ : 0;
+    // picks from a list of candidates only (the others are masked in the C0 blocks),
+    // then a scan of all pairs, whose correlations wait in tensor memory meanwhile.
+    // A rank-one update scales its G1 row, and the back substitution runs down the rows.
+    static constexpr bool kShort = SHORT_;
+    static constexpr bool kTmem = kTM || kShort;
+    static constexpr bool kAsc = FAST_ && !SHORT_;
+    static constexpr int MW = (RI_ * RJ_ + 31) / 32;   // words of a lane's candidate marks
+    static constexpr int TUSED = kTmem ? WARPS_ / 4 * RI_ * RJ_ : 0;
     static constexpr int TCOLS = TUSED <= 64 ? TUSED : TUSED <= 128 ? 128 : TUSED <= 256 ? 256 : 512;   // of a CTA
-    static_assert(!kTM || (GL_ >= 32 && RI_ == 8 && RJ_ == 8 && WARPS_ % 4 == 0 && (TCOLS & (TCOLS - 1)) == 0 &&
-                           TCOLS >= 32 && TCOLS * MINB_ <= 512),
+    static_assert(!kTM || (GL_ >= 32 && RI_ == 8 && RJ_ == 8), "one signal per warp");
+    static_assert(!kShort || (GL_ <= 32 && RI_ * RJ_ % 8 == 0 && FAST_ && N1_ > 0 && ORTHO_ == 0 && !TM_), "shortlists");
+    static_assert(!kTmem || (WARPS_ % 4 == 0 && (TCOLS & (TCOLS - 1)) == 0 && TCOLS >= 32 && TCOLS * MINB_ <= 512),
                   "tensor memory");
     static constexpr bool kOrtho = ORTHO_ > 0;
     static constexpr int CHAINS = ORTHO_ > 0 ? ORTHO_ : CHAINS_;   // of ||Y||^2 (128: four warps' worth)
     static constexpr int CPL = CHAINS / GL_;                       // per lane
     // a group of 64 lanes is a team of two warps that meet at a named barrier
     static constexpr int TW = GL_ > 32 ? GL_ / 32 : 1;
-    static constexpr int XS = TW > 1 ? 16 : 0;                     // exchange slots between them
+    // exchange slots between them; or the candidates (32) and the lanes' marks
+    static constexpr int XS = TW > 1 ? 16 : kShort ? 32 + up4(GL_ * MW) : 0;
     static_assert(CHAINS == 128 || CPL == 1 || CPL == 2 || CPL == 4, "chains");
     static_assert(TW == 1 || CHAINS == 128, "a team's chains");
     static constexpr int GL = GL_, LI = LI_, LJ = GL_ / LI_, RI = RI_, RJ = RJ_;
@@ -123,7 +132,7 @@ __host__ __device__ inline Layout layout(int p1, int p2, int s, int warps) {
     // same offsets together
     while (st % 32 != 8 && st % 32 != 24) st += 4;
     L.sig_stride = st;
-    L.total = L.warp0 + warps * 32 / C::GL * st + (C::kTM ? 4 : 0);   // (the tensor-memory address)
+    L.total = L.warp0 + warps * 32 / C::GL * st + (C::kTmem ? 4 : 0);   // (the tensor-memory address)
     return L;
 }
 
@@ -231,6 +240,19 @@ __device__ __forceinline__ void tm_ld32(unsigned ta, float* v) {
         : "r"(ta));
 }
 
+template <int E>
+__device__ __forceinline__ void tm_ld_block(unsigned ta, float (&v)[E]) {
+#pragma unroll
+    for (int k = 0; k + 32 <= E; k += 32) tm_ld32(ta + k, v + k);
+#pragma unroll
+    for (int k = E & ~31; k < E; k += 8) tm_ld8(ta + k, v + k);
+}
+template <int E>
+__device__ __forceinline__ void tm_st_block(unsigned ta, const float (&v)[E]) {
+#pragma unroll
+    for (int k = 0; k < E; k += 8) tm_st8(ta + k, v + k);
+}
+
 // One pick of a signal: its coefficient, and the offsets of its rows of G1
 // (low half) and G2 (high half) in shared memory, one 8-byte load.
 struct alignas(8) Rec {
@@ -240,11 +262,17 @@ struct alignas(8) Rec {
     __device__ __forceinline__ int o2() const { return (int)(o >> 16); }
 };
 
+// A signal whose final residual correlates with some unpicked pair more strongly
+// than this fraction of its weakest greedy score is flagged: plain 2D-OMP might
+// have taken a pair that the shortlist missed.
+constexpr float kCheckMargin = 0.7f;
+
 // One greedy step's Cholesky row T and the coefficients of the T + 1 picks
 // (every lane of the signal holds the same values; `writer` stores them).
 // Returns false (state untouched) when the pick is degenerate or !live.
 // gram(r): the product of the Gram entries of the new pick and pick r.
-template <int T, bool kFast, class Gram>
+// kAsc: back substitution in increasing row order.
+template <int T, bool kFast, bool kAsc = kFast, class Gram>
 __device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, float* lf, float* iv, float* yv,
                                           Gram gram, float Att, float b, const Rec& pick, float& E) {
     constexpr int NL = T * (T - 1) / 2;
@@ -285,7 +313,7 @@ __device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, floa
 #pragma unroll
     for (int k = T - 1; k >= 0; --k) {
         float v = yo[k];
-        if constexpr (kFast) {
+        if constexpr (kAsc) {
 #pragma unroll
             for (int l = k + 1; l < T; ++l) v = fmaf(-L[l * (l - 1) / 2 + k], x[l], v);
             v = fmaf(-w[k], x[T], v);
@@ -460,6 +488,10 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
     // a signal's records start valid: a finished signal's lanes run along with
     // the others of the warp on whatever its records hold
     for (int l = gl; l < s; l += GL) rec[l] = Rec{0.f, 0u};
+    int* cands = reinterpret_cast<int*>(sb + L.xs);          // shortlists only
+    unsigned* marks = reinterpret_cast<unsigned*>(sb + L.xs + 32);
+    if constexpr (C::kShort)
+        for (int m = 0; m < C::MW; ++m) marks[gl * C::MW + m] = 0u;
     __syncthreads();
     if constexpr (!C::kOrtho) {
         gram<RI, RIP, C::N1P, LD1>(D1s, p1, G1s);
@@ -470,7 +502,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
     // tensor memory of the CTA, and this warp's place in it
     unsigned tbase = 0, tmine = 0;
     unsigned* tslot = reinterpret_cast<unsigned*>(sm + L.total - 4);
-    if constexpr (C::kTM) {
+    if constexpr (C::kTmem) {
         if (w == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sptr(tslot)),
                          "r"(C::TCOLS)
@@ -501,6 +533,10 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 cp4(Ys + b * p1s + (e - b * p1), src + e);
             }
         }
+        if constexpr (C::kShort)
+            for (int c = gl; c < a.cand_k; c += GL)
+                cp4(reinterpret_cast<float*>(cands + c),
+                    reinterpret_cast<const float*>(a.cand + (size_t)k * a.cand_ld + c));
     };
 
     float es = 0.f, ec = 0.f;      // this lane's residual-energy sum (compensated)
@@ -519,6 +555,13 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
         const long long ko = !act ? 0 : (a.idx && !a.idx_compact) ? (long long)a.idx[pos] : pos;
         cp_wait();
         sync();
+        if constexpr (C::kShort) {   // a mark for each candidate, with the lane that owns its entry
+            for (int c = gl; c < (act ? a.cand_k : 0); c += GL) {
+                const int q = cands[c], i = q % C::N1, j = q / C::N1, e = j % RJ * RI + i % RI;
+                if (q >= 0 && j < C::N2)
+                    atomicOr(marks + (j / RJ * LI + i / RI) * C::MW + e / 32, 1u << (e % 32));
+            }
+        }
         // ---- ||Y||^2: the strided partial sums of the one-signal-per-warp (or half
         // warp) coders (this lane takes CPL of them) and their combining tree
         float part[C::CPL];
@@ -651,18 +694,38 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     if (li * RI + r >= n1 || lj * RJ + c >= n2) sc[c * RI + r] = __int_as_float(0x7fc00000);
         }
         sync();   // every lane has read Z: its place takes the C0 blocks
-        if constexpr (C::kTM) {
-#pragma unroll
-            for (int e = 0; e < E; e += 8) tm_st8(tmine + e, sc + e);
+        if constexpr (C::kTmem) {
+            tm_st_block<E>(tmine, sc);
             tm_wait_st();
-        } else {
+        }
+        if constexpr (C::kShort) {   // only the candidates stay
+#pragma unroll
+            for (int m = 0; m < C::MW; ++m) {
+                const unsigned mk = marks[gl * C::MW + m];
+                marks[gl * C::MW + m] = 0u;
+#pragma unroll
+                for (int e = 32 * m; e < (32 * m + 32 < E ? 32 * m + 32 : E); ++e)
+                    if (!((mk >> (e - 32 * m)) & 1u)) sc[e] = __int_as_float(0x7fc00000);
+            }
+        }
+        if constexpr (!C::kTM) {
             st<E>(myc0, sc);
             sync();
         }
 
+        // a pick's coefficient goes to one of its two rows
+        auto scale = [&](float (&x)[RI], float (&v)[RJ], float f) {
+            if constexpr (C::kShort) {
+#pragma unroll
+                for (int r = 0; r < RI; ++r) x[r] *= -f;
+            } else {
+#pragma unroll
+                for (int c = 0; c < RJ; ++c) v[c] *= -f;
+            }
+        };
         // ---- greedy steps
         int cnt = 0;
-        float E2 = ss;
+        float E2 = ss, weakest = __int_as_float(0x7f800000);   // (the smallest score of a pick)
         float* masked = nullptr;
 #pragma unroll 1
         for (int t = 0; t < s; ++t) {
@@ -673,9 +736,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 // every lane has read the entry
                 if constexpr (C::kTM) {
                     __syncwarp();
-                    static_assert(!C::kTM || E == 64, "block");
-                    tm_ld32(tmine, sc);
-                    tm_ld32(tmine + 32, sc + (C::kTM ? 32 : 0));
+                    tm_ld_block<E>(tmine, sc);
                     tm_wait_ld();
                 } else {
                     if (masked) *masked = __int_as_float(0x7fc00000);
@@ -687,8 +748,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     float x[RI], v[RJ];
                     ld<RI>(x, G1s + r.o1() + li * RIP);
                     ld<RJ>(v, G2s + r.o2() + lj * RJP);
-#pragma unroll
-                    for (int c = 0; c < RJ; ++c) v[c] *= -r.x;
+                    scale(x, v, r.x);
                     rank1<RI, RJ>(sc, x, v);
                 }
             }
@@ -788,7 +848,7 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             } else {
             auto gram = [&](const Rec& r) { return G1s[r.o1() + c1] * G2s[r.o2() + c2]; };
             auto step = [&](auto tc) {
-                ok = chol_step<decltype(tc)::value, C::kFast>(pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
+                ok = chol_step<decltype(tc)::value, C::kFast, C::kAsc>(pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
             };
             switch (t) {
                 case 0: step(std::integral_constant<int, 0>{}); break;
@@ -818,8 +878,41 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             }
             }
             if (ok) cnt = t + 1;
+            if (C::kShort && ok) weakest = fminf(weakest, M);
             go = ok;
             sync();   // the step's state is visible
+        }
+
+        // ---- the scan after a full shortlist code: the largest correlation of the
+        // residual with a pair that was not picked
+        float left = 0.f;
+        if constexpr (C::kShort) {
+            if (any(act && cnt == s)) {
+                __syncwarp();
+                tm_ld_block<E>(tmine, sc);
+                tm_wait_ld();
+                unsigned picked[C::MW] = {};
+#pragma unroll 1
+                for (int l = 0; l < s; ++l) {
+                    const Rec r = rec[l];
+                    float x[RI], v[RJ];
+                    ld<RI>(x, G1s + r.o1() + li * RIP);
+                    ld<RJ>(v, G2s + r.o2() + lj * RJP);
+                    scale(x, v, r.x);
+                    rank1<RI, RJ>(sc, x, v);
+                    const int i = r.o1() / LD1, j = r.o2() / LD2, e = j % RJ * RI + i % RI;
+#pragma unroll
+                    for (int m = 0; m < C::MW; ++m)
+                        if (i / RI == li && j / RJ == lj && e / 32 == m) picked[m] |= 1u << (e % 32);
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if ((picked[e / 32] >> (e % 32)) & 1u) sc[e] = 0.f;
+#pragma unroll
+                for (int e = 0; e < E; e += 2) left = max3abs(left, sc[e], sc[e + 1]);
+#pragma unroll
+                for (int o = GL / 2; o > 0; o >>= 1) left = fmaxf(left, __shfl_xor_sync(kFull, left, o));
+            }
         }
 
         // ---- the code
@@ -833,16 +926,20 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
             if (gl == 0) {
                 const float e = fmaxf(E2, 0.f);
                 if (a.nnz) a.nnz[ko] = cnt;
-                if (a.res_energy) a.res_energy[ko] = finite ? e : __int_as_float(0x7fc00000);
-                if (finite) ksum(es, ec, e);
-                else record_error(a.err, SDL_ERR_NONFINITE);
+                if (a.res_energy) a.res_energy[ko] = finite || C::kShort ? e : __int_as_float(0x7fc00000);
+                if constexpr (C::kShort) {   // (a flagged signal is coded again)
+                    a.flag[ko] = !finite || (cnt == s && left > kCheckMargin * weakest) ? 1 : 0;
+                } else {
+                    if (finite) ksum(es, ec, e);
+                    else record_error(a.err, SDL_ERR_NONFINITE);
+                }
             }
         }
         sync();   // records are read before the next unit writes them
         pos = pos_next;
     }
 
-    if constexpr (C::kTM) {
+    if constexpr (C::kTmem) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (w == 0) {

@@ -69,6 +69,11 @@ struct PassArgs {
     // [esum_slots][2] (entry 0; slots past its grid and entries 1 are cleared)
     double* esum;
     int esum_slots;
+    // shortlist coder only: the pairs that signal k may use (the first cand_k <= 32 of
+    // cand_ld entries, negative: none), and a flag per signal to code it again
+    const int32_t* cand;
+    int cand_k, cand_ld;
+    int32_t* flag;
 };
 
 // Host launchers (omp_pass.cu).  They return the number of partial-sum
@@ -83,9 +88,11 @@ int launch_accumulate_pass(const PassArgs& a, int side, cudaStream_t st, int num
 // omp_group_*.cu: code-only passes with 8 or 16 lanes per signal, in the
 // arithmetic of the compiled tilings (fixed: their shapes; w_first: correlations
 // as (D1^T Y) D2, at most max_grid CTAs) or of the generic kernel (any: n1 <= 32,
-// n2 <= 128).  SDL_ERR_UNSUPPORTED for other shapes.
+// n2 <= 128).  short: picks from candidate lists (8x8 and 12x12 signals).
+// SDL_ERR_UNSUPPORTED for other shapes.
 int launch_code_group_fixed(const PassArgs& a, bool w_first, cudaStream_t st, int num_sms,
                             int max_grid = 0);
+int launch_code_group_short(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_any(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_cols(const PassArgs& a, cudaStream_t st, int num_sms);
