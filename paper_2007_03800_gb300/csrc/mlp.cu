@@ -313,15 +313,24 @@ __global__ void topk_kernel(const float* __restrict__ Z, int ldz, long long N, i
         for (int e = 0; e < EQ; ++e) c += key[e] >= t ? 1 : 0;
         return (int)__reduce_add_sync(kFull, (unsigned)c);
     };
-    // largest threshold with at least kk keys >= it, or the first one met with
-    // exactly kk: then no key ties for the last place, and the set is the same
+    // At least 32 keys reach the smallest of the lanes' maxima: the search for up to
+    // 32 of them starts there and ends at the largest key (256 scores, k = 32:
+    // 28 -> 23 us per 32 768 signals against bisecting all 17 bits).
+    unsigned top = key[0];
+#pragma unroll
+    for (int e = 1; e < EQ; ++e) top = max(top, key[e]);
+    const unsigned low = __reduce_min_sync(kFull, top);
+    top = __reduce_max_sync(kFull, top);
+    // largest threshold with at least kk keys >= it (0: there are fewer), or the first
+    // one met with exactly kk: then no key ties for the last place, and the set is the same
     auto threshold = [&](int kk, bool& exact) {
-        unsigned t = 0;
+        unsigned t = kk <= 32 ? low : 0u, hi = top;
         exact = false;
-        for (int bit = 16; bit >= 0; --bit) {
-            const unsigned c = t | (1u << bit);
+        while (t < hi) {
+            const unsigned c = (t + hi + 1u) >> 1;
             const int n = count_ge(c);
             if (n >= kk) t = c;
+            else hi = c - 1u;
             if (n == kk) {
                 exact = true;
                 break;
@@ -439,7 +448,7 @@ __global__ void write_index_kernel(const int32_t* __restrict__ flag, long long N
 // if the learned codes' RMSE there exceeds the plain coder's by more than 1 %,
 // every signal is coded again by the plain coder.
 constexpr double kGuardRmseRatio = 1.01;
-constexpr int kGuardThreads = 1024;
+constexpr int kGuardThreads = 256;
 constexpr long long kGuardMinSample = 4096;
 
 __global__ void sample_index_kernel(int32_t* __restrict__ idx, int m, long long stride,
@@ -449,15 +458,16 @@ __global__ void sample_index_kernel(int32_t* __restrict__ idx, int m, long long 
     if (r == 0) *count = m;
 }
 
-// fixed-order FP64 sums of the two residual energies over the sample
+// Fixed-order FP64 sums of the two residual energies over the sample, a pair per CTA
+// (one CTA alone spends 24 us on 2 x 12 500 of them, FP64 adds at one SM's rate; 13 us
+// with the verdict in a launch of its own).
+constexpr int kGuardCtas = 64;
 __global__ void __launch_bounds__(kGuardThreads)
-    guard_kernel(const float* __restrict__ plainE, const float* __restrict__ learnedE,
-                 const int32_t* __restrict__ idx, int m, long long N, int P, int* __restrict__ recode_count,
-                 int32_t* __restrict__ n_fallback, float* __restrict__ guard_out) {
+    guard_sums_kernel(const float* __restrict__ plainE, const float* __restrict__ learnedE,
+                      const int32_t* __restrict__ idx, int m, double2* __restrict__ part) {
     __shared__ double sp[kGuardThreads / 32], sl[kGuardThreads / 32];
     double a = 0.0, b = 0.0;
-#pragma unroll 4
-    for (int r = threadIdx.x; r < m; r += blockDim.x) {
+    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += (long long)gridDim.x * blockDim.x) {
         a += (double)plainE[r];
         b += (double)learnedE[idx[r]];
     }
@@ -477,6 +487,24 @@ __global__ void __launch_bounds__(kGuardThreads)
             ta += sp[w];
             tb += sl[w];
         }
+        part[blockIdx.x] = make_double2(ta, tb);
+    }
+}
+
+// one warp: the verdict from the kGuardCtas pairs
+__global__ void guard_kernel(const double2* __restrict__ part, int m, long long N, int P, int* __restrict__ recode_count,
+                             int32_t* __restrict__ n_fallback, float* __restrict__ guard_out) {
+    double ta = 0.0, tb = 0.0;
+    for (int c = threadIdx.x; c < kGuardCtas; c += 32) {
+        ta += part[c].x;
+        tb += part[c].y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ta += __shfl_down_sync(kFull, ta, o);
+        tb += __shfl_down_sync(kFull, tb, o);
+    }
+    if (threadIdx.x == 0) {
         const bool fail = tb > kGuardRmseRatio * kGuardRmseRatio * ta;
         *recode_count = fail ? (int)N : 0;
         if (fail) *n_fallback = (int32_t)N;
@@ -834,7 +862,8 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     const size_t need = sizeof(float) * (size_t)chunk * Q + sizeof(int32_t) * (size_t)N * k2 +
                         sizeof(int) * (nblk + 8) +
                         sizeof(int32_t) * (size_t)N + sizeof(int32_t) * (size_t)m_s +
-                        sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + 10 * 256 +
+                        sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + sizeof(double2) * kGuardCtas +
+                        10 * 256 +
                         infer_bytes(m, chunk);
     int rc = learn_workspace(c, need);
     if (rc) return rc;
@@ -847,6 +876,7 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     float* plainE = carve<float>(p, (size_t)m_s);
     float* learnedE = res_energy ? res_energy : carve<float>(p, (size_t)N);
     int* cnt_s = carve<int>(p, 2);
+    double2* part = carve<double2>(p, kGuardCtas);
     bf16* Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
     bf16* Hb = carve<bf16>(p, (size_t)chunk * m->H);
     // 1. scores and shortlists, chunk by chunk
@@ -917,8 +947,8 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
         if (rc < 0) return rc;
     }
     // 5. RMSE guard; when it trips, every signal is coded again by the plain coder
-    guard_kernel<<<1, kGuardThreads, 0, st>>>(plainE, learnedE, idx_s, (int)m_s, N, p1 * p2,
-                                              cnt_s + 1, n_fallback, guard_out);
+    guard_sums_kernel<<<kGuardCtas, kGuardThreads, 0, st>>>(plainE, learnedE, idx_s, (int)m_s, part);
+    guard_kernel<<<1, 32, 0, st>>>(part, (int)m_s, N, p1 * p2, cnt_s + 1, n_fallback, guard_out);
     mark_all_kernel<<<std::max(1, std::min(blocks_for(N, 256), c->num_sms * 8)), 256, 0, st>>>(
         cnt_s + 1, N, idx, fallback);
     a.idx_count = cnt_s + 1;
