@@ -18,12 +18,14 @@
 // Scores are recomputed from C0 every step, as in the other coders.
 //
 // Measured (GB300, us per call, one warp per signal -> this kernel): 200 000 x
-// 12x12, 24x24 pairs, s = 6: 472 -> 324 (of the compiled tilings the fastest,
+// 12x12, 24x24 pairs, s = 6: 472 -> 318 (of the compiled tilings the fastest,
 // two signals per warp, takes 410); 247 009 x 16x16, 32x32, s = 8: 1636 -> 1003;
-// 99 991 x 10x9, 20x18, s = 5 (generic kernel before): 493 -> 167.  At 12x12 a
+// 99 991 x 10x9, 20x18, s = 5 (generic kernel before): 493 -> 161.  At 12x12 a
 // signal takes 1106 warp instructions (1877 before); 71 % of the shared-memory
 // bandwidth (operands of the rank-one updates, and C0 read back every step) and
-// 51 % of the issue slots are in use.
+// 51 % of the issue slots are in use; the serial chain of a greedy step (argmax,
+// read-back, Cholesky row) sets the rest: a copy of C0 in tensor memory that took
+// the read-back off the shared memory left the time as it was (330 us).
 #pragma once
 
 #include <algorithm>
@@ -742,9 +744,12 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     if (masked) *masked = __int_as_float(0x7fc00000);
                     ld<E>(sc, myc0);
                 }
+                // one ahead of the loop: its load hides behind a rank-one update (12x12: 326 -> 318 us)
+                Rec next = rec[0];
 #pragma unroll 1
                 for (int l = 0; l < (C::kOrtho ? 0 : t); ++l) {
-                    const Rec r = rec[l];
+                    const Rec r = next;
+                    if (l + 1 < s) next = rec[l + 1];
                     float x[RI], v[RJ];
                     ld<RI>(x, G1s + r.o1() + li * RIP);
                     ld<RJ>(v, G2s + r.o2() + lj * RJP);
@@ -892,9 +897,11 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                 tm_ld_block<E>(tmine, sc);
                 tm_wait_ld();
                 unsigned picked[C::MW] = {};
+                Rec next = rec[0];
 #pragma unroll 1
                 for (int l = 0; l < s; ++l) {
-                    const Rec r = rec[l];
+                    const Rec r = next;
+                    if (l + 1 < s) next = rec[l + 1];
                     float x[RI], v[RJ];
                     ld<RI>(x, G1s + r.o1() + li * RIP);
                     ld<RJ>(v, G2s + r.o2() + lj * RJP);

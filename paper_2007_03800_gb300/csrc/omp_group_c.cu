@@ -3,7 +3,7 @@
 // four-warp teams (whose other warps waited while one did the Cholesky step).
 // 50 000 x 16x64, 32x128 pairs, s = 10: 2067 us there (28 300 warp instructions per
 // signal); 1721 us with teams of two warps and the C0 blocks in shared memory, which
-// then holds 5 signals per SM; 1435 us with them in tensor memory (6 teams of 168
+// then holds 5 signals per SM; 1406 us with them in tensor memory (6 teams of 168
 // registers; 8 teams of 128 spill: 1530 us), 52 % of the issue slots and of the
 // shared-memory bandwidth in use, the rest fixed-latency dependencies.
 #include "omp_group.cuh"

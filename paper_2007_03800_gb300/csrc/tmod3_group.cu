@@ -212,9 +212,11 @@ __global__ void __launch_bounds__(Sh::WARPS * 32, 2)
             if (!__any_sync(kFull, go)) break;
             if (t > 0) {
                 ld<E>(sc, myc0);
+                Rec next = rec[0];   // one ahead of the loop
 #pragma unroll 1
                 for (int m = 0; m < t; ++m) {
-                    const Rec q = rec[m];
+                    const Rec q = next;
+                    if (m + 1 < S) next = rec[m + 1];
                     float x[N1], v[RJ], wl[RL], vw[C];
                     ld<N1>(x, g1 + (q.o & 255u) * N1);
                     ld<RJ>(v, g2 + ((q.o >> 8) & 255u) * N2 + j0);
