@@ -744,17 +744,19 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     if (masked) *masked = __int_as_float(0x7fc00000);
                     ld<E>(sc, myc0);
                 }
-                // one ahead of the loop: its load hides behind a rank-one update (12x12: 326 -> 318 us)
-                Rec next = rec[0];
+                if constexpr (!C::kOrtho) {
+                    // one ahead of the loop: its load hides behind a rank-one update (12x12: 326 -> 318 us)
+                    Rec next = rec[0];
 #pragma unroll 1
-                for (int l = 0; l < (C::kOrtho ? 0 : t); ++l) {
-                    const Rec r = next;
-                    if (l + 1 < s) next = rec[l + 1];
-                    float x[RI], v[RJ];
-                    ld<RI>(x, G1s + r.o1() + li * RIP);
-                    ld<RJ>(v, G2s + r.o2() + lj * RJP);
-                    scale(x, v, r.x);
-                    rank1<RI, RJ>(sc, x, v);
+                    for (int l = 0; l < t; ++l) {
+                        const Rec r = next;
+                        if (l + 1 < s) next = rec[l + 1];
+                        float x[RI], v[RJ];
+                        ld<RI>(x, G1s + r.o1() + li * RIP);
+                        ld<RJ>(v, G2s + r.o2() + lj * RJP);
+                        scale(x, v, r.x);
+                        rank1<RI, RJ>(sc, x, v);
+                    }
                 }
             }
             // the lane's largest |score|, its first column, by column maxima

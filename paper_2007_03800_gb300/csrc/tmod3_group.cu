@@ -8,7 +8,7 @@
 // lane's block is all n1 rows of RJ x RL columns (j, l), so that one row of G1
 // feeds RJ RL columns, the maximum goes down the columns with three-input |max|,
 // and only the Cholesky row is unrolled per step.  50 000 cubes of 4x4x16, 8x8x16
-// atoms, s = 8: 353 us with one warp per signal, 234 us here (2645 instead of 4264
+// atoms, s = 8: 353 us with one warp per signal, 230 us here (2645 instead of 4264
 // warp instructions per signal).
 #include "omp_group.cuh"
 
