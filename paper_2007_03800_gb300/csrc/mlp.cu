@@ -460,7 +460,7 @@ __global__ void sample_index_kernel(int32_t* __restrict__ idx, int m, long long 
 
 // Fixed-order FP64 sums of the two residual energies over the sample, a pair per CTA
 // (one CTA alone spends 24 us on 2 x 12 500 of them, FP64 adds at one SM's rate; 13 us
-// with the verdict in a launch of its own).
+// with the decision in a launch of its own).
 constexpr int kGuardCtas = 64;
 __global__ void __launch_bounds__(kGuardThreads)
     guard_sums_kernel(const float* __restrict__ plainE, const float* __restrict__ learnedE,
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kGuardThreads)
     }
 }
 
-// one warp: the verdict from the kGuardCtas pairs
+// one warp: the decision from the kGuardCtas pairs
 __global__ void guard_kernel(const double2* __restrict__ part, int m, long long N, int P, int* __restrict__ recode_count,
                              int32_t* __restrict__ n_fallback, float* __restrict__ guard_out) {
     double ta = 0.0, tb = 0.0;
