@@ -311,14 +311,8 @@ __global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassA
 template <int PA, int SIDE>
 int launch(const PassArgs& a, bool want_energy, cudaStream_t st, int num_sms, size_t bytes, int warps) {
     auto kern = accum_lane_kernel<PA, SIDE>;
-    static bool attr[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-    if (dev >= 64 || !attr[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024) != cudaSuccess)
-            return SDL_ERR_CUDA;
-        if (dev < 64) attr[dev] = true;
-    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024) != cudaSuccess)
+        return SDL_ERR_CUDA;
     const int bps = std::max(1, std::min<int>(kMinCtas, (int)((228 * 1024) / (bytes + 2048))));
     const long long grid = std::max<long long>(1, std::min<long long>((a.N + warps - 1) / warps, (long long)num_sms * bps));
     kern<<<(int)grid, warps * 32, bytes, st>>>(a, want_energy ? 1 : 0);

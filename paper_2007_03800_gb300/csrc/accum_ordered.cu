@@ -191,14 +191,8 @@ int launch(const PassArgs& a, cudaStream_t st, int num_sms) {
     constexpr size_t bytes = sizeof(float) * (size_t)L::total;
     static_assert(bytes * Sh::CPS + 1024 * Sh::CPS <= 228 * 1024, "shared memory");
     auto kern = accum_ordered_kernel<Sh, SIDE>;
-    static bool attr[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-    if (dev >= 64 || !attr[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return SDL_ERR_CUDA;
-        if (dev < 64) attr[dev] = true;
-    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+        return SDL_ERR_CUDA;
     kern<<<ordered_slots(a, num_sms), Sh::WPC * 64, bytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
 }

@@ -990,15 +990,8 @@ int launch(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid) {
         warps -= C::TW;
     if (bytes > kSmMax) return SDL_ERR_UNSUPPORTED;
     auto kern = code_group_kernel<C>;
-    // the shared-memory opt-in, once per device
-    static bool attr[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-    if (dev >= 64 || !attr[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmMax) != cudaSuccess)
-            return SDL_ERR_CUDA;
-        if (dev < 64) attr[dev] = true;
-    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmMax) != cudaSuccess)
+        return SDL_ERR_CUDA;
     // the registers allow MINB CTAs per SM (launch bounds); 1 KB per CTA is reserved
     const int bps = std::max(1, std::min<int>(C::MINB, (int)(kSmTotal / (bytes + 1024))));
     const long long units = (a.N + C::SPW - 1) / C::SPW;

@@ -318,14 +318,8 @@ int run(const float* Y, long long N, const float* D1, const float* D2, const flo
     constexpr size_t bytes = sizeof(float) * (size_t)Sh::total;
     static_assert(2 * (bytes + 1024) <= 228 * 1024, "two CTAs per SM");
     auto kern = code3_group_kernel<Sh>;
-    static bool attr[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-    if (dev >= 64 || !attr[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return SDL_ERR_CUDA;
-        if (dev < 64) attr[dev] = true;
-    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+        return SDL_ERR_CUDA;
     const long long grid = std::max<long long>(1, std::min<long long>((N + 1) / 2, 2LL * num_sms));
     kern<<<(int)grid, Sh::WARPS * 32, bytes, st>>>(Y, N, D1, D2, D3, support, coef, nnz, res, err);
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
