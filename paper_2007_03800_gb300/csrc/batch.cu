@@ -25,7 +25,7 @@ struct sdl_batch {
     std::vector<int> generic;      // groups coded by the generic kernel
     std::vector<int> gslots[3];    // their partial-sum slots per pass side
     int n_fast = 0;                // groups in the multi-problem kernel
-    bool large_groups = false;     // each of them fills the GPU by itself
+    bool large_groups = false;     // code-only passes run group by group (kLanesWork)
     std::vector<int> cta_begin;    // G + 1 prefix of CTAs per group
     std::vector<float> cost_us;    // time of one fused pass of the group alone
     int single_cps = 0;            // one group: the CTAs per SM the autotuner chose
@@ -60,10 +60,16 @@ namespace {
 constexpr int kSlotsPerSm = 8;   // partial-sum slots reserved per SM and group
 constexpr int kMultiWarps = 8;   // warps per CTA of the persistent multi-problem kernel
 
-// Signals from which a group's code-only pass runs as its own launch of the
-// lane-group coder (omp_group.cuh) rather than inside the multi-problem launch.
-constexpr long long kLargeGroup = 8192;
-// (and up to which the list of an error-driven one fits its partial-sum slots)
+// Signals times atom pairs, on average over the groups, from which a code-only pass
+// runs each group as its own launches of the lane-group coder (omp_group.cuh) rather
+// than all of them in the multi-problem launch.  Error-driven groups of an image's
+// patches, us in one launch | in their own: 8x16 x 15 129 signals (3.9M) 21 | 25, x 37 249
+// (9.5M) 27 | 27; 12x24 x 7 921 (4.6M) 29 | 33, x 14 161 (8.2M) 35 | 35, x 35 721 52 | 46;
+// 16x32 x 7 225 (7.4M) 56 | 54, x 13 225 78 | 62; all three (14.2M) 96 | 105, (25.6M) 150 | 116.
+// Without a large dictionary the one launch packs its SMs better and wins longer:
+// 8x16 and 12x24 x 66 000 (27.5M on average, few picks) 74 | 80, x 103 000 (43M) 98 | 85.
+constexpr long long kLanesWork = 8'000'000, kLanesWorkSmall = 40'000'000;
+// Signals up to which the list of an error-driven group fits its partial-sum slots.
 constexpr long long kMostListed = 1 << 20;
 
 // A coding pass of every group: one persistent multi-problem launch, or for a
@@ -197,9 +203,16 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         if (gen) b->generic.push_back(g);
     }
     b->n_fast = G - (int)b->generic.size();
-    b->large_groups = true;
-    for (int g = 0; g < G; ++g)
-        if (!variants[g].empty() && (groups[g].N < kLargeGroup || groups[g].N > kMostListed)) b->large_groups = false;
+    long long work = 0;
+    bool large = false;     // some dictionary pair of 1024 or more atom pairs
+    b->large_groups = b->n_fast > 0;
+    for (int g = 0; g < G; ++g) {
+        if (variants[g].empty()) continue;
+        work += groups[g].N * (groups[g].n1 * groups[g].n2);
+        large = large || groups[g].n1 * groups[g].n2 >= 1024;
+        if (groups[g].N > kMostListed) b->large_groups = false;
+    }
+    if (work < (large ? kLanesWork : kLanesWorkSmall) * b->n_fast) b->large_groups = false;
 
     // ---- device memory
     const int max_slots = c->num_sms * kSlotsPerSm;
