@@ -367,8 +367,9 @@ def run_ours(args):
     flush = torch.empty(FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
     stream = torch.cuda.current_stream()
 
-    # the per-call path runs the tiling the tuner measured fastest on these
-    # signals (every tiling gives the same codes), or the one --tiling names
+    # the per-call path runs what the tuner measured fastest on these signals (a
+    # fused tiling or the lane-group form; the same codes), or the tiling that
+    # --tiling names
     if args.tiling is None:
         tiling, tune_log = ctx.tune_tiling(Yg, D1g, D2g, s)
         tune_log = [dict(tiling=e["tiling"], ctas_per_sm=e["ctas_per_sm"], us=round(e["us"], 1))

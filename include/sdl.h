@@ -348,13 +348,23 @@ int sdl_set_precision(sdl_ctx* ctx, int flags);
  * sdl_tilings: the tiling ids compiled for the shape (host array of max_ids,
  *   may be NULL); returns their number (0: no specialised coder, the generic
  *   kernel runs), SDL_ERR_ARG for max_ids < 0.
+ * They are the kernels of a coding pass fused with its partial sums; unpinned
+ * calls that only code, and learning iterations on many signals, run the
+ * lane-group coder instead, which is faster there (the same codes, and sums in
+ * the default tiling's order).
+ *
  * sdl_set_tiling: pin `tiling` (one of those ids) and ctas_per_sm (0 = as many
- *   CTAs per SM as fit, else 1..8) for the shape in this context; tiling < 0
- *   unpins.  SDL_ERR_UNSUPPORTED if the shape has no such tiling.
+ *   CTAs per SM as fit, else 1..8) for the shape in this context: every call of
+ *   the shape then runs that fused kernel; tiling < 0 unpins.
+ *   SDL_ERR_UNSUPPORTED if the shape has no such tiling.
  * sdl_tune_tiling: time one D1-side coding pass (Y p1 x p2 x N and D1, D2 as
  *   in sdl_iterate, device pointers, Y 16-byte aligned; nothing is written but
- *   workspace) with every tiling at 1 and 2 CTAs per SM, pin the fastest and
- *   return its id in *tiling_out (may be NULL).  Synchronises the stream.
+ *   workspace and an allocation of the codes' size, freed again) with every
+ *   tiling at 1 and 2 CTAs per SM, and return the fastest's id in *tiling_out
+ *   (may be NULL).  From then on a pass of the shape that runs fused uses that
+ *   tiling; a call that the lane-group coder takes keeps it, except that a
+ *   learning iteration on up to N signals runs fused if the fastest tiling beat
+ *   the lane-group form of the same pass here.  Synchronises the stream.
  *   SDL_ERR_UNSUPPORTED if the shape has no specialised coder or Y is not
  *   16-byte aligned.
  * sdl_tune_log: the measurements of the last sdl_tune_tiling (tiling id, CTAs

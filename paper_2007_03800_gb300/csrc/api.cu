@@ -58,6 +58,12 @@ int check_shape(int p1, int p2, int n1, int n2, int s) {
     return SDL_OK;
 }
 
+sdl_ctx::Pin* find_pin(sdl_ctx* c, int p1, int p2, int n1, int n2, int s) {
+    for (auto& pin : c->pins)
+        if (pin.p1 == p1 && pin.p2 == p2 && pin.n1 == n1 && pin.n2 == n2 && pin.s == s) return &pin;
+    return nullptr;
+}
+
 PassArgs base_args(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const float* D1, int n1,
                    const float* D2, int n2, int s) {
     PassArgs a;
@@ -77,22 +83,17 @@ PassArgs base_args(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const 
     a.part_d = c->part_d;
     a.n_slots = 1;
     a.err = c->err;
-    for (const auto& pin : c->pins)
-        if (pin.p1 == p1 && pin.p2 == p2 && pin.n1 == n1 && pin.n2 == n2 && pin.s == s) {
-            a.tiling = pin.id + 1;
-            a.tiling_cps = pin.cps;
-        }
+    if (const sdl_ctx::Pin* pin = find_pin(c, p1, p2, n1, n2, s)) {
+        a.tiling = pin->id + 1;
+        a.tiling_cps = pin->cps;
+        a.tiling_forced = pin->forced ? 1 : 0;
+    }
     return a;
 }
 
-void pin_tiling(sdl_ctx* c, int p1, int p2, int n1, int n2, int s, int id, int cps) {
-    for (auto& pin : c->pins)
-        if (pin.p1 == p1 && pin.p2 == p2 && pin.n1 == n1 && pin.n2 == n2 && pin.s == s) {
-            pin.id = id;
-            pin.cps = cps;
-            return;
-        }
-    c->pins.push_back(sdl_ctx::Pin{p1, p2, n1, n2, s, id, cps});
+void pin_tiling(sdl_ctx* c, const sdl_ctx::Pin& p) {
+    if (sdl_ctx::Pin* old = find_pin(c, p.p1, p.p2, p.n1, p.n2, p.s)) *old = p;
+    else c->pins.push_back(p);
 }
 
 void grams(sdl_ctx* c, const float* D1, int p1, int n1, const float* D2, int p2, int n2,
@@ -131,14 +132,14 @@ int prepare_tc_pass(sdl_ctx* c, PassArgs& a, bool fill_y, cudaStream_t st) {
 
 // Partial-sum slots of a learning pass that runs as the lane-group coder followed
 // by the ordered sums (compiled shapes, fixed sparsity, aligned signals, no tiling
-// pinned), or 0: the fused kernels.  Two launches instead of one pay off from
+// forced or tuned to be faster), or 0: the fused kernels.  Two launches instead of one pay off from
 // about 2.1M correlations on: an iteration (us, split / fused) at 8x8 x 4000 78 / 75,
 // x 16000 95 / 99, x 64000 169 / 202; at 12x12 x 2000 94 / 88, x 4000 97 / 100,
 // x 64000 332 / 421; at 16x16 x 1000 110 / 101, x 4000 130 / 137, x 64000 688 / 987.
 constexpr long long kSplitPairs = 2100000;
 int split_pass_slots(const PassArgs& a, bool tc, int num_sms) {
     if (a.N * a.n1 * a.n2 < kSplitPairs) return 0;
-    if (tc || a.tiling > 0 || a.eps2 > 0.f || a.N < 1 || (reinterpret_cast<uintptr_t>(a.Y) & 15u)) return 0;
+    if (tc || a.tiling_forced || a.eps2 > 0.f || a.N < 1 || (reinterpret_cast<uintptr_t>(a.Y) & 15u)) return 0;
     return std::max(0, ordered_slots(a, num_sms));
 }
 
@@ -388,6 +389,8 @@ int sdl_iterate(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, float* D1
     PassArgs a = base_args(c, Y, p1, p2, N, D1, n1, D2, n2, s);
     a.eps2 = eps2;
     const bool tc = (c->prec & SDL_PREC_BF16_CORR) != 0;
+    const sdl_ctx::Pin* pin = find_pin(c, p1, p2, n1, n2, s);
+    if (pin && N <= pin->fused_n) a.tiling_forced = 1;
     const int ordered = split_pass_slots(a, tc, c->num_sms);
     // one coding pass with its sums: the number of partial-sum slots
     auto code_side = [&](int side) -> int {
@@ -446,7 +449,7 @@ int sdl_set_tiling(sdl_ctx* c, int p1, int p2, int n1, int n2, int s, int tiling
     const int n = fast_shape_variants(p1, p2, n1, n2, s, all, 64);
     for (int v = 0; v < n; ++v)
         if (all[v] == tiling) {
-            pin_tiling(c, p1, p2, n1, n2, s, tiling, ctas_per_sm);
+            pin_tiling(c, sdl_ctx::Pin{p1, p2, n1, n2, s, tiling, ctas_per_sm, true, 0});
             return SDL_OK;
         }
     return SDL_ERR_UNSUPPORTED;
@@ -472,25 +475,29 @@ int sdl_tune_tiling(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const
         cudaEventDestroy(e0);
         return SDL_ERR_CUDA;
     }
+    // one untimed run, then the mean of three, in us (negative: did not run)
+    bool failed = false;
+    auto timed = [&](auto&& run) -> float {
+        if (run() < 0) return -1.f;
+        cudaEventRecord(e0, st);
+        for (int r = 0; r < 3; ++r) run();
+        cudaEventRecord(e1, st);
+        float ms = 0.f;
+        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+            failed = true;
+            return -1.f;
+        }
+        return ms * 1000.f / 3.f;
+    };
     c->tune_log.clear();
     int best_id = -1, best_cps = 0;
     float best = 1e30f;
-    for (int v = 0; v < n; ++v) {
-        for (int cps = 1; cps <= 2; ++cps) {
-            // one untimed launch, then the mean of three (D1-side passes, the
-            // heavier of the two epilogues)
-            if (launch_code_pass_variant(a, kSideD1, ids[v], cps, st, c->num_sms) < 0) continue;
-            cudaEventRecord(e0, st);
-            for (int r = 0; r < 3; ++r) launch_code_pass_variant(a, kSideD1, ids[v], cps, st, c->num_sms);
-            cudaEventRecord(e1, st);
-            if (cudaEventSynchronize(e1) != cudaSuccess) {
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                return SDL_ERR_CUDA;
-            }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            const float us = ms * 1000.f / 3.f;
+    // the fused tilings: D1-side passes, the heavier of the two epilogues
+    for (int v = 0; v < n && !failed; ++v) {
+        for (int cps = 1; cps <= 2 && !failed; ++cps) {
+            const float us =
+                timed([&] { return launch_code_pass_variant(a, kSideD1, ids[v], cps, st, c->num_sms); });
+            if (us < 0.f) continue;
             c->tune_log.push_back(sdl_ctx::TuneRec{ids[v], cps, us});
             if (us < best) {
                 best = us;
@@ -499,10 +506,33 @@ int sdl_tune_tiling(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const
             }
         }
     }
+    // The same pass by lane groups, where a learning iteration on N signals would
+    // run so: it keeps that form unless the best tiling beats it here.
+    sdl_ctx::Pin pin{p1, p2, n1, n2, s, best_id, best_cps, false, 0};
+    a.tiling_forced = 0;
+    const int slots = failed ? 0 : split_pass_slots(a, false, c->num_sms);
+    char* codes = nullptr;
+    const size_t words = (size_t)N * s;
+    if (slots > 0 && cudaMalloc(&codes, 4 * (2 * words + (size_t)N)) == cudaSuccess) {
+        int32_t* sup = reinterpret_cast<int32_t*>(codes);
+        float* coef = reinterpret_cast<float*>(sup + words);
+        int32_t* nnz = reinterpret_cast<int32_t*>(coef + words);
+        int64_t kept[SDL_NUM_KERNEL_KINDS];   // timing runs are not counted
+        std::copy(c->launches, c->launches + SDL_NUM_KERNEL_KINDS, kept);
+        const bool traced = c->timing;
+        c->timing = false;
+        const float us = timed([&] { return split_pass(c, a, kSideD1, slots, sup, coef, nnz, st); });
+        c->timing = traced;
+        std::copy(kept, kept + SDL_NUM_KERNEL_KINDS, c->launches);
+        if (us < 0.f || us > best) pin.fused_n = N;
+        cudaFree(codes);
+    } else {
+        cudaGetLastError();
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best_id < 0) return SDL_ERR_CUDA;
-    pin_tiling(c, p1, p2, n1, n2, s, best_id, best_cps);
+    if (failed || best_id < 0) return SDL_ERR_CUDA;
+    pin_tiling(c, pin);
     if (tiling_out) *tiling_out = best_id;
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
 }

@@ -34,10 +34,15 @@ struct sdl_ctx {
     unsigned long long* rescored = nullptr;
     size_t cap_g1 = 0, cap_g2 = 0, cap_part = 0, cap_slots = 0, cap_red = 0, cap_redd = 0,
            cap_norms = 0;
-    // coder tilings pinned per shape (sdl_tune_tiling / sdl_set_tiling) and
-    // the measurements of the last sdl_tune_tiling
+    // coder tilings pinned per shape and the measurements of the last
+    // sdl_tune_tiling.  sdl_set_tiling forces the fused kernels in every call;
+    // sdl_tune_tiling chooses the tiling wherever they run, and sends a learning
+    // pass to them where it timed them ahead of the lane groups (up to fused_n
+    // signals)
     struct Pin {
         int p1, p2, n1, n2, s, id, cps;
+        bool forced;
+        int64_t fused_n;
     };
     std::vector<Pin> pins;
     struct TuneRec {

@@ -111,7 +111,7 @@ long long list_capacity(size_t ws_n) {
 bool code_lanes_take(const PassArgs& a, size_t ws_n) {
     // correlations from the tensor cores, a pinned tiling and wider dictionaries
     // have coders of their own
-    if (a.c0ext || a.tiling > 0 || a.n1 > 32 || a.n2 > 128) return false;
+    if (a.c0ext || a.tiling_forced || a.n1 > 32 || a.n2 > 128) return false;
     // the scan's sums are those of the coders with 32 chains
     return !(a.eps2 > 0.f) || (!a.idx && a.n2 <= 32 && a.N <= kSegments * list_capacity(ws_n));
 }

@@ -65,6 +65,8 @@ struct PassArgs {
     // as fit)
     int tiling;
     int tiling_cps;
+    // the pinned tiling's fused kernel runs this call (0: the lane groups may take it)
+    int tiling_forced;
     // lane-group coder only, optional: per-CTA sums of the residual energies,
     // [esum_slots][2] (entry 0; slots past its grid and entries 1 are cleared)
     double* esum;

@@ -390,8 +390,9 @@ class Context:
                "sdl_set_tiling")
 
     def tune_tiling(self, Y, D1, D2, s, stream=None):
-        """Time every tiling of the shape on these signals, pin the fastest;
-        returns (tiling id, [dict(tiling, ctas_per_sm, us), ...])."""
+        """Time every fused tiling of the shape on these signals; passes that run fused
+        use the fastest from then on, calls that the lane-group coder takes keep it
+        where it is faster.  Returns (tiling id, [dict(tiling, ctas_per_sm, us), ...])."""
         N, p1, p2 = _check_Y(Y)
         n1, n2 = _check_D(D1, p1, "D1"), _check_D(D2, p2, "D2")
         tid = ctypes.c_int(-1)
