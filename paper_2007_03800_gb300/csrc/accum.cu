@@ -319,27 +319,42 @@ int launch(const PassArgs& a, bool want_energy, cudaStream_t st, int num_sms, si
     return cudaGetLastError() == cudaSuccess ? (int)grid : SDL_ERR_CUDA;
 }
 
+// Rows per lane block, warps per CTA (0: the pass does not take these sizes) and
+// shared memory of a CTA.
+struct AccumPlan {
+    int PA = 0, warps = 0;
+    size_t bytes = 0;
+};
+AccumPlan plan(const PassArgs& a, int side) {
+    const int pa = side == kSideD1 ? a.p1 : a.p2, pc = side == kSideD1 ? a.p2 : a.p1;
+    const int na = side == kSideD1 ? a.n1 : a.n2, nc = side == kSideD1 ? a.n2 : a.n1;
+    AccumPlan q;
+    if (na > 32 || pa > 32) return q;
+    q.PA = pa <= 8 ? 8 : pa <= 16 ? 16 : 32;
+    for (int warps = kWarps; warps >= 4; --warps) {
+        q.bytes = sizeof(float) * (size_t)AccumLayout(a.p1, a.p2, pa, pc, na, nc, a.s, q.PA, side, warps).total;
+        if (q.bytes <= 200 * 1024) {
+            q.warps = warps;
+            break;
+        }
+    }
+    return q;
+}
+
 template <int SIDE>
 int run(const PassArgs& a, bool want_energy, cudaStream_t st, int num_sms) {
-    const int pa = SIDE == kSideD1 ? a.p1 : a.p2, pc = SIDE == kSideD1 ? a.p2 : a.p1;
-    const int na = SIDE == kSideD1 ? a.n1 : a.n2, nc = SIDE == kSideD1 ? a.n2 : a.n1;
-    if (na > 32 || pa > 32) return SDL_ERR_UNSUPPORTED;
-    const int PA = pa <= 8 ? 8 : pa <= 16 ? 16 : 32;
-    int warps = kWarps;
-    size_t bytes;
-    for (;; --warps) {
-        bytes = sizeof(float) * (size_t)AccumLayout(a.p1, a.p2, pa, pc, na, nc, a.s, PA, SIDE, warps).total;
-        if (bytes <= 200 * 1024) break;
-        if (warps <= 4) return SDL_ERR_UNSUPPORTED;
-    }
-    switch (PA) {
-        case 8: return launch<8, SIDE>(a, want_energy, st, num_sms, bytes, warps);
-        case 16: return launch<16, SIDE>(a, want_energy, st, num_sms, bytes, warps);
-        default: return launch<32, SIDE>(a, want_energy, st, num_sms, bytes, warps);
+    const AccumPlan q = plan(a, SIDE);
+    if (q.warps == 0) return SDL_ERR_UNSUPPORTED;
+    switch (q.PA) {
+        case 8: return launch<8, SIDE>(a, want_energy, st, num_sms, q.bytes, q.warps);
+        case 16: return launch<16, SIDE>(a, want_energy, st, num_sms, q.bytes, q.warps);
+        default: return launch<32, SIDE>(a, want_energy, st, num_sms, q.bytes, q.warps);
     }
 }
 
 }  // namespace
+
+bool accumulate_lanes_take(const PassArgs& a, int side) { return plan(a, side).warps > 0; }
 
 int launch_accumulate_lanes(const PassArgs& a, int side, bool want_energy, cudaStream_t st, int num_sms) {
     return side == kSideD1 ? run<kSideD1>(a, want_energy, st, num_sms) : run<kSideD2>(a, want_energy, st, num_sms);

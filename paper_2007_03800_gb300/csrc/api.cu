@@ -339,15 +339,14 @@ static int update_common(sdl_ctx* c, int side, const float* Y, int p1, int p2, i
     PassArgs a = base_args(c, Y, p1, p2, N, D1, n1, D2, n2, s);
     a.in_support = support;
     a.in_coef = coef;
+    const bool lanes = accumulate_lanes_take(a, side);
+    if (!lanes) grams(c, D1, p1, n1, D2, p2, n2, st);
     int slots;
     {
         // the residual energy before the update goes to objective_out alone
         Trace tr(c, side == kSideD1 ? kAccD1 : kAccD2, st);
-        slots = launch_accumulate_lanes(a, side, objective_out != nullptr, st, c->num_sms);
-    }
-    if (slots == SDL_ERR_UNSUPPORTED) {
-        grams(c, D1, p1, n1, D2, p2, n2, st);
-        slots = launch_accumulate_pass(a, side, st, c->num_sms);
+        slots = lanes ? launch_accumulate_lanes(a, side, objective_out != nullptr, st, c->num_sms)
+                      : launch_accumulate_pass(a, side, st, c->num_sms);
     }
     if (slots < 0) return slots;
     float* D = side == kSideD1 ? D1w : D2w;

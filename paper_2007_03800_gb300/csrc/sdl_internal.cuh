@@ -130,7 +130,8 @@ int multi_ctas_per_sm(size_t smem, int side);
 // accum.cu: partial sums of one side from given codes (a.in_support, a.in_coef),
 // up to 32 atoms and rows on that side; the residual energy with the given
 // dictionaries only if wanted.  Returns the slots written, or
-// SDL_ERR_UNSUPPORTED.  Needs no Gram matrices.
+// SDL_ERR_UNSUPPORTED for sizes that it does not take.  Needs no Gram matrices.
+bool accumulate_lanes_take(const PassArgs& a, int side);
 int launch_accumulate_lanes(const PassArgs& a, int side, bool want_energy, cudaStream_t st, int num_sms);
 // accum_ordered.cu: the sums of a fused coding pass at a compiled shape from codes
 // already written (a.in_support, a.in_coef; Y 16-byte aligned), in the fused
@@ -143,15 +144,16 @@ int max_partial_slots(int num_sms);
 // tmod3_fast.cu: three-mode coding pass specialised at compile time for the
 // compiled shapes (SDL_ERR_UNSUPPORTED otherwise or for a Y not 16-byte
 // aligned); returns the partial-sum slots written (mode 1-3) or 0 (mode 0)
-// tmod3_group.cu: the same shapes without partial sums (no Gram matrices needed)
-int launch_code3_group(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, long long N, const float* D1,
-                       const float* D2, const float* D3, int s, int32_t* support, float* coef, int32_t* nnz,
-                       float* res, int* err, int num_sms, cudaStream_t st);
 int launch_code3_fast(int mode, const float* Y, int p1, int p2, int p3, int n1, int n2, int n3,
                       long long N, const float* D1, const float* D2, const float* D3,
                       const float* G1, const float* G2, const float* G3, int s, int32_t* support,
                       float* coef, int32_t* nnz, float* res, float* part_f, double* part_d,
                       int max_slots, int* err, int num_sms, cudaStream_t st);
+// tmod3_group.cu: coding alone at the same shapes (no Gram matrices needed)
+bool code3_group_takes(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, int s);
+int launch_code3_group(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, long long N, const float* D1,
+                       const float* D2, const float* D3, int s, int32_t* support, float* coef, int32_t* nnz,
+                       float* res, int* err, int num_sms, cudaStream_t st);
 
 // tmod.cu
 void launch_gram(const float* D, int p, int n, float* G, cudaStream_t st);

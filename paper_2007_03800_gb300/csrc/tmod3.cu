@@ -417,16 +417,13 @@ int sdl_sparse_code3(sdl_ctx* c, const float* Y, int p1, int p2, int p3, int64_t
     if (!Y || !D1 || !D2 || !D3 || !support || !coef || !nnz) return SDL_ERR_ARG;
     DeviceGuard g(c->device);
     cudaStream_t st = (cudaStream_t)stream;
-    int rc;
-    {
+    if (code3_group_takes(Y, p1, p2, p3, n1, n2, n3, s)) {
         Trace tr(c, kCode, st);
-        rc = launch_code3_group(Y, p1, p2, p3, n1, n2, n3, N, D1, D2, D3, s, support, coef, nnz, res_energy, c->err,
-                                c->num_sms, st);
+        return launch_code3_group(Y, p1, p2, p3, n1, n2, n3, N, D1, D2, D3, s, support, coef, nnz, res_energy,
+                                  c->err, c->num_sms, st);
     }
-    if (rc != SDL_ERR_UNSUPPORTED) return rc;
-    c->launches[kCode] -= 1;   // not taken: counted below
     float *G1, *G2, *G3;
-    rc = grams3(c, D1, p1, n1, D2, p2, n2, D3, p3, n3, &G1, &G2, &G3, st);
+    int rc = grams3(c, D1, p1, n1, D2, p2, n2, D3, p3, n3, &G1, &G2, &G3, st);
     if (rc != SDL_OK) return rc;
     Trace tr(c, kCode, st);
     rc = launch_code3(0, Y, h, N, D1, D2, D3, G1, G2, G3, s, support, coef, nnz, res_energy,

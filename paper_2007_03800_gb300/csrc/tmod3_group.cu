@@ -328,20 +328,33 @@ int run(const float* Y, long long N, const float* D1, const float* D2, const flo
 using G3cube = Shape3G<4, 4, 16, 8, 8, 16, 8, 4, 2>;
 using G3small = Shape3G<4, 4, 4, 8, 8, 8, 4, 4, 1>;
 
-}  // namespace
-
-int launch_code3_group(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, long long N, const float* D1,
-                       const float* D2, const float* D3, int s, int32_t* support, float* coef, int32_t* nnz,
-                       float* res, int* err, int num_sms, cudaStream_t st) {
-    if ((reinterpret_cast<uintptr_t>(Y) & 15u) != 0) return SDL_ERR_UNSUPPORTED;
+// the compiled shape of these sizes, if any
+template <class F>
+int with_shape(int p1, int p2, int p3, int n1, int n2, int n3, int s, F&& f) {
     auto is = [&](auto sh) {
         using Sh = decltype(sh);
         return p1 == Sh::P1 && p2 == Sh::P2 && p3 == Sh::P3 && n1 == Sh::N1 && n2 == Sh::N2 && n3 == Sh::N3 &&
                s == Sh::S;
     };
-    if (is(G3cube{})) return run<G3cube>(Y, N, D1, D2, D3, support, coef, nnz, res, err, num_sms, st);
-    if (is(G3small{})) return run<G3small>(Y, N, D1, D2, D3, support, coef, nnz, res, err, num_sms, st);
+    if (is(G3cube{})) return f(G3cube{});
+    if (is(G3small{})) return f(G3small{});
     return SDL_ERR_UNSUPPORTED;
+}
+
+}  // namespace
+
+bool code3_group_takes(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, int s) {
+    return (reinterpret_cast<uintptr_t>(Y) & 15u) == 0 &&
+           with_shape(p1, p2, p3, n1, n2, n3, s, [](auto) { return (int)SDL_OK; }) == SDL_OK;
+}
+
+int launch_code3_group(const float* Y, int p1, int p2, int p3, int n1, int n2, int n3, long long N, const float* D1,
+                       const float* D2, const float* D3, int s, int32_t* support, float* coef, int32_t* nnz,
+                       float* res, int* err, int num_sms, cudaStream_t st) {
+    if ((reinterpret_cast<uintptr_t>(Y) & 15u) != 0) return SDL_ERR_UNSUPPORTED;
+    return with_shape(p1, p2, p3, n1, n2, n3, s, [&](auto sh) {
+        return run<decltype(sh)>(Y, N, D1, D2, D3, support, coef, nnz, res, err, num_sms, st);
+    });
 }
 
 }  // namespace sdl
