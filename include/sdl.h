@@ -393,7 +393,10 @@ typedef struct sdl_mlp sdl_mlp;
 
 /* Network for p1 x p2 signals and n1 x n2 pairs (n1*n2 <= 1024, a multiple
  * of 8), `hidden` units (multiple of 8), batches of up to max_batch (multiple
- * of 8) signals.  Weights start at zero: set them with sdl_mlp_set_weights. */
+ * of 8) signals.  Weights start at zero: set them with sdl_mlp_set_weights.
+ * The network holds the buffers of its training batch and of an inference chunk
+ * (max_batch signals, or up to 32768 while they fit 64 MB); training and forward
+ * calls allocate nothing. */
 int sdl_mlp_create(sdl_ctx* ctx, int p1, int p2, int n1, int n2, int hidden, int max_batch,
                    sdl_mlp** out);
 int sdl_mlp_destroy(sdl_mlp* mlp);
@@ -417,7 +420,8 @@ int sdl_mlp_gradients(sdl_mlp* mlp, const float* Y, const int32_t* support, int 
                       float* loss_out, float* gW1, float* gb1, float* gW2, float* gb2,
                       void* stream);
 
-/* Scores of N signals: device FP32 N x n1n2. */
+/* Scores of N signals: device FP32 N x n1n2.  Any N; runs in chunks through the
+ * network's buffers. */
 int sdl_mlp_forward(sdl_mlp* mlp, const float* Y, int64_t N, float* scores, void* stream);
 
 /*
@@ -439,7 +443,10 @@ int sdl_mlp_forward(sdl_mlp* mlp, const float* Y, int64_t N, float* scores, void
  * Outputs as sdl_sparse_code plus fallback[N] (1 = re-coded), device
  * int n_fallback[1] and guard_out: NULL or device float[3] = {RMSE of the
  * learned codes on the sample (after step 3), RMSE of the full coder there,
- * 1 if step 4 re-coded everything else 0}.  N <= 2^31 - 1.  Compiled for
+ * 1 if step 4 re-coded everything else 0}.  N <= 2^31 - 1.  Grows a context
+ * workspace (shortlists and indices of all signals, the FP32 scores of one
+ * inference chunk) by an allocation that waits for the device; a call that fits
+ * what earlier ones left allocates nothing.  Compiled for
  * (p1,p2,n1,n2,s_max) = (12,12,24,24,6) and (8,8,16,16,4); the network must
  * match the shape.
  */

@@ -26,6 +26,7 @@ using bf16 = __nv_bfloat16;
 struct sdl_mlp {
     sdl_ctx* ctx = nullptr;
     int P = 0, H = 0, Q = 0, Kp = 0, Bmax = 0, step = 0;
+    int rows = 0;                // signals that Xb and Hb hold: a training batch or an inference chunk
     float *W1 = nullptr, *b1 = nullptr, *W2 = nullptr, *b2 = nullptr;
     float *mW1, *vW1, *mb1, *vb1, *mW2, *vW2, *mb2, *vb2;
     float *gW1, *gb1, *gW2, *gb2;
@@ -534,7 +535,7 @@ T* carve(char*& p, size_t n) {
     return r;
 }
 
-// The context's second stream and its events, made on first use.
+// The context's second stream and its events, made with its first network.
 int side_stream(sdl_ctx* c) {
     if (!c->side && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) return SDL_ERR_CUDA;
     for (cudaEvent_t& e : c->side_ev)
@@ -543,6 +544,15 @@ int side_stream(sdl_ctx* c) {
 }
 
 int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
+
+// Inference runs in chunks of this many signals: a 4096-signal chunk leaves
+// every SM one 128 x 128 tile per GEMM, so that nothing hides the epilogue's GELU
+// (23 us per chunk at 64 -> 512; 8 times the signals take 36 us), while the
+// activations and scores of a chunk still stay in L2.  The network holds the
+// buffers of a chunk from its creation on, so that a forward pass allocates
+// nothing and may be captured; wide networks take shorter chunks.
+constexpr int kInferChunk = 32768;
+constexpr size_t kInferBytes = size_t(64) << 20;
 
 }  // namespace
 
@@ -565,10 +575,17 @@ int sdl_mlp_create(sdl_ctx* c, int p1, int p2, int n1, int n2, int hidden, int m
     m->Q = n1 * n2;
     m->Bmax = max_batch;
     const size_t H = m->H, Kp = m->Kp, Q = m->Q, B = m->Bmax;
+    m->rows = std::max(m->Bmax, (int)std::min<size_t>(kInferChunk, kInferBytes / (2 * (Kp + H)) & ~size_t(127)));
+    const size_t R = m->rows;
     const size_t nf = 4 * (H * Kp + H + Q * H + Q) + 1024;     // params, m, v, grads
     const size_t nloss = B * ((Q + kBceCols - 1) / kBceCols);
-    const size_t bytes = (nf * 4 + nloss * 4 + (H * Kp + 2 * Q * H) * 2 + (2 * B * Kp + 2 * B * H + 2 * B * Q + B * H) * 2 +
+    const size_t bytes = (nf * 4 + nloss * 4 + (H * Kp + 2 * Q * H) * 2 +
+                          (R * Kp + B * Kp + R * H + B * H + 2 * B * Q + B * H) * 2 +
                           (B * H + B * Q + B) * 4) + 64 * 256;
+    if (side_stream(c) != SDL_OK) {
+        delete m;
+        return SDL_ERR_CUDA;
+    }
     if (cudaMalloc(&m->mem, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete m;
@@ -585,8 +602,8 @@ int sdl_mlp_create(sdl_ctx* c, int p1, int p2, int n1, int n2, int hidden, int m
     m->gW1 = carve<float>(p, H * Kp); m->gb1 = carve<float>(p, H);
     m->gW2 = carve<float>(p, Q * H); m->gb2 = carve<float>(p, Q);
     m->W1b = carve<bf16>(p, H * Kp); m->W2b = carve<bf16>(p, Q * H); m->W2Tb = carve<bf16>(p, H * Q);
-    m->Xb = carve<bf16>(p, B * Kp); m->XTb = carve<bf16>(p, Kp * B);
-    m->Hb = carve<bf16>(p, B * H); m->HTb = carve<bf16>(p, H * B);
+    m->Xb = carve<bf16>(p, R * Kp); m->XTb = carve<bf16>(p, Kp * B);
+    m->Hb = carve<bf16>(p, R * H); m->HTb = carve<bf16>(p, H * B);
     m->dZb = carve<bf16>(p, B * Q); m->dZTb = carve<bf16>(p, Q * B);
     m->dPreTb = carve<bf16>(p, H * B);
     m->pre = carve<float>(p, B * H); m->Z = carve<float>(p, B * Q); m->lossp = carve<float>(p, nloss);
@@ -658,8 +675,7 @@ static int mlp_batch(sdl_mlp* m, const float* Y, const int32_t* support, int s, 
                      float lr, float* loss_out, cudaStream_t st) {
     sdl_ctx* c = m->ctx;
     const int H = m->H, Kp = m->Kp, Q = m->Q, Bm = m->Bmax;
-    int rc = side_stream(c);
-    if (rc) return rc;
+    int rc;
     {
         Trace tr(c, kMlp, st);
         prep_batch_kernel<<<blocks_for(B, 32), 256, 0, st>>>(Y, B, m->P, Kp, m->Xb, m->XTb, Bm);
@@ -740,35 +756,11 @@ int sdl_mlp_gradients(sdl_mlp* m, const float* Y, const int32_t* support, int s,
     return SDL_OK;
 }
 
-// Inference runs in chunks of this many signals: a 4096-signal chunk leaves
-// every SM one 128 x 128 tile per GEMM, so that nothing hides the epilogue's GELU
-// (23 us per chunk at 64 -> 512; 8 times the signals take 36 us), while the
-// activations and scores of a chunk still stay in L2.
-constexpr int64_t kInferChunk = 32768;
-
-static size_t infer_bytes(const sdl_mlp* m, int64_t rows) {
-    return (size_t)rows * (m->Kp + m->H) * sizeof(bf16) + 2 * 256;
-}
-
-// Grow the context's learned-coder workspace.
-static int learn_workspace(sdl_ctx* c, size_t need) {
-    if (need <= c->cap_learn) return SDL_OK;
-    if (c->learn) cudaFree(c->learn);
-    c->learn = nullptr;
-    c->cap_learn = 0;
-    if (cudaMalloc(&c->learn, need) != cudaSuccess) {
-        cudaGetLastError();
-        return SDL_ERR_WORKSPACE;
-    }
-    c->cap_learn = need;
-    return SDL_OK;
-}
-
-// Scores of `rows` signals (at most the rows that Xb and Hb hold).
-static int infer_rows(sdl_mlp* m, const float* Y, int64_t rows, bf16* Xb, bf16* Hb, float* scores,
-                      cudaStream_t st) {
+// Scores of `rows` (<= m->rows) signals.
+static int infer_rows(sdl_mlp* m, const float* Y, int64_t rows, float* scores, cudaStream_t st) {
     sdl_ctx* c = m->ctx;
     const int H = m->H, Kp = m->Kp, Q = m->Q, B = (int)rows;
+    bf16 *Xb = m->Xb, *Hb = m->Hb;
     if (m->P % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0)
         prep_rows_kernel<<<blocks_for(rows * 8, 256), 256, 0, st>>>(Y, B, m->P, Kp, Xb);
     else
@@ -786,21 +778,11 @@ int sdl_mlp_forward(sdl_mlp* m, const float* Y, int64_t N, float* scores, void* 
     DeviceGuard guard(m->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     sdl_ctx* c = m->ctx;
-    // a call within the training batch uses the network's own buffers
-    bf16 *Xb = m->Xb, *Hb = m->Hb;
-    int64_t chunk = m->Bmax;
-    if (N > chunk) {
-        chunk = std::max<int64_t>(chunk, std::min<int64_t>(N, kInferChunk));
-        const int rc = learn_workspace(c, infer_bytes(m, chunk));
-        if (rc) return rc;
-        char* p = c->learn;
-        Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
-        Hb = carve<bf16>(p, (size_t)chunk * m->H);
-    }
+    const int64_t chunk = m->rows;
     Trace tr(c, kMlp, st);
     for (int64_t r0 = 0; r0 < N; r0 += chunk) {
         const int64_t B = std::min<int64_t>(chunk, N - r0);
-        const int rc = infer_rows(m, Y + (size_t)r0 * m->P, B, Xb, Hb, scores + (size_t)r0 * m->Q, st);
+        const int rc = infer_rows(m, Y + (size_t)r0 * m->P, B, scores + (size_t)r0 * m->Q, st);
         if (rc) return rc;
     }
     return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
@@ -855,7 +837,7 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     cudaStream_t st = (cudaStream_t)stream;
     const int k2 = k, Q = m->Q;     // the shortlist only: the fallback test scans every pair
     // workspace: scores of one chunk, candidates, scan buffers, index list
-    const long long chunk = std::max<long long>(m->Bmax, std::min<long long>(N, kInferChunk));
+    const long long chunk = std::min<long long>(N, m->rows);
     const int nblk = (int)((N + kScanBlock - 1) / kScanBlock);
     const long long m_s = std::min<long long>(N, std::max<long long>(kGuardMinSample, N / 16));
     const long long stride_s = N / m_s;
@@ -863,10 +845,18 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
                         sizeof(int) * (nblk + 8) +
                         sizeof(int32_t) * (size_t)N + sizeof(int32_t) * (size_t)m_s +
                         sizeof(float) * (size_t)m_s + sizeof(float) * (size_t)N + sizeof(double2) * kGuardCtas +
-                        10 * 256 +
-                        infer_bytes(m, chunk);
-    int rc = learn_workspace(c, need);
-    if (rc) return rc;
+                        10 * 256;
+    if (need > c->cap_learn) {
+        if (c->learn) cudaFree(c->learn);
+        c->learn = nullptr;
+        c->cap_learn = 0;
+        if (cudaMalloc(&c->learn, need) != cudaSuccess) {
+            cudaGetLastError();
+            return SDL_ERR_WORKSPACE;
+        }
+        c->cap_learn = need;
+    }
+    int rc;
     char* p = c->learn;
     float* scores = carve<float>(p, (size_t)chunk * Q);
     int32_t* cand = carve<int32_t>(p, (size_t)N * k2);
@@ -877,14 +867,12 @@ extern "C" int sdl_sparse_code_learned(sdl_ctx* c, sdl_mlp* m, const float* Y, i
     float* learnedE = res_energy ? res_energy : carve<float>(p, (size_t)N);
     int* cnt_s = carve<int>(p, 2);
     double2* part = carve<double2>(p, kGuardCtas);
-    bf16* Xb = carve<bf16>(p, (size_t)chunk * m->Kp);
-    bf16* Hb = carve<bf16>(p, (size_t)chunk * m->H);
     // 1. scores and shortlists, chunk by chunk
     for (int64_t r0 = 0; r0 < N; r0 += chunk) {
         const int B = (int)std::min<int64_t>(chunk, N - r0);
         {
             Trace tr(c, kMlp, st);
-            if ((rc = infer_rows(m, Y + (size_t)r0 * p1 * p2, B, Xb, Hb, scores, st))) return rc;
+            if ((rc = infer_rows(m, Y + (size_t)r0 * p1 * p2, B, scores, st))) return rc;
         }
         Trace tr(c, kTopk, st);
         if (Q <= 256)
