@@ -227,8 +227,11 @@ int sdl_create(sdl_ctx** out, int device) {
         delete c;
         return SDL_ERR_CUDA;
     }
-    if (cudaMalloc(&c->err, sizeof(int)) != cudaSuccess || cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&c->err, sizeof(int)) != cudaSuccess || cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&c->scan_word, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMemset(c->scan_word, 0, sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
+        cudaFree(c->err);
         delete c;
         return SDL_ERR_WORKSPACE;
     }
@@ -241,6 +244,7 @@ int sdl_destroy(sdl_ctx* c) {
     DeviceGuard g(c->device);
     cudaDeviceSynchronize();
     cudaFree(c->err);
+    cudaFree(c->scan_word);
     cudaFree(c->G1);
     cudaFree(c->G2);
     cudaFree(c->part_f);
@@ -314,7 +318,7 @@ int sdl_sparse_code(sdl_ctx* c, const float* Y, int p1, int p2, int64_t N, const
     a.res_energy = res_energy;
     if (!(c->prec & SDL_PREC_BF16_CORR) && code_lanes_take(a, c->cap_part)) {
         Trace tr(c, kCode, st);
-        return launch_code_lanes(a, c->part_f, c->cap_part, st, c->num_sms);
+        return launch_code_lanes(a, c->part_f, c->cap_part, c->scan_word, st, c->num_sms);
     }
     grams(c, D1, p1, n1, D2, p2, n2, st);
     if ((c->prec & SDL_PREC_BF16_CORR) && (rc = prepare_tc_pass(c, a, true, st)) != SDL_OK) return rc;

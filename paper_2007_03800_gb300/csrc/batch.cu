@@ -52,6 +52,7 @@ struct sdl_batch {
     std::vector<double*> red_d, part_d;
     std::vector<float*> part_f;
     std::vector<size_t> part_cap;  // floats of each
+    unsigned long long* scan_word = nullptr;   // omp_scan.cu: zero between scans
     cudaGraphExec_t graph = nullptr;
 };
 
@@ -80,7 +81,8 @@ int code_pass(const sdl_batch* b, int side, cudaStream_t st) {
     if (side == kCodeOnly && b->large_groups) {
         for (int g = 0; g < b->G; ++g) {
             if (b->shape[g] < 0) continue;
-            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], st, b->ctx->num_sms);
+            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], b->scan_word, st,
+                                   b->ctx->num_sms);
             if (rc != SDL_OK) return rc;
         }
     } else if (b->n_fast > 0) {
@@ -92,7 +94,8 @@ int code_pass(const sdl_batch* b, int side, cudaStream_t st) {
     for (size_t i = 0; i < b->generic.size(); ++i) {
         if (side == kCodeOnly) {
             const int g = b->generic[i];
-            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], st, b->ctx->num_sms);
+            rc = launch_code_lanes(b->args[side][g], b->part_f[g], b->part_cap[g], b->scan_word, st,
+                                   b->ctx->num_sms);
             if (rc == SDL_OK) continue;
             if (rc != SDL_ERR_UNSUPPORTED) return rc;
             rc = SDL_OK;
@@ -247,7 +250,9 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
     const size_t o_sol = take(sizeof(SolveDesc) * 2 * G);
     const size_t o_res = take(sizeof(RescaleDesc) * G);
     const size_t o_rmse = take(sizeof(double) * 2 * G);
-    if (cudaMalloc(&b->dmem, bytes) != cudaSuccess) {
+    const size_t o_word = take(sizeof(unsigned long long));
+    if (cudaMalloc(&b->dmem, bytes) != cudaSuccess ||
+        cudaMemset(b->dmem + o_word, 0, sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
         destroy(b);
         return SDL_ERR_WORKSPACE;
@@ -273,6 +278,7 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
     b->d_solve[1] = b->d_solve[0] + G;
     b->d_rescale = reinterpret_cast<RescaleDesc*>(b->dmem + o_res);
     b->rmse_stage = reinterpret_cast<double*>(b->dmem + o_rmse);
+    b->scan_word = reinterpret_cast<unsigned long long*>(b->dmem + o_word);
 
     // ---- per-group pass arguments
     for (int side = 0; side < 3; ++side) b->args[side].resize(G);

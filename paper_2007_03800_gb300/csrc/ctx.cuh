@@ -10,6 +10,7 @@ struct sdl_ctx {
     int device = 0;
     int num_sms = 0;
     int* err = nullptr;          // device error word
+    unsigned long long* scan_word = nullptr;   // omp_scan.cu: zero between scans
     float* G1 = nullptr;         // Gram matrices of the current dictionaries
     float* G2 = nullptr;
     float* part_f = nullptr;     // partial-sum slots

@@ -100,9 +100,11 @@ int launch_code_group_wide(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_code_group_cols(const PassArgs& a, cudaStream_t st, int num_sms);
 int launch_ortho_group(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid = 0);
 // omp_scan.cu: the above for a code-only call, behind an error scan when it is
-// error-driven (ws: ws_n floats of scratch, or null)
+// error-driven and large (ws: ws_n floats of scratch, or null; scan_word: a device
+// word that is zero between scans, or null)
 bool code_lanes_take(const PassArgs& a, size_t ws_n);
-int launch_code_lanes(const PassArgs& a, float* ws, size_t ws_n, cudaStream_t st, int num_sms);
+int launch_code_lanes(const PassArgs& a, float* ws, size_t ws_n, unsigned long long* scan_word, cudaStream_t st,
+                      int num_sms);
 // omp_fast.cu: compile-time-shape kernels; SDL_ERR_UNSUPPORTED when no
 // specialisation matches (the caller then uses the generic kernel).
 int launch_code_pass_fast(const PassArgs& a, int side, cudaStream_t st, int num_sms);
