@@ -63,15 +63,24 @@ constexpr int kMultiWarps = 8;   // warps per CTA of the persistent multi-proble
 
 // Signals times atom pairs, on average over the groups, from which a code-only pass
 // runs each group as its own launches of the lane-group coder (omp_group.cuh) rather
-// than all of them in the multi-problem launch.  Error-driven groups of an image's
-// patches, us in one launch | in their own: 8x16 x 15 129 signals (3.9M) 21 | 25, x 37 249
-// (9.5M) 27 | 27; 12x24 x 7 921 (4.6M) 29 | 33, x 14 161 (8.2M) 35 | 35, x 35 721 52 | 46;
-// 16x32 x 7 225 (7.4M) 56 | 54, x 13 225 78 | 62; all three (14.2M) 96 | 105, (25.6M) 150 | 116.
-// Without a large dictionary the one launch packs its SMs better and wins longer:
-// 8x16 and 12x24 x 66 000 (27.5M on average, few picks) 74 | 80, x 103 000 (43M) 98 | 85.
+// than all of them in the multi-problem launch.  One launch packs the SMs better: the
+// launches of a group cost some 13 us of ramp and tail that the next group's wait for,
+// so error-driven batches, whose groups are short, need more work per group the more
+// groups there are.  us in one launch | in their own:
+//   every signal s picks: 16x32 x 8000 signals (8.2M) 62 | 51, 8x16 and 16x32 x 16 000
+//   162 | 100, all three shapes x 13 000 170 | 116, eight 16x32 x 8000 516 | 383, x 20 000 1364 | 779;
+//   patches of an image with noise (sigma 20, 40), all three: 150 x 150 (11.7M) 164 | 112 and
+//   99 | 86, 300 x 300 381 | 216 and 209 | 152; 16x32 alone, 100 x 100 (7.4M) 55 | 42 and 38 | 37;
+//   signals of which a tenth takes one pick or two, the least that a batch can hold, lose
+//   until the groups are large: 16x32 x 8000 17 | 23, x 20 000 24 | 23, all three x 13 000 (8M)
+//   33 | 49, x 40 000 58 | 60, four 16x32 x 20 000 57 | 80, eight x 8000 49 | 154.
+// Without a large dictionary the multi-problem kernel's 8x16 and 12x24 bodies hold out longer:
+// both x 50 000 (21M on average) 162 | 131, with few picks 41 | 37, 68 | 60.
 constexpr long long kLanesWork = 8'000'000, kLanesWorkSmall = 40'000'000;
-// Signals up to which the list of an error-driven group fits its partial-sum slots.
-constexpr long long kMostListed = 1 << 20;
+long long lanes_work(bool large, bool error_driven, int groups) {
+    const long long w = large ? kLanesWork : kLanesWorkSmall;
+    return error_driven ? w * (5 + groups) / 6 : w;
+}
 
 // A coding pass of every group: one persistent multi-problem launch, or for a
 // single group its tiling's own kernel on the same CTAs (no other problem's
@@ -206,17 +215,6 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         if (gen) b->generic.push_back(g);
     }
     b->n_fast = G - (int)b->generic.size();
-    long long work = 0;
-    bool large = false;     // some dictionary pair of 1024 or more atom pairs
-    b->large_groups = b->n_fast > 0;
-    for (int g = 0; g < G; ++g) {
-        if (variants[g].empty()) continue;
-        work += groups[g].N * (groups[g].n1 * groups[g].n2);
-        large = large || groups[g].n1 * groups[g].n2 >= 1024;
-        if (groups[g].N > kMostListed) b->large_groups = false;
-    }
-    if (work < (large ? kLanesWork : kLanesWorkSmall) * b->n_fast) b->large_groups = false;
-
     // ---- device memory
     const int max_slots = c->num_sms * kSlotsPerSm;
     size_t bytes = 0;
@@ -311,6 +309,19 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
         b->args[kCodeOnly][g] = a;               // sparse coding only
         b->args[kSideD2][g] = a;                 // pass 2: codes + partial sums
     }
+    long long work = 0;
+    bool large = false;     // some dictionary pair of 1024 or more atom pairs
+    bool eps = false;       // some error-driven group
+    b->large_groups = b->n_fast > 0;
+    for (int g = 0; g < G; ++g) {
+        if (variants[g].empty()) continue;
+        const PassArgs& a = b->args[kCodeOnly][g];
+        work += a.N * (a.n1 * a.n2);
+        large = large || a.n1 * a.n2 >= 1024;
+        eps = eps || a.eps2 > 0.f;
+        if (!code_lanes_take(a, b->part_cap[g])) b->large_groups = false;
+    }
+    if (work < lanes_work(large, eps, b->n_fast) * b->n_fast) b->large_groups = false;
     // slots the generic groups' passes will write (their reductions are sized now)
     for (int side = 0; side < 3; ++side)
         for (int g : b->generic) {
