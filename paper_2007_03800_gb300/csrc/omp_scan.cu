@@ -10,6 +10,7 @@
 // three sizes as one batch 668 -> 362.  The same scan inside the coder
 // (32 signals at a time per warp, the others queued) took 90, 444 and 518 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "sdl_internal.cuh"
 
@@ -17,9 +18,9 @@ namespace sdl {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kWarps = 8;           // a block scans 8 x 4 its signals
+constexpr int kWarps = 8;           // a block scans 8 x 4 ITS signals
 
-// A group of 8 lanes sums one signal, 4 signals per warp and step, `its` (1, 2, 4 or
+// A group of 8 lanes sums one signal, 4 signals per warp and step, ITS (1, 2, 4 or
 // 8) steps per warp: few signals spread over more blocks (8000 of 32x32 values in
 // blocks of 256 took 33 us, most of it one warp's chain of loads).  The partial
 // sums and their combining tree are the coders' (32 strided chains, then xor
@@ -28,20 +29,23 @@ constexpr int kWarps = 8;           // a block scans 8 x 4 its signals
 // 16-byte aligned).
 // `word` starts at zero: blocks that have come in the upper half, signals listed in
 // the lower.  The last block to come moves the total to *count and clears the
-// word for the next scan, which costs no launch of its own.
-template <bool VEC>
+// word for the next scan, which costs no launch of its own (a memset costs the host
+// 3 us).  A scan of 8 steps per warp, whose time the host does not feel, adds to a cleared
+// *count instead, and blocks that list nothing skip the atomic (three scans of 250 000
+// signals: 363 us with their coders, 381 through the word).
+template <bool VEC, int ITS>
 __global__ void __launch_bounds__(kWarps * 32)
-    energy_scan_kernel(const float* __restrict__ Y, int pp, long long N, int its, float eps2, int s,
+    energy_scan_kernel(const float* __restrict__ Y, int pp, long long N, float eps2, int s,
                        int32_t* __restrict__ support, float* __restrict__ coef, int32_t* __restrict__ nnz,
                        float* __restrict__ res_energy, int32_t* __restrict__ list, int* __restrict__ count,
                        unsigned long long* __restrict__ word) {
     __shared__ int wcount[kWarps], base_s;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane >> 3, j = lane & 7;
-    const long long first = ((long long)blockIdx.x * kWarps + w) * (4 * its);
-    const int m = (int)max(0LL, min((long long)(4 * its), N - first));
+    const long long first = ((long long)blockIdx.x * kWarps + w) * (4 * ITS);
+    const int m = (int)max(0LL, min(4LL * ITS, N - first));
     float mine = 0.f;
 #pragma unroll 2
-    for (int it = 0; it < its; ++it) {
+    for (int it = 0; it < ITS; ++it) {
         const int i = it * 4 + grp;
         float v[4] = {0.f, 0.f, 0.f, 0.f};
         if (i < m) {
@@ -83,7 +87,7 @@ __global__ void __launch_bounds__(kWarps * 32)
     }
     if (support && dm) {
         const unsigned inv_s = (65536u + s - 1) / s;   // e / s for e < 1024
-        for (int e = lane; e < 4 * its * s; e += 32)
+        for (int e = lane; e < 4 * ITS * s; e += 32)
             if ((dm >> ((unsigned)e * inv_s >> 16)) & 1u) {
                 support[(size_t)first * s + e] = -1;
                 coef[(size_t)first * s + e] = 0.f;
@@ -99,11 +103,15 @@ __global__ void __launch_bounds__(kWarps * 32)
             tot += c;
         }
         // the list's order does not matter
-        const unsigned long long old = atomicAdd(word, (1ULL << 32) | (unsigned)tot);
-        base_s = (int)(unsigned)old;
-        if ((unsigned)(old >> 32) + 1 == gridDim.x) {   // every other block has come
-            *count = base_s + tot;
-            *word = 0;
+        if constexpr (ITS == 8) {
+            base_s = tot ? atomicAdd(count, tot) : 0;
+        } else {
+            const unsigned long long old = atomicAdd(word, (1ULL << 32) | (unsigned)tot);
+            base_s = (int)(unsigned)old;
+            if ((unsigned)(old >> 32) + 1 == gridDim.x) {   // every other block has come
+                *count = base_s + tot;
+                *word = 0;
+            }
         }
     }
     __syncthreads();
@@ -171,9 +179,17 @@ int launch_code_lanes(const PassArgs& a, float* ws, size_t ws_n, unsigned long l
         // four blocks per SM before a warp takes more signals
         int its = 8;
         while (its > 1 && q.N < (long long)kWarps * 4 * its * 4 * num_sms) its /= 2;
+        if (its == 8 && cudaMemsetAsync(count, 0, sizeof(int), st) != cudaSuccess) return SDL_ERR_CUDA;
         const unsigned blocks = (unsigned)((q.N + kWarps * 4 * its - 1) / (kWarps * 4 * its));
-        auto kern = aligned && pp % 4 == 0 ? energy_scan_kernel<true> : energy_scan_kernel<false>;
-        kern<<<blocks, kWarps * 32, 0, st>>>(q.Y, pp, q.N, its, a.eps2, a.s, q.support, q.coef, q.nnz, q.res_energy,
+        auto scan = [&](auto ic) {
+            constexpr int I = decltype(ic)::value;
+            return aligned && pp % 4 == 0 ? energy_scan_kernel<true, I> : energy_scan_kernel<false, I>;
+        };
+        auto kern = its == 8   ? scan(std::integral_constant<int, 8>{})
+                    : its == 4 ? scan(std::integral_constant<int, 4>{})
+                    : its == 2 ? scan(std::integral_constant<int, 2>{})
+                               : scan(std::integral_constant<int, 1>{});
+        kern<<<blocks, kWarps * 32, 0, st>>>(q.Y, pp, q.N, a.eps2, a.s, q.support, q.coef, q.nnz, q.res_energy,
                                              list, count, scan_word);
         if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
         q.idx = list;
