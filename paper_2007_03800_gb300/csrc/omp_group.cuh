@@ -98,6 +98,7 @@ struct Cfg {
     static_assert(E % 2 == 0 && RI % 2 == 0, "row pairs, 16-byte block stores");
     static_assert((LI & (LI - 1)) == 0 && LI * LJ == GL, "lane grid");
     static_assert(!kW || P2 > 0, "the W stage is compiled for fixed sizes");
+    static_assert(!FAST_ || S_ > 0, "steps past the unrolled ones take the generic kernel's forms");
     static_assert(P1 == 0 || (P1 % LI == 0 && ZA % 2 == 0 && P1 % 4 == 0 && P2 % LJ == 0), "fixed sizes");
     static_assert(N1 == 0 || (N1 == N1P && N2 == N2P), "fixed sizes fill the tile");
 };
@@ -342,49 +343,86 @@ __device__ __forceinline__ bool chol_step(bool live, bool writer, Rec* rec, floa
     return ok;
 }
 
-// The same for any t, as loops through shared memory (row t of the factor and
-// the coefficients are written by every lane of the signal with equal values;
-// a step that fails leaves them unread).
-template <bool kFast, class Gram>
+// The same for any t < 32 (the generic kernel's forms): W lanes share the rows of
+// the factor, row m with lane m % W, and the unknowns travel by shuffle, so that a
+// step is a chain of t shuffles down and t back.  Every chain keeps its order: a
+// row takes the unknowns one after the other.  A step that every lane computed by
+// itself, loads of the factor in the chain, cost t^2 of them: 64 signals of 8x8 with
+// s = 32 picks took 224 us, 105 in the one-warp coder and 90 so; 8000 of them 515, 432 and
+// 213.
+// All lanes of the warp (of both warps of a team, which agree) call it together;
+// `t` is the same for all of them.
+template <int W, class Gram>
 __device__ __forceinline__ bool chol_step_any(int t, bool live, bool writer, Rec* rec, float* lf, float* iv,
                                               float* yv, Gram gram, float Att, float b, const Rec& pick, float& E) {
-    float* w = lf + t * (t - 1) / 2;
-    float ww = 0.f, wy = 0.f;
-    for (int m = 0; m < t; ++m) {
-        float v = gram(rec[m]);
-        const float* Lm = lf + m * (m - 1) / 2;
-        for (int l = 0; l < m; ++l) v = fmaf(-Lm[l], w[l], v);
-        const float wm = v * iv[m];
-        w[m] = wm;
-        ww = fmaf(wm, wm, ww);
-        wy = fmaf(wm, yv[m], wy);
+    constexpr int R = 32 / W;          // rows per lane
+    const int j = threadIdx.x % W;
+    const float* row[R];               // own rows of the factor
+    float v[R], inv_m[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int m = r * W + j, mm = m < t ? m : 0;   // rows past t run along on row 0
+        row[r] = lf + mm * (mm - 1) / 2;
+        v[r] = gram(rec[mm]);
+        inv_m[r] = iv[mm];
     }
+    // ---- row t of the factor: w_m = (a_m - sum_{l < m} L_ml w_l) / L_mm
+    float ww = 0.f, wy = 0.f;
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+        for (int i = 0; i < W && q * W + i < t; ++i) {
+            const int l = q * W + i;
+            const float wl = __shfl_sync(kFull, v[q] * inv_m[q], i, W);
+            ww = fmaf(wl, wl, ww);
+            wy = fmaf(wl, yv[l], wy);
+#pragma unroll
+            for (int r = q; r < R; ++r)
+                if (r * W + j > l && r * W + j < t) v[r] = fmaf(-row[r][l], wl, v[r]);
+        }
+    float w[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) w[r] = v[r] * inv_m[r];
     const float d = Att - ww;
     const bool ok = live && d > kPivotRel * Att;
-    if (!ok) return false;
-    const float inv = kFast ? rsqrtf(d) : 1.f / sqrtf(d);
+    const float inv = 1.f / sqrtf(d);
     const float yt = (b - wy) * inv;
     const float xt = yt * inv;
-    for (int k = t - 1; k >= 0; --k) {
-        float v = yv[k];
-        if constexpr (kFast) {
-            for (int l = k + 1; l < t; ++l) v = fmaf(-lf[l * (l - 1) / 2 + k], rec[l].x, v);
-            v = fmaf(-w[k], xt, v);
-        } else {
-            v = fmaf(-w[k], xt, v);
-            for (int l = t - 1; l > k; --l) v = fmaf(-lf[l * (l - 1) / 2 + k], rec[l].x, v);
+    // ---- back substitution, pick t first
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int m = r * W + j;
+        v[r] = fmaf(-w[r], xt, m < t ? yv[m] : 0.f);
+    }
+#pragma unroll
+    for (int q = R - 1; q >= 0; --q)
+        for (int i = min(W, t - q * W) - 1; i >= 0; --i) {
+            const int l = q * W + i;
+            const float xl = __shfl_sync(kFull, v[q] * inv_m[q], i, W);
+            const float* Ll = lf + l * (l - 1) / 2;
+#pragma unroll
+            for (int r = 0; r <= q; ++r)
+                if (r * W + j < l) v[r] = fmaf(-Ll[r * W + j], xl, v[r]);
         }
-        rec[k].x = v * iv[k];
+    if (ok) {
+        float* wrow = lf + t * (t - 1) / 2;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int m = r * W + j;
+            if (m < t) {
+                wrow[m] = w[r];
+                rec[m].x = v[r] * inv_m[r];
+            }
+        }
+        if (writer) {
+            iv[t] = inv;
+            yv[t] = yt;
+            Rec r = pick;
+            r.x = xt;
+            rec[t] = r;
+        }
+        E = fmaf(-yt, yt, E);
     }
-    if (writer) {
-        iv[t] = inv;
-        yv[t] = yt;
-        Rec r = pick;
-        r.x = xt;
-        rec[t] = r;
-    }
-    E = fmaf(-yt, yt, E);
-    return true;
+    return ok;
 }
 
 // G (row i: the products with every position of a lane-block row) of the
@@ -435,7 +473,9 @@ __device__ __forceinline__ void ksum(float& s, float& c, float v) {
 // Positions 0 .. count-1 (signals, or entries of the index list) are coded in
 // units of SPW: warp w of CTA b takes units w gridDim + b, + gridDim warps, ...
 // (a small call spreads over the SMs).
-template <class C>
+// MANY: sparsities past the unrolled steps (a kernel of its own: that path's registers
+// cost the others 1 to 2 % in spills).
+template <class C, bool MANY>
 __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(PassArgs a) {
     constexpr int GL = C::GL, LI = C::LI, LJ = C::LJ, RI = C::RI, RJ = C::RJ, E = C::E, SPW = C::SPW;
     constexpr int LD1 = C::LD1, LD2 = C::LD2, RIP = C::RIP, RJP = C::RJP, ZA = C::ZA, WB = C::WB;
@@ -879,8 +919,8 @@ __global__ void __launch_bounds__(C::WARPS * 32, C::MINB) code_group_kernel(Pass
                     }
                     [[fallthrough]];
                 default:
-                    if constexpr (C::S == 0)
-                        ok = chol_step_any<C::kFast>(t, pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
+                    if constexpr (MANY)
+                        ok = chol_step_any<(GL < 32 ? GL : 32)>(t, pick, wr, rec, lf, iv, yv, gram, Att, b, pk, E2);
                     break;
             }
             }
@@ -989,7 +1029,9 @@ int launch(const PassArgs& a, cudaStream_t st, int num_sms, int max_grid) {
     while ((bytes = sizeof(float) * (size_t)layout<C>(a.p1, a.p2, a.s, warps).total) > kSmMax && warps > C::TW)
         warps -= C::TW;
     if (bytes > kSmMax) return SDL_ERR_UNSUPPORTED;
-    auto kern = code_group_kernel<C>;
+    auto kern = code_group_kernel<C, false>;
+    if constexpr (C::S == 0 && !C::kOrtho)
+        if (a.s > C::SMAX) kern = code_group_kernel<C, true>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmMax) != cudaSuccess)
         return SDL_ERR_CUDA;
     // the registers allow MINB CTAs per SM (launch bounds); 1 KB per CTA is reserved
