@@ -11,12 +11,13 @@
 // entry.  B stays in registers (PA per lane), P in a warp-private n x n block of
 // shared memory, added up over the warps in a fixed order at the end: the
 // sums are deterministic.  Bound by issue (61 % of the slots, 750 warp
-// instructions per signal): 100 000 signals of 16x16, 32x32 atoms, s = 8 take 98 us
-// (D1) and 93 us (D2), against 287 and 430 us with one block-wide accumulator
-// under shared-memory atomics and the residual energy always formed.
+// instructions per signal): 100 000 signals of 16x16, 32x32 atoms, s = 8 take 92 us
+// (D1) and 90 us (D2), against 287 and 430 us with one block-wide accumulator
+// under shared-memory atomics and the residual energy always formed (206 and 199 with it).
 // Registers for two 12-warp CTAs per SM; the Gram matrix is formed here, so an
 // update needs no launch for it.
 #include <algorithm>
+#include <type_traits>
 
 #include "sdl_internal.cuh"
 
@@ -38,7 +39,10 @@ struct AccumLayout {
         // side D2 reads a column as 16-byte pieces, one column per lane: a stride
         // of an odd number of pieces spreads the lanes over the banks
         ys = side == kSideD1 ? p1 : up4(p1) + (up4(p1) / 4 % 2 ? 0 : 4);
-        ds = up4(pc);
+        // rows of D and of G: an odd number of 16-byte pieces, so that eight lanes on
+        // eight rows hit distinct banks (with up4(64) = 64 all 32 lanes of the Gram
+        // product met in one: 16x64 signals, 32x128 atoms, 92 us per CTA)
+        ds = up4(pc) + (up4(pc) / 4 % 2 ? 0 : 4);
         gs = nc | 1;
         dc = 0;                              // D[c, j] at j * ds + c, zero-padded
         g = dc + up4(ds * nc);               // G
@@ -67,8 +71,9 @@ struct alignas(16) AccumPick {
     int i, j, g;   // atoms of the updated and of the other side, offset of the latter's row of G
 };
 
-template <int PA, int SIDE>
-__global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassArgs a, int want_energy) {
+// ENERGY: the residual energy too (a kernel of its own, for its registers)
+template <int PA, int SIDE, bool ENERGY>
+__global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassArgs a) {
     extern __shared__ __align__(16) float sm[];
     constexpr bool kD1 = SIDE == kSideD1;
     constexpr int LG = 32 / PA;              // picks projected at once
@@ -98,7 +103,15 @@ __global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassA
     for (int e = threadIdx.x; e < nc * nc; e += blockDim.x) {   // as the Gram kernels form it
         const int i = e / nc, j = e - i * nc;
         float g = 0.f;
-        for (int c = 0; c < pc; ++c) g = fmaf(ds[i * L.ds + c], ds[j * L.ds + c], g);
+#pragma unroll 2
+        for (int c = 0; c < pc; c += 4) {   // (zeros past pc)
+            const float4 u = *reinterpret_cast<const float4*>(ds + i * L.ds + c);
+            const float4 v = *reinterpret_cast<const float4*>(ds + j * L.ds + c);
+            g = fmaf(u.x, v.x, g);
+            g = fmaf(u.y, v.y, g);
+            g = fmaf(u.z, v.z, g);
+            g = fmaf(u.w, v.w, g);
+        }
         gs[i * L.gs + j] = g;
     }
     __syncthreads();
@@ -183,21 +196,47 @@ __global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassA
         // 32 partial sums below 1e37 cannot add up to infinity
         const bool finite = __all_sync(kFull, y2 < 1e37f) || isfinite(warp_sum(y2));
         if (!finite && lane == 0) record_error(a.err, SDL_ERR_NONFINITE);
-        if (want_energy && finite) {
-            // exact residual energy with the current dictionaries
+        if (ENERGY && finite) {
+            // exact residual energy with the current dictionaries, U entries of a lane
+            // at a time (one at a time, a pick's loads are a chain of their own).  Per update
+            // with the objective, us, block-wide kernel | U = 1 | 2 | 4: 40 000 of 32x32 439 | 409 | 358 |
+            // 326, of 16x64 with 32x128 atoms 770 | 549 | 453 | 430; 40 000 of 16x16 157 | 115 | 110 | 111,
+            // of 12x12 103 | 86 | 86 | 92.
             float e2 = 0.f;
-            for (int e = lane; e < pp; e += 32) {
-                const int b = (int)((unsigned)e * inv_p1 >> 16), aa = e - b * p1;
-                float rec = 0.f;
-                for (int l = 0; l < cnt; ++l) {
-                    const AccumPick q = pk[l];
-                    const float da = __ldg(Da + (kD1 ? aa : b) + pa * q.i);
-                    const float dc = ds[q.j * L.ds + (kD1 ? b : aa)];
-                    rec = kD1 ? fmaf(q.x * da, dc, rec) : fmaf(q.x * dc, da, rec);
+            auto residual = [&](auto uc) {
+                constexpr int U = decltype(uc)::value;
+                for (int e0 = lane; e0 < pp; e0 += 32 * U) {
+                    float rec[U];
+                    int at[U], oa[U], oc[U];   // in the signal, the updated and the other dictionary's columns
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int e = min(e0 + 32 * u, pp - 1);
+                        const int b = (int)((unsigned)e * inv_p1 >> 16), aa = e - b * p1;
+                        at[u] = b * L.ys + aa;
+                        oa[u] = kD1 ? aa : b;
+                        oc[u] = kD1 ? b : aa;
+                        rec[u] = 0.f;
+                    }
+                    for (int l = 0; l < cnt; ++l) {
+                        const AccumPick q = pk[l];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const float da = __ldg(Da + oa[u] + pa * q.i);
+                            const float dc = ds[q.j * L.ds + oc[u]];
+                            rec[u] = kD1 ? fmaf(q.x * da, dc, rec[u]) : fmaf(q.x * dc, da, rec[u]);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (e0 + 32 * u < pp) {
+                            const float res = Ys[at[u]] - rec[u];
+                            e2 = fmaf(res, res, e2);
+                        }
                 }
-                const float res = Ys[b * L.ys + aa] - rec;
-                e2 = fmaf(res, res, e2);
-            }
+            };
+            if (pp <= 64) residual(std::integral_constant<int, 1>{});
+            else if (pp < 512) residual(std::integral_constant<int, 2>{});
+            else residual(std::integral_constant<int, 4>{});
             e2 = warp_sum(e2);
             energy += (double)e2;
         }
@@ -310,12 +349,12 @@ __global__ void __launch_bounds__(kWarps * 32, kMinCtas) accum_lane_kernel(PassA
 
 template <int PA, int SIDE>
 int launch(const PassArgs& a, bool want_energy, cudaStream_t st, int num_sms, size_t bytes, int warps) {
-    auto kern = accum_lane_kernel<PA, SIDE>;
+    auto kern = want_energy ? accum_lane_kernel<PA, SIDE, true> : accum_lane_kernel<PA, SIDE, false>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024) != cudaSuccess)
         return SDL_ERR_CUDA;
     const int bps = std::max(1, std::min<int>(kMinCtas, (int)((228 * 1024) / (bytes + 2048))));
     const long long grid = std::max<long long>(1, std::min<long long>((a.N + warps - 1) / warps, (long long)num_sms * bps));
-    kern<<<(int)grid, warps * 32, bytes, st>>>(a, want_energy ? 1 : 0);
+    kern<<<(int)grid, warps * 32, bytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? (int)grid : SDL_ERR_CUDA;
 }
 
