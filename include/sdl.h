@@ -256,8 +256,10 @@ int sdl_extract_patches(const float* image, int H, int W, int p, float* patches,
  * sdl_patch_average - rebuild the image from coded patches: pixel (y, x) is
  *   the plain average, over every patch k covering it, of
  *   means[k] + (D1 X_k D2^T)[y - r, x - c]   (D1 p x n1, D2 p x n2).
- *   Codes as written by the coders (N x s_max slots).  The reconstructed
- *   patches go through a context-owned workspace of N*p*p floats.  Output
+ *   Codes as written by the coders (N x s_max slots).  Uses a context-owned
+ *   workspace: (p + 1) rows of W floats per patch row for p <= 32, or the
+ *   reconstructed patches, N*p*p floats, for larger patches, dictionaries past
+ *   the shared memory and small images with many slots.  Output
  *   image_out: H*W floats, row-major.  Deterministic (fixed summation order).
  */
 int sdl_patch_average(sdl_ctx* ctx, const int32_t* support, const float* coef,

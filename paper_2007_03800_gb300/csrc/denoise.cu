@@ -185,8 +185,21 @@ __global__ void average_patches_kernel(const float* __restrict__ rec, int H, int
 // and M (p + 1 floats per pixel) stay in L2; average_rows_kernel adds them up.  All
 // sums run in a fixed order.  251 001 patches of 12x12 with 0.8 picks on average:
 // 41 us (cold caches) against 316 us through 144.6 MB of written and re-read patches.
+// Its chain per warp, every slot of up to 31 + p corners, is what a small image of full
+// codes waits for: there the patches are written after all (patches_faster).
 constexpr int kOvWarps = 8;
 constexpr int kOvList = 128;         // picks compacted at a time
+
+// Whether codes with all s slots in use are faster through written patches, by the
+// times of both forms in us: a pick costs a warp of overlap_rows_kernel 0.09, a value of a
+// written patch 2e-6 per pick; reading the patches back costs p p / 14 + 14 more than
+// a short chain (drawn so that sparse codes of images from 120 x 120 on keep the planes).  Planes | patches, all slots used: p = 8, 50 x 50, s = 4 22 | 22, s = 8 33 | 22, s = 32
+// 109 | 31; 128 x 128, s = 8 39 | 34, s = 16 70 | 47; 256 x 256, s = 32 144 | 228; p = 16, 80 x 80, s = 8
+// 51 | 60, s = 16 93 | 78; p = 24, 80 x 80, s = 32 214 | 204; p = 32, 50 x 50, s = 32 95 | 201.
+bool patches_faster(int p, int H, int W, int s) {
+    const double pp = (double)p * p, N = (double)(H - p + 1) * (W - p + 1);
+    return s * (0.09 * std::min(31 + p, W - p + 1) - 2e-6 * N * pp) > 14.0 + pp / 14.0;
+}
 
 struct alignas(16) OvPick {
     float x;
@@ -436,7 +449,7 @@ int sdl_patch_average(sdl_ctx* c, const int32_t* support, const float* coef, con
     const int pr = p <= 8 ? 8 : p <= 12 ? 12 : p <= 16 ? 16 : 32;
     const size_t bytes = sizeof(float) * (((size_t)n1 * pr + (size_t)n2 * p + 3) & ~size_t(3)) +
                          sizeof(OvPick) * kOvWarps * kOvList;
-    const bool planes = p <= 32 && bytes <= 48 * 1024 && H <= 8 * 65535;
+    const bool planes = p <= 32 && bytes <= 48 * 1024 && H <= 8 * 65535 && !patches_faster(p, H, W, s_max);
     const size_t need = planes ? (size_t)(H - p + 1) * (p + 1) * W : (size_t)N * p * p;
     if (need > c->cap_rec) {
         if (c->rec) cudaFree(c->rec);
