@@ -41,6 +41,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -650,22 +651,34 @@ int cached_map(CUtensorMap* out, const MapKey& k, Encode encode) {
     return SDL_OK;
 }
 
-// contraction length up to which the 16-warp epilogue is taken
+// Contraction length (of all terms) up to which a plain product takes the 16-warp
+// epilogue.  us with 16 | 4 epilogue warps: 50000 x 576, K = 256 34 | 53, 512 45 | 54, 1024 74 | 65;
+// 20000 x 1000, 512 35 | 41, 1000 72 | 72; 50000 x 4096, 64 148 | 319, 256 157 | 326, 512 227 | 330,
+// 1024 366 | 361; 4096 x 4096, 768 32 | 41, 1024 38 | 42; with the BF16 output alone 1000 x 1000,
+// 1000 12 | 14, 4096 x 576, 1024 16 | 20, 50000 x 4096, 1024 289 | 334.
 constexpr long long kShortK = 1024;
-// and from which a GEMM with few output tiles takes 128 x 32 ones
+// C += into more than this (three quarters of L2) waits for memory behind each tile's
+// reduce-add, and 16 warps with one output slot each hide less of it: 16384 x 4096, K = 512
+// 125 | 117, K = 1024 160 | 128, 8192 x 4096, 1024 84 | 69; within it 4096 x 4096 (67 MB), 768 33 | 40,
+// 20000 x 1000 (80 MB), 512 35 | 41.
+constexpr long long kReduceBytes = 96LL << 20;
+// And the length from which a GEMM with few output tiles takes 128 x 32 ones, us with
+// 128 x 32 | 128 x 128: 512 x 144, K = 1024 11.6 | 11.5, 4096 19.6 | 22.6, 16384 61 | 68; 256 x 256,
+// 4096 19.6 | 22.6; 128 x 1152, 2048 12.4 | 16.4; 384 x 384 (9 tiles), 1536 11.6 | 14.3; 64 x 64, 2048
+// 12.4 | 14.4; 128 x 128, 8192 33 | 39.
 constexpr int kThinK = 1024;
 
 int sm_count() {
-    static int count[64] = {0};
+    static std::atomic<int> count[64];   // one write per device; threads may race to the same value
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-    if (!count[dev]) {
-        int n = 0;
+    int n = count[dev].load(std::memory_order_relaxed);
+    if (!n) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
             n = 1;
-        count[dev] = n;
+        count[dev].store(n, std::memory_order_relaxed);
     }
-    return count[dev];
+    return n;
 }
 
 }  // namespace
@@ -741,16 +754,17 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
     e.tma = tma ? 1 : 0;
     auto launch = [&](auto kern, int BN, int EW) -> int {
         const size_t bytes = smem_bytes(BN, EW);
-        // the shared-memory opt-in is set once per device and variant
-        static bool attr_set[5][64] = {};
+        // the shared-memory opt-in is made once per device and variant (1 us of a small
+        // product's 11); threads that meet here make it twice
+        static std::atomic<bool> attr_set[5][64];
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return SDL_ERR_CUDA;
-        bool& done = attr_set[BN == 32 ? 4 : (BN == 256) + 2 * (EW == 16)][dev & 63];
-        if (!done || dev >= 64) {
+        std::atomic<bool>& done = attr_set[BN == 32 ? 4 : (BN == 256) + 2 * (EW == 16)][dev & 63];
+        if (!done.load(std::memory_order_acquire) || dev >= 64) {
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
                 cudaSuccess)
                 return SDL_ERR_CUDA;
-            done = dev < 64;
+            done.store(dev < 64, std::memory_order_release);
         }
         const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
         const int grid = (int)std::min<long long>(tiles, sm_count());
@@ -758,9 +772,12 @@ int tc_gemm_terms(const void* const* A, int lda, const void* const* B, int ldb, 
         return cudaGetLastError() == cudaSuccess ? SDL_OK : SDL_ERR_CUDA;
     };
     // 16 epilogue warps where a tile's epilogue outlasts its main loop: an
-    // activation, an output that leaves row by row, or a short contraction
+    // activation, an output that leaves row by row, or a short contraction (but for
+    // a large accumulation)
     if (bn == 32) return launch(tc_gemm_kernel<32, 4>, 32, 4);
-    const bool wide = act != 0 || !tma || (long long)K * terms <= kShortK;
+    const bool reduce = C && accumulate && (long long)M * N * 4 > kReduceBytes;
+    const bool wide = act != 0 || !tma ||
+                      ((long long)K * terms <= kShortK && !reduce);
     if (bn == 256) return wide ? launch(tc_gemm_kernel<256, 16>, 256, 16) : launch(tc_gemm_kernel<256, 4>, 256, 4);
     return wide ? launch(tc_gemm_kernel<128, 16>, 128, 16) : launch(tc_gemm_kernel<128, 4>, 128, 4);
 }
