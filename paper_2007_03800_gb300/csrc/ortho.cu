@@ -815,11 +815,22 @@ bool ortho_shape_supported(int p1, int p2, int s) {
 
 // Learning passes that run as the lane-group coder and ortho_sums_kernel: compiled
 // square shapes, aligned signals, fixed sparsity, and enough signals for two
-// launches to beat one.
+// launches to beat one.  An iteration, us fused | split, just past the line: 24 000 of 8x8,
+// s = 4 99 | 91, s = 16 153 | 126; 12 000 of 12x12, s = 6 125 | 103; 6000 of 16x16, s = 8 155 | 118, s = 16
+// 180 | 130 (half of it the shorter Jacobi rounds, which both forms have); 200 000 of 12x12
+// 495 | 383.
 constexpr long long kOrthoSplitPairs = 1500000;
 bool ortho_split(int p1, int p2, long long N, int s, float eps2, const float* Y) {
     return p1 == p2 && (p1 == 8 || p1 == 12 || p1 == 16) && s <= 16 && !(eps2 > 0.f) &&
            (reinterpret_cast<uintptr_t>(Y) & 15u) == 0 && N * p1 * p2 >= kOrthoSplitPairs;
+}
+
+// Code-only calls that keep most of a signal's entries and leave the lane groups few
+// rounds: a step's block read and maximum take 8 lanes as long as a warp's whole step.
+// us, lane groups | a warp per signal: s = 32, 200 signals of 10x6 20.5 | 17, 4000 22 | 19, of 8x8 21 | 18,
+// 20 000 49 | 60; 20 000 of 4x8, s = 16 37 | 31, s = 32 63 | 52, 100 000 132 | 139.
+bool ortho_by_warp(int p1, int p2, long long N, int s) {
+    return N <= 8192 ? s > 24 : N <= 50000 && p1 * p2 <= 32 && s >= 16;
 }
 
 int launch_ortho_code(const float* Y, int p1, int p2, long long N, const float* D1,
@@ -841,7 +852,7 @@ int launch_ortho_code(const float* Y, int p1, int p2, long long N, const float* 
     a.err = err;
     // fixed sparsity: the lane-group coder, for a learning pass with the sums from
     // its codes (the caller passes arrays for them) where that pays off
-    if (side == kCodeOnly && !(eps2 > 0.f)) return launch_ortho_group(a, st, num_sms);
+    if (side == kCodeOnly && !(eps2 > 0.f) && !ortho_by_warp(p1, p2, N, s)) return launch_ortho_group(a, st, num_sms);
     if (side != kCodeOnly && ortho_split(p1, p2, N, s, eps2, Y)) {
         const int cps = p1 == 8 ? kSqCps<8> : p1 == 12 ? kSqCps<12> : kSqCps<16>;
         const long long need = (N + kHalfTeams - 1) / kHalfTeams;
