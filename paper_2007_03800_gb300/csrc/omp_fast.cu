@@ -347,17 +347,15 @@ __device__ __forceinline__ void code_fast_body(const PassArgs& a, int cta, int n
     __syncthreads();
 
     const long long stride = (long long)n_ctas * wpc;
-    // positions j index either the signals themselves or a list of signals
-    const long long count = a.idx ? (long long)*a.idx_count : a.N;
-    long long j = wact ? (long long)cta * wpc + w : count;
-    long long k = (a.idx && j < count) ? (long long)a.idx[j] : j;
+    const long long count = a.N;
+    long long k = wact ? (long long)cta * wpc + w : count;
     if (wact && lane == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
         mbar_fence_init();
     }
     __syncwarp();
-    if (lane == 0 && j < count) {
+    if (lane == 0 && k < count) {
         mbar_arrive_tx(&bar[0], kBytes);
         tma_load_1d(Ybuf, a.Y + (size_t)k * PP, kBytes, &bar[0]);
     }
@@ -368,8 +366,7 @@ __device__ __forceinline__ void code_fast_body(const PassArgs& a, int cta, int n
     bool alive = true;
     int pending = 0;
 
-    for (int it = 0; j < count && alive; ++it, j += stride) {
-        k = a.idx ? (long long)a.idx[j] : j;
+    for (int it = 0; k < count && alive; ++it, k += stride) {
         const int buf = it & 1;
         float* Ys = Ybuf + buf * al4(PP);
         const bool got = mbar_wait(&bar[buf], buf ? phase1 : phase0);
@@ -381,9 +378,8 @@ __device__ __forceinline__ void code_fast_body(const PassArgs& a, int cta, int n
         }
         if (buf) phase1 ^= 1u; else phase0 ^= 1u;
         // prefetch this warp's next signal into the other buffer
-        const long long jn = j + stride;
-        if (lane == 0 && jn < count) {
-            const long long kn = a.idx ? (long long)a.idx[jn] : jn;
+        const long long kn = k + stride;
+        if (lane == 0 && kn < count) {
             fence_proxy_async();
             mbar_arrive_tx(&bar[buf ^ 1], kBytes);
             tma_load_1d(Ybuf + (buf ^ 1) * al4(PP), a.Y + (size_t)kn * PP, kBytes, &bar[buf ^ 1]);
@@ -398,14 +394,13 @@ __device__ __forceinline__ void code_fast_body(const PassArgs& a, int cta, int n
         const bool finite = isfinite(ss);
         if (finite && a.eps2 > 0.f && ss <= a.eps2) {
             // already within the error target: an empty code, no correlations
-            const long long ko = (a.idx && a.idx_compact) ? j : k;
             if (a.support && lane < S) {
-                a.support[(size_t)ko * S + lane] = -1;
-                a.coef[(size_t)ko * S + lane] = 0.f;
+                a.support[(size_t)k * S + lane] = -1;
+                a.coef[(size_t)k * S + lane] = 0.f;
             }
             if (lane == 0) {
-                if (a.nnz) a.nnz[ko] = 0;
-                if (a.res_energy) a.res_energy[ko] = ss;
+                if (a.nnz) a.nnz[k] = 0;
+                if (a.res_energy) a.res_energy[k] = ss;
                 const float ye = ss - w_energy_c;
                 const float te = w_energy + ye;
                 w_energy_c = (te - w_energy) - ye;
@@ -677,14 +672,13 @@ __device__ __forceinline__ void code_fast_body(const PassArgs& a, int cta, int n
         }
 
         // ---- emit the code (lane l holds pick l)
-        const long long ko = (a.idx && a.idx_compact) ? j : k;
         if (a.support && lane < S) {
-            a.support[(size_t)ko * S + lane] = (lane < cnt) ? myi + N1 * myj : -1;
-            a.coef[(size_t)ko * S + lane] = (lane < cnt) ? myx : 0.f;
+            a.support[(size_t)k * S + lane] = (lane < cnt) ? myi + N1 * myj : -1;
+            a.coef[(size_t)k * S + lane] = (lane < cnt) ? myx : 0.f;
         }
         if (lane == 0) {
-            if (a.nnz) a.nnz[ko] = cnt;
-            if (a.res_energy) a.res_energy[ko] = finite ? fmaxf(E2, 0.f) : __int_as_float(0x7fc00000);
+            if (a.nnz) a.nnz[k] = cnt;
+            if (a.res_energy) a.res_energy[k] = finite ? fmaxf(E2, 0.f) : __int_as_float(0x7fc00000);
             if (!finite) record_error(a.err, SDL_ERR_NONFINITE);
         }
 
@@ -888,7 +882,7 @@ __device__ __forceinline__ void code_half_body(const PassArgs& a, int cta, int n
     // halves (half 1 idles when only jb is left), so the warp meets at every
     // full-warp synchronisation point.
     const long long stride = (long long)n_ctas * wpc * 2;
-    const long long count = a.idx ? (long long)*a.idx_count : a.N;
+    const long long count = a.N;
     const long long first = ((long long)cta * wpc + w) * 2;
     if (hl == 0) {
         mbar_init(bar, 1);
@@ -897,9 +891,8 @@ __device__ __forceinline__ void code_half_body(const PassArgs& a, int cta, int n
     __syncwarp();
     bool inflight = first + h < count;   // a copy into Ys is outstanding
     if (hl == 0 && inflight) {
-        const long long k0 = a.idx ? (long long)a.idx[first + h] : first + h;
         mbar_arrive_tx(bar, kBytes);
-        tma_load_1d(Ys, a.Y + (size_t)k0 * PP, kBytes, bar);
+        tma_load_1d(Ys, a.Y + (size_t)(first + h) * PP, kBytes, bar);
     }
     unsigned phase = 0;
     float w_energy = 0.f, w_energy_c = 0.f, w_ynorm = 0.f, w_ynorm_c = 0.f;
@@ -908,7 +901,7 @@ __device__ __forceinline__ void code_half_body(const PassArgs& a, int cta, int n
     for (long long jb = first; jb < count && alive; jb += stride) {
         const long long jj = jb + h;
         const bool act = jj < count;
-        const long long k = act ? (a.idx ? (long long)a.idx[jj] : jj) : 0;
+        const long long k = act ? jj : 0;
         bool got = true;
         if (act) got = mbar_wait(bar, phase);
         if (!__all_sync(kFull, got)) {
@@ -983,10 +976,9 @@ __device__ __forceinline__ void code_half_body(const PassArgs& a, int cta, int n
             if (act && jn < count) {
                 inflight = true;
                 if (hl == 0) {
-                    const long long kn = a.idx ? (long long)a.idx[jn] : jn;
                     fence_proxy_async();
                     mbar_arrive_tx(bar, kBytes);
-                    tma_load_1d(Ys, a.Y + (size_t)kn * PP, kBytes, bar);
+                    tma_load_1d(Ys, a.Y + (size_t)jn * PP, kBytes, bar);
                 }
             }
         }
@@ -1177,14 +1169,13 @@ __device__ __forceinline__ void code_half_body(const PassArgs& a, int cta, int n
 
         // ---- emit the code (lane hl of the half holds pick hl)
         if (act) {
-            const long long ko = (a.idx && a.idx_compact) ? jj : k;
             if (a.support && hl < S) {
-                a.support[(size_t)ko * S + hl] = (hl < cnt) ? myi + N1 * myj : -1;
-                a.coef[(size_t)ko * S + hl] = (hl < cnt) ? myx : 0.f;
+                a.support[(size_t)k * S + hl] = (hl < cnt) ? myi + N1 * myj : -1;
+                a.coef[(size_t)k * S + hl] = (hl < cnt) ? myx : 0.f;
             }
             if (hl == 0) {
-                if (a.nnz) a.nnz[ko] = cnt;
-                if (a.res_energy) a.res_energy[ko] = finite ? fmaxf(E2, 0.f) : __int_as_float(0x7fc00000);
+                if (a.nnz) a.nnz[k] = cnt;
+                if (a.res_energy) a.res_energy[k] = finite ? fmaxf(E2, 0.f) : __int_as_float(0x7fc00000);
                 if (!finite) record_error(a.err, SDL_ERR_NONFINITE);
             }
         }

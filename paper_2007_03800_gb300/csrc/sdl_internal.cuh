@@ -50,7 +50,7 @@ struct PassArgs {
     int n_slots;          // global-accumulator mode: slots (CTA % n_slots)
     int* err;
     const int32_t* idx;   // optional: code only the signals idx[0 .. *idx_count)
-    const int* idx_count; //   (specialised kernels only; device count)
+    const int* idx_count; //   (lane-group coder only; device count)
     int idx_compact;      // with idx: outputs at list position j, not at idx[j]
     // optional correlations C0 from outside (BF16 tensor-core path), N x ldc0
     // FP32 with entry q = i + n1*j, each within c0_err_rel * ||Y_k|| of the
@@ -145,7 +145,7 @@ bool code_shape_supported(int p1, int p2, int n1, int n2, int s);
 int max_partial_slots(int num_sms);
 // tmod3_fast.cu: three-mode coding pass specialised at compile time for the
 // compiled shapes (SDL_ERR_UNSUPPORTED otherwise or for a Y not 16-byte
-// aligned); returns the partial-sum slots written (mode 1-3) or 0 (mode 0)
+// aligned; modes 1-3); returns the partial-sum slots written
 int launch_code3_fast(int mode, const float* Y, int p1, int p2, int p3, int n1, int n2, int n3,
                       long long N, const float* D1, const float* D2, const float* D3,
                       const float* G1, const float* G2, const float* G3, int s, int32_t* support,

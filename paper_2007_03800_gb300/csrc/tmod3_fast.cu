@@ -100,7 +100,7 @@ struct Layout3F {
     static constexpr int g3 = g2 + r4(N2 * N2);         // N3 x N3
     static constexpr int acc = g3 + r4(N3 * N3);
     __host__ __device__ static constexpr int nf(int mode) {
-        return mode == 1 ? N1 * N1 + P1 * N1 : mode == 2 ? N2 * N2 + P2 * N2 : mode == 3 ? N3 * N3 + P3 * N3 : 0;
+        return mode == 1 ? N1 * N1 + P1 * N1 : mode == 2 ? N2 * N2 + P2 * N2 : N3 * N3 + P3 * N3;
     }
     __host__ __device__ static constexpr int acce(int mode) { return acc + r4(nf(mode)) * Sh::WPC; }
     __host__ __device__ static constexpr int warp0(int mode) { return acce(mode) + r4(2 * Sh::WPC); }
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(Sh::WPC * 32, 2)
         }
 
         // ---- partial sums of the mode-k update (Remark 3 -> Corollary 1)
-        if constexpr (MODE != 0) {
+        {
             constexpr int nk = MODE == 1 ? N1 : MODE == 2 ? N2 : N3;
             constexpr int pk = MODE == 1 ? P1 : MODE == 2 ? P2 : P3;
             float* accP = wacc;
@@ -467,23 +467,21 @@ __global__ void __launch_bounds__(Sh::WPC * 32, 2)
         }
     }
 
-    if constexpr (MODE != 0) {
-        if (lane == 0) {
-            acce[2 * w] = w_energy - w_energy_c;
-            acce[2 * w + 1] = w_ynorm - w_ynorm_c;
-        }
-        __syncthreads();
-        float* dst = part_f + (size_t)blockIdx.x * nf;
-        for (int e = threadIdx.x; e < nf; e += blockDim.x) {
-            float v = 0.f;
-            for (int ww = 0; ww < Sh::WPC; ++ww) v += sm[L::acc + ww * r4(nf) + e];
-            dst[e] = v;
-        }
-        if (threadIdx.x < 2) {
-            double d = 0.0;
-            for (int ww = 0; ww < Sh::WPC; ++ww) d += (double)acce[2 * ww + threadIdx.x];
-            part_d[(size_t)blockIdx.x * 2 + threadIdx.x] = d;
-        }
+    if (lane == 0) {
+        acce[2 * w] = w_energy - w_energy_c;
+        acce[2 * w + 1] = w_ynorm - w_ynorm_c;
+    }
+    __syncthreads();
+    float* dst = part_f + (size_t)blockIdx.x * nf;
+    for (int e = threadIdx.x; e < nf; e += blockDim.x) {
+        float v = 0.f;
+        for (int ww = 0; ww < Sh::WPC; ++ww) v += sm[L::acc + ww * r4(nf) + e];
+        dst[e] = v;
+    }
+    if (threadIdx.x < 2) {
+        double d = 0.0;
+        for (int ww = 0; ww < Sh::WPC; ++ww) d += (double)acce[2 * ww + threadIdx.x];
+        part_d[(size_t)blockIdx.x * 2 + threadIdx.x] = d;
     }
 }
 
@@ -503,15 +501,14 @@ int launch_fast3(int mode, const float* Y, long long N, const float* D1, const f
             return SDL_ERR_CUDA;
         bps = std::max(1, std::min(bps, 8));
         const long long need = (N + Sh::WPC - 1) / Sh::WPC;
-        long long grid = std::max<long long>(1, std::min<long long>(need, (long long)num_sms * bps));
-        if (mode != 0) grid = std::min<long long>(grid, max_slots);
+        const long long grid =
+            std::max<long long>(1, std::min<long long>({need, (long long)num_sms * bps, (long long)max_slots}));
         kern<<<(int)grid, Sh::WPC * 32, bytes, st>>>(Y, N, D1, D2, D3, G1, G2, G3, support, coef, nnz,
                                                      res, part_f, part_d, err);
         if (cudaGetLastError() != cudaSuccess) return SDL_ERR_CUDA;
-        return mode == 0 ? 0 : (int)grid;
+        return (int)grid;
     };
     switch (mode) {
-        case 0: return run(code3_fast_kernel<Sh, 0>);
         case 1: return run(code3_fast_kernel<Sh, 1>);
         case 2: return run(code3_fast_kernel<Sh, 2>);
         default: return run(code3_fast_kernel<Sh, 3>);
@@ -535,7 +532,8 @@ int launch_code3_fast(int mode, const float* Y, int p1, int p2, int p3, int n1, 
                       const float* G1, const float* G2, const float* G3, int s, int32_t* support,
                       float* coef, int32_t* nnz, float* res, float* part_f, double* part_d,
                       int max_slots, int* err, int num_sms, cudaStream_t st) {
-    if ((reinterpret_cast<uintptr_t>(Y) & 15u) != 0) return SDL_ERR_UNSUPPORTED;
+    // coding alone at these shapes is tmod3_group.cu's
+    if (mode == 0 || (reinterpret_cast<uintptr_t>(Y) & 15u) != 0) return SDL_ERR_UNSUPPORTED;
     if (is_shape<F3cube>(p1, p2, p3, n1, n2, n3, s))
         return launch_fast3<F3cube>(mode, Y, N, D1, D2, D3, G1, G2, G3, support, coef, nnz, res,
                                     part_f, part_d, max_slots, err, num_sms, st);
