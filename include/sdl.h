@@ -165,8 +165,8 @@ int sdl_iterate(sdl_ctx* ctx, const float* Y, int p1, int p2, int64_t N,
  * Batching: several independent dictionary-learning problems ("groups") that
  * differ in signal size, dictionary size, sparsity and stopping rule, run
  * together.  This is the GB300 counterpart of the paper's many-worker setting
- * (Algorithm 1 with its data split over nodes): each coding pass of all groups
- * is ONE persistent launch, each update stage (Gram, reduction, solve,
+ * (Algorithm 1 with its data split over nodes): each coding pass of an iteration
+ * is ONE persistent launch for all groups, each update stage (Gram, reduction, solve,
  * rescale) is one launch for all groups, and with SDL_BATCH_GRAPH the whole
  * iteration is captured once into a CUDA graph and replayed.
  *
@@ -177,8 +177,8 @@ int sdl_iterate(sdl_ctx* ctx, const float* Y, int p1, int p2, int64_t N,
  * and Y 16-byte aligned joins the persistent multi-problem launch.  Any other
  * group that sdl_sparse_code supports (n1 <= 32 and n2 <= 128, n1 <= 128 and
  * n2 <= 32, or both <= 64) is coded by the generic kernel in a launch of its
- * own within the same iteration (and graph); its update stages still share
- * the one launch per stage.  Other shapes: SDL_ERR_UNSUPPORTED.  eps > 0 gives
+ * own within the same iteration (and graph; code-only passes as sdl_sparse_code does);
+ * its update stages still share the one launch per stage.  Other shapes: SDL_ERR_UNSUPPORTED.  eps > 0 gives
  * the group an error-driven stop (Sec. IV), per group.
  */
 typedef struct sdl_group {
@@ -213,7 +213,9 @@ typedef struct sdl_batch sdl_batch;
 int sdl_batch_create(sdl_ctx* ctx, const sdl_group* groups, int n_groups, int flags,
                      void* stream, sdl_batch** out);
 
-/* 2D-OMP of every group's signals in one persistent launch (codes only). */
+/* 2D-OMP of every group's signals (codes only): in one persistent launch, or, for
+ * groups large enough to fill the GPU one after the other, in launches of their own
+ * (the same codes). */
 int sdl_batch_sparse_code(sdl_batch* batch, void* stream);
 
 /* One Algorithm-1 iteration of every group (graph replay when captured).
@@ -575,9 +577,9 @@ int sdl_iterate3(sdl_ctx* ctx, const float* Y, int p1, int p2, int p3, int64_t N
  * nothing is enqueued.
  *  - The first call on a device looks up the array's device address (with
  *    that device current); make that first call before any stream capture.
- *  - Every call on a device shares the one array, which keeps the contents
- *    of the last call (each call rewrites both Gram matrices before reading
- *    them).  Calls whose work overlaps on the GPU (different streams, no
+ *  - Every call on a device shares the one array (calls that the lane-group
+ *    coder takes do not use it), which keeps the contents of the last call that
+ *    used it (each such call rewrites both Gram matrices before reading them).  Calls whose work overlaps on the GPU (different streams, no
  *    ordering between them) race on the array and give wrong codes.
  *  - Device-side errors (a signal with NaN/Inf, which also gets nnz = 0; a
  *    bounded wait for a signal copy that gave up, after which the remaining

@@ -8,8 +8,10 @@
 // signals b WPC + w, + grid WPC, ..., adds (pick, row) and (pick, pick) terms to its
 // private accumulators, terms that meet in one entry in increasing pick order, and
 // the warps are combined in warp order.  (The fused epilogue adds with
-// shared-memory atomics in rounds of 32 lanes, which the hardware applies to one
-// address in increasing lane order.)  Two warps share a sequence, one for B and
+// shared-memory atomics in rounds of 32 lanes.  No document says in which order those
+// of one warp reach one address; the boards measured take increasing lane order, as
+// B here does, and the P half uses the same atomics, so that the two forms give the same
+// bits there.)  Two warps share a sequence, one for B and
 // one for P: a sequence is a serial chain and they are as many as the fused
 // kernel had warps.  B: lane = row r of pick l = G t + g, the G picks of a
 // round added one after the other; P: lane = (pick, pick), by the same atomics.

@@ -6,7 +6,9 @@
 // tilings of every group and splits the CTAs between groups by measured cost.
 // A group whose shape has no compiled tiling (for instance 16 x 64 signals
 // with 32 x 128 atoms) is coded by the generic kernel in a launch of its own
-// inside the same iteration; its update stages join the others'.
+// inside the same iteration; its update stages join the others'.  Code-only passes
+// run the lane-group coder (omp_group.cuh) for such a group where it takes its sizes,
+// and for all groups where that beats the one launch (lanes_work).
 #include <algorithm>
 #include <cmath>
 #include <cstring>

@@ -7,9 +7,9 @@
 //
 // Forward and backward run as tcgen05 GEMMs (tc_gemm.cu) with fused
 // epilogues; this file holds the element-wise kernels (input scaling, the
-// loss gradient, bias-gradient reductions, Adam), the warp top-k, the
-// shortlist 2D-OMP kernel with its fallback test, and the deterministic
-// compaction of the fallback signals.
+// loss gradient, bias-gradient reductions, Adam), the warp top-k and the deterministic
+// compaction of the fallback signals; 2D-OMP on the shortlists with its fallback
+// test is omp_group_short.cu.
 #include <cuda_bf16.h>
 
 #include <algorithm>

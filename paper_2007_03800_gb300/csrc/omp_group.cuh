@@ -1,5 +1,6 @@
 // 2D-OMP coding pass with a small group of lanes per signal: a warp codes
-// 32 / GL signals at once, GL = 8 or 16 lanes each.
+// 32 / GL signals at once, GL = 8 or 16 lanes each; wide dictionaries take a whole warp
+// (32) or a team of two (64) per signal.
 //
 // Same method and arithmetic as the one-warp-per-signal coders (omp_fast.cu,
 // omp_pass.cu): every entry of Z, C0 and of the scores, the Cholesky rows and
@@ -41,10 +42,12 @@ constexpr unsigned kFull = 0xffffffffu;
 
 __host__ __device__ constexpr int up4(int x) { return (x + 3) & ~3; }
 
-// SF / P1F ...: sizes fixed at compile time (0: taken from the call).
-// kFastNum: 1/sqrt by rsqrtf and back substitution in increasing row order
+// GL lanes per signal in a grid of LI x GL / LI, RI x RJ entries of C0 per lane, WARPS
+// per CTA, MINB CTAs per SM.
+// P1 .. N2, S: sizes fixed at compile time (0: taken from the call).
+// FAST: 1/sqrt by rsqrtf and back substitution in increasing row order
 // (the compiled tilings' forms); else 1/sqrtf and decreasing order (the
-// generic kernel's).  kW: C0 = (D1^T Y) D2 rather than D1^T (Y D2).
+// generic kernel's).  W: C0 = (D1^T Y) D2 rather than D1^T (Y D2).
 // ORTHO_: 0, or the orthonormal variant (n = p; a pick's coefficient is its
 // correlation and leaves the others alone) with ||Y||^2 in that many chains.
 template <int GL_, int LI_, int RI_, int RJ_, int WARPS_, int MINB_, bool FAST_, bool W_, int P1_ = 0,

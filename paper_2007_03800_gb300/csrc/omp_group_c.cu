@@ -21,7 +21,9 @@ int launch_code_group_cols(const PassArgs& a, cudaStream_t st, int num_sms) {
     if (n1 <= 16 && n2 <= 64) return group::launch<Wide<16, 2, 8, 8, 8, 2>>(a, st, num_sms, 0);
     if (n1 <= 32 && n2 <= 64) return group::launch<Wide<32, 4, 8, 8, 8, 2>>(a, st, num_sms, 0);
     if (n1 <= 16 && n2 <= 128) return group::launch<Wide<32, 2, 8, 8, 8, 2>>(a, st, num_sms, 0);
-    // the hyperspectral-shaped problem with its sizes fixed
+    // the hyperspectral-shaped problem with its sizes fixed (as in the generic kernel's
+    // dispatch): 8000 signals, us fixed | run-time sizes, s = 4 to 32: s = 8 204 | 216, s = 10
+    // 251 | 264, s = 16 679 | 694; 64 signals, s = 10 35 | 37
     if (a.p1 == 16 && a.p2 == 64 && n1 == 32 && n2 == 128)
         return group::launch<Wide<64, 4, 8, 8, 12, 1, 16, 64, 32, 128, true>>(a, st, num_sms, 0);
     if (n1 <= 32 && n2 <= 128) return group::launch<Wide<64, 4, 8, 8, 12, 1, 0, 0, 0, 0, true>>(a, st, num_sms, 0);

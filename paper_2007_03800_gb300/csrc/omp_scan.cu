@@ -7,7 +7,7 @@
 // reads the signals at the memory's rate and the coder's units are then full
 // and evenly dealt.  Measured on the patches of a 512 x 512 image (13-19 % of them
 // over the target): 8x8 84 -> 39 us, 12x12 158 -> 94, 16x16 397 -> 221; the
-// three sizes as one batch 668 -> 362.  The same scan inside the coder
+// three sizes as one batch 630-750 -> 360-385 by board.  The same scan inside the coder
 // (32 signals at a time per warp, the others queued) took 90, 444 and 518 us.
 #include <algorithm>
 #include <type_traits>
@@ -21,8 +21,8 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = 8;           // a block scans 8 x 4 ITS signals
 
 // A group of 8 lanes sums one signal, 4 signals per warp and step, ITS (1, 2, 4 or
-// 8) steps per warp: few signals spread over more blocks (8000 of 32x32 values in
-// blocks of 256 took 33 us, most of it one warp's chain of loads).  The partial
+// 8) steps per warp: few signals spread over more blocks (up to 8000 of 32x32 values
+// in blocks of 256 took 33 us, most of it one warp's chain of loads).  The partial
 // sums and their combining tree are the coders' (32 strided chains, then xor
 // 16, 8, 4, 2, 1), so the comparison with the target comes out the same: lane j
 // holds chains 4j .. 4j+3.  VEC: 16-byte loads (p1 p2 a multiple of 4, Y

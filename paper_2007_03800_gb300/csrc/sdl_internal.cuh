@@ -87,7 +87,7 @@ int launch_code_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms);
 int launch_code_pass_generic(const PassArgs& a, int side, cudaStream_t st, int num_sms,
                              bool plan_only = false);
 int launch_accumulate_pass(const PassArgs& a, int side, cudaStream_t st, int num_sms);
-// omp_group_*.cu: code-only passes with 8 or 16 lanes per signal, in the
+// omp_group_*.cu: code-only passes with 8 to 64 lanes per signal, in the
 // arithmetic of the compiled tilings (fixed: their shapes; w_first: correlations
 // as (D1^T Y) D2, at most max_grid CTAs) or of the generic kernel (any: n1 <= 32,
 // n2 <= 128).  short: picks from candidate lists (8x8 and 12x12 signals).

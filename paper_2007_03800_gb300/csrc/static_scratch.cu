@@ -109,8 +109,8 @@ extern "C" int sdl_sparse_code_static(const float* Y, int p1, int p2, int64_t N,
     a.res_energy = res_energy;
     a.n_slots = 1;
     a.err = err;       // read by sdl_static_status
-    // calls with a fixed sparsity form the Grams inside the coder; the others run
-    // the coders that read them from memory
+    // calls with a fixed sparsity, and small error-driven ones, form the Grams inside
+    // the coder; the others run the coders that read them from memory
     rc = launch_code_lanes(a, nullptr, 0, nullptr, st, num_sms);
     if (rc != SDL_ERR_UNSUPPORTED) return rc;
     // Both Grams are fully rewritten before the coding pass reads them, so
