@@ -60,20 +60,21 @@ def make_inputs():
 # ------------------------------------------------------------- algorithmic work
 def flops_per_signal_pass(p1, p2, n1, n2, s, side):
     """Algorithmic FLOPs of one 2D-OMP coding pass of one signal (with the
-    fused partial sums of `side`): correlation C0 = D1^T (Y D2) in the cheaper
+    fused partial sums of `side`, 0: none): correlation C0 = D1^T (Y D2) in the cheaper
     association, the Gram-domain correlation updates sum_t 2 t n1 n2, the
     incremental Cholesky/solves ~2 t^2 per step, and the epilogue sums (B1 takes
     rows of Z = Y D2, B2 rows of W = D1^T Y, both already formed for C0)."""
     c0 = 2 * min(p1 * p2 * n2 + n1 * p1 * n2, n1 * p1 * p2 + n1 * p2 * n2)
     upd = sum(2 * t * n1 * n2 for t in range(s))
     chol = sum(2 * t * t + 4 * t + 4 for t in range(s))
-    epi = 2 * (p1 if side == 1 else p2) * s + 3 * s * s
+    epi = 2 * (p1 if side == 1 else p2) * s + 3 * s * s if side else 0
     return c0 + upd + chol + epi
 
 
 def bytes_per_signal_pass(p1, p2, s, side):
-    """Algorithmic HBM bytes: Y read once per pass; codes written by pass 2."""
-    return 4 * p1 * p2 + (8 * s + 4 if side == 2 else 0)
+    """Algorithmic HBM bytes: Y read once per pass; codes written by pass 2, and
+    by a pass without sums (side 0)."""
+    return 4 * p1 * p2 + (8 * s + 4 if side != 1 else 0)
 
 
 def flops_pass_hist(p1, p2, n1, n2, s, side, nnz_hist):
@@ -129,15 +130,16 @@ PEAK_BASIS = "measured FP32 FMA rate (sdl_fp32_fma_peak, packed fma.rn.f32x2)"
 
 
 # sources of the coding-pass kernels timed by the roofline (the specialised
-# kernel and its shared header): stored DRAM counters are only used while
-# these files are unchanged
-KERNEL_SOURCES = ("omp_fast.cu", "sdl_internal.cuh")
+# kernel or the lane-group coder, and their shared header): stored DRAM
+# counters are only used while these files are unchanged
+KERNEL_SOURCES = {"fused": ("omp_fast.cu", "sdl_internal.cuh"),
+                  "lanes": ("omp_group.cuh", "omp_group_fixed.cu", "sdl_internal.cuh")}
 
 
-def source_hash():
+def source_hash(form):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2007_03800_gb300", "csrc")
-    for f in KERNEL_SOURCES:
+    for f in KERNEL_SOURCES[form]:
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -542,7 +544,9 @@ def run_ours(args):
         kinds = {k: v for k, v in prof.items() if v[1] > 0}
         dom = max(kinds, key=lambda k: kinds[k][0])
         dom_ms, dom_n = kinds[dom]
-        side = {"code_D1": 1, "code_D2": 2}.get(dom, 2)
+        # sums in a launch of their own: the lane-group coder ran, and its pass has no epilogue
+        form = "lanes" if kinds.get("accum_D1") else "fused"
+        side = 0 if form == "lanes" else {"code_D1": 1, "code_D2": 2}.get(dom, 2)
         flops = N * flops_per_signal_pass(p1, p2, n1, n2, s, side)
         achieved = flops / (dom_ms / dom_n / 1e3) / 1e12
         traffic = issue = None
@@ -550,8 +554,8 @@ def run_ours(args):
         clk = clk.summary()
         if os.path.exists(tpath):
             t = json.load(open(tpath))
-            ent = t.get(f"{dom}/tiling{tiling}")
-            if ent and ent.get("source_hash") == source_hash() and ent.get("N") == N:
+            ent = t.get(f"{dom}/lanes" if form == "lanes" else f"{dom}/tiling{tiling}")
+            if ent and ent.get("source_hash") == source_hash(form) and ent.get("N") == N:
                 traffic = ent["dram_bytes_per_launch"]
                 inst = ent.get("warp_instructions_per_launch")
                 if inst:
@@ -601,10 +605,13 @@ def run_ours(args):
                 "batch_graph_autotuned": {"value": value, "ms_per_step": ms_per_step,
                                           "tuning": tuning, "tuning_log": tuning_log},
                 "per_call_launches": {"value": value_plain, "ms_per_step": ms_plain,
+                                      "form": "lane-group coder and ordered sums" if form == "lanes"
+                                              else "fused passes",
                                       "tiling": tiling, "tune_log": tune_log},
             },
             "kernels_ms_per_step": {k: round(v[0] / args.steps, 4) for k, v in kinds.items()},
-            "roofline": {"bound": "alu", "kernel": f"{dom} (tiling {tiling})", "achieved": achieved,
+            "roofline": {"bound": "alu", "kernel": f"{dom} ({'lane groups' if form == 'lanes' else f'tiling {tiling}'})",
+                         "achieved": achieved,
                          "peak": fp32_peak,
                          "unit": "TFLOP/s", "frac": achieved / fp32_peak, "traffic": traffic,
                          "peak_basis": "measured: FP32 FMA microbenchmark (sdl_fp32_fma_peak, packed "
@@ -856,7 +863,7 @@ def study_ortho(args):
 def study_nsweep(args):
     """Signals/s per Algorithm-1 iteration against N on the c2 shapes (12x12
     patches of the 64 seeded images, D 12x24, s = 6): the batched path (graph
-    replay, autotuned) and per-call sdl_iterate (tuned tiling), L2 flushed
+    replay, autotuned) and per-call sdl_iterate (tuned), L2 flushed
     before every timed iteration, median of steps.  The patches of each N are
     the first N of one seeded stream (chunks of 250 000)."""
     import torch
