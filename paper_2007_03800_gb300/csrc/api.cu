@@ -229,9 +229,11 @@ int sdl_create(sdl_ctx** out, int device) {
     }
     if (cudaMalloc(&c->err, sizeof(int)) != cudaSuccess || cudaMemset(c->err, 0, sizeof(int)) != cudaSuccess ||
         cudaMalloc(&c->scan_word, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMemset(c->scan_word, 0, sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMemset(c->scan_word, 0, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {   // calls on any stream find them cleared
         cudaGetLastError();
         cudaFree(c->err);
+        cudaFree(c->scan_word);
         delete c;
         return SDL_ERR_WORKSPACE;
     }

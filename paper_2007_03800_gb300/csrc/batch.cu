@@ -252,7 +252,8 @@ int sdl_batch_create(sdl_ctx* c, const sdl_group* groups, int n_groups, int flag
     const size_t o_rmse = take(sizeof(double) * 2 * G);
     const size_t o_word = take(sizeof(unsigned long long));
     if (cudaMalloc(&b->dmem, bytes) != cudaSuccess ||
-        cudaMemset(b->dmem + o_word, 0, sizeof(unsigned long long)) != cudaSuccess) {
+        cudaMemset(b->dmem + o_word, 0, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {
         cudaGetLastError();
         destroy(b);
         return SDL_ERR_WORKSPACE;

@@ -88,3 +88,20 @@ def test_captured_scan_replays(gpu_ctx):
         graph.replay()
         same(out, ref)
     assert gpu_ctx.status() == 0
+
+
+def test_first_scan_of_a_context_on_another_stream():
+    """The counter is cleared before the context is handed out, also for a stream that
+    does not wait for the default one."""
+    Y, D1, D2 = problem(40_000, 8, 8, 16, 16, 4)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ref = None
+    for _ in range(8):
+        ctx = sdl.Context(0)
+        with torch.cuda.stream(side):
+            got = ctx.sparse_code(Y, D1, D2, 4, eps=7.0, stream=side)
+        assert ctx.status(side) == 0
+        ref = ref or got
+        same(got, ref)
+        ctx.close()
